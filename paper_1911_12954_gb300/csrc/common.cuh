@@ -103,6 +103,71 @@ struct EigJob {
   int n, chi;
 };
 
+// ---------------------------------------------------------------------------- Z2 sectors
+// (sectors.cu) Without a field every bond index carries a Z2 charge and tensors are zero where
+// the charges do not add up. A set of index charges is a bit mask (bit j: the charge of index j).
+struct SectorState {          // per batch element, persistent
+  uint32_t charge[2][4];      // of each direction's bond, for the tensors in buffer 0 and 1
+  int dropped;                // an isometry column mixed charges: every charge counts as 0 from then on
+  int pad[3];
+};
+struct SectorPlan {           // per batch element of a group and step
+  int row[2][kMaxLeg + 1];    // operand rows of charge q with new a index < x
+  int grp[2][kMaxLeg + 1];    // row groups (X, Y, c', mu) of charge q with new a index < x
+  int K[2];                   // summed indices (a2, b2, a1', b1', k) of charge q
+  uint32_t na, nb, nc;        // charges of the new a, b, c legs
+  uint32_t mb, mc, mm;        // of the old b, c legs and of mu
+};
+struct SectorTables {
+  uint32_t* row;              // operand row (X, Y, c, c', mu): rank within its charge, charge in bit 31
+  uint2* kA;                  // summed indices, charge 0 first: offset in A's first pass and leg b2
+  uint2* kB;                  // the same for B: offset and leg b1'
+  uint32_t* grank;            // row group: rank, charge in bit 31
+  uint32_t* grp;              // row groups, charge 0 first
+  SectorPlan* plan;
+};
+struct SectorTab {            // the tables of element e start e * stride bytes after base
+  char* base;
+  int64_t stride, o_row, o_kA, o_kB, o_grank, o_grp, o_plan;
+  __host__ __device__ SectorTables at(int e) const {
+    char* p = base + e * stride;
+    return SectorTables{(uint32_t*)(p + o_row),   (uint2*)(p + o_kA),     (uint2*)(p + o_kB),
+                        (uint32_t*)(p + o_grank), (uint32_t*)(p + o_grp), (SectorPlan*)(p + o_plan)};
+  }
+};
+struct SectorArgs {           // sector_tables_kernel
+  const SectorState* state;   // of the group's first element
+  SectorTab tab;
+  int cur;                    // buffer of the tensors before the step
+  int a, b, c, mu;            // directions
+  int Da, Db, Dc, Dm, ca, cb;
+  uint32_t kA[5], kB[5];      // strides of the summed legs in the first passes' outputs
+};
+struct SectorOperand {        // second half-contraction pass of one tensor
+  SectorTab tab;
+  int sideB, parity;          // operand side, the tensor's own parity
+  int x0, xs, cb, Db, Dc, Dm;
+  int nouter;                 // xs Dc Dc Dm
+  int64_t in_x, in_j, in_c0, in_c1, in_m;   // strides of the first pass's output
+  int u_j, u_r;               // U strides of the contracted and the new leg (the column has stride 1)
+  int64_t rows, kps;          // panel geometry of the operand
+  int P, kalign;              // panels; summed indices are zero filled up to a multiple of kalign
+  int64_t in_bs, u_bs, out_bs;
+  unsigned* amax;
+  float amax_mul;
+  int amax_bs;
+};
+struct SectorClose {          // the two closing passes of one tensor
+  SectorTab tab;
+  int parity;                 // the output tensor's
+  int x0, xs, x20, xs2, ca, cb, cc, Dc, Dm;
+  int64_t ldc, c_bs, u_bs, o3_bs, t_bs;
+  // second pass: output fibre legs (all but Z', the output's order) with their strides in the row
+  // group of m, of n, in Z and in the output; the output stride of Z'
+  int fd[7], fm[7], fn[7], fz[7];
+  int64_t ft[7], tz, nfib;
+};
+
 // Side choice for one transverse direction: candidates from the nu and nu' Gram matrices.
 struct SelectJob {
   const double* U[2];      // candidate isometries (n x chi), nu side and nu' side
@@ -120,6 +185,10 @@ struct SelectJob {
   struct DevRecord* rec_b;
   const int* step;
   int nu;
+  // charges of the kept columns from those of the rows (nullptr: none kept): the bond masks of
+  // buffer `cur` before the step, written for buffer 1 - cur; job 0 also carries over mu's
+  SectorState* sectors;
+  int cur, mu, Dn;
 };
 
 // Step record as kept on the device for each batch element and step.
@@ -157,7 +226,7 @@ struct SelectPack {
   int64_t sU64 = 0;         // chosen isometry, FP64
   int64_t sUr = 0;          // chosen isometry, storage precision (elements)
   int64_t sRec = 0;         // step records (DevRecord)
-};
+};  // (sector states: one per batch element)
 
 // Message returned by hotrg_last_error for this host thread.
 void set_last_error(const char* msg);
@@ -182,6 +251,19 @@ cudaError_t launch_gram_merge_batch(const double* half, int64_t RRs, const int D
 cudaError_t launch_jacobi(const EigPack& jobs, int njobs, int nmax, double cluster_tau, int* status,
                           cudaStream_t st, int max_sweeps = kJacobiMaxSweeps, double tie_rel = 1e-8);
 cudaError_t launch_wait_selftest(int* status, unsigned long long limit_ns, cudaStream_t st);
+// Sector extents of a product: the rows of the A (B) operand's slice are the new a indices
+// [xa, xa + na) ([xb, xb + nb)) of the plan; row_limit > 0 keeps only the first rows of each
+// sector (timing probes). tab.base == nullptr: a dense product.
+struct GemmSectors {
+  SectorTab tab;
+  int xa, na, xb, nb;
+  int64_t row_limit;
+};
+// The same for the entry points that compute one product per launch: element and parities.
+struct OneProduct {
+  GemmSectors sec;
+  int elem, pa, parity;
+};
 // FP64-grade product on the fp16 tensor cores: C[M][N] (double, row stride ldc) =
 // alpha A B^T with A, B given as kOzSlices integer planes each (K panels as in
 // launch_gemm_group; plane p of A at A + p aps elements, of B at B + p bps), each operand
@@ -189,7 +271,8 @@ cudaError_t launch_wait_selftest(int* status, unsigned long long limit_ns, cudaS
 // accumulate: C += alpha A B^T.
 cudaError_t launch_gemm_oz(const void* A, const void* B, int64_t aps, int64_t bps, int64_t Kp, int64_t kps, int64_t P,
                            int64_t M, int64_t N, double* C, int64_t ldc, double alpha, const unsigned* amax_a,
-                           const unsigned* amax_b, bool accumulate, int* status, cudaStream_t st);
+                           const unsigned* amax_b, bool accumulate, int* status, cudaStream_t st,
+                           const OneProduct& one);
 // One output of a grouped block-spin GEMM: C = alpha * sum_{s < nseg} A_{a[s]} B_{b[s]}^T,
 // where A_w, B_w are the w-th operand tensors of the launch (the k loop runs over the nseg
 // segments one after the other, each the full K).
@@ -198,6 +281,8 @@ struct GemmProblem {
   float alpha;
   int nseg;
   int a[2], b[2];
+  int pa[2];                // sectors: parity of the A operand of each segment
+  int parity;               // sectors: parity of the output
 };
 constexpr int kMaxGemmProblems = 96;   // 32 temperatures x 3 tensors per launch
 struct GemmGroup {
@@ -209,6 +294,7 @@ struct GemmGroup {
   const unsigned* amax_a;
   const unsigned* amax_b;
   int per_elem;
+  GemmSectors sec;          // element of problem pb: pb / per_elem
 };
 // Tensor-core GEMM over W operand tensors per plane (hi, lo), each [P][rows][kps] in K
 // panels, tensor w of a plane aws (A) or bws (B) elements after tensor w - 1; every problem
@@ -221,7 +307,7 @@ template <typename R>
 cudaError_t launch_select(const SelectPack& jobs, int njobs, double side_rel, cudaStream_t st);
 template <typename R>
 cudaError_t launch_init(const double* beta, const double* h, R* T, R* S, int64_t slot, double* lnz_acc,
-                        int batch, cudaStream_t st);
+                        SectorState* sectors, int batch, cudaStream_t st);
 template <typename R>
 cudaError_t launch_norm(const R* x, int64_t n, int nb, int64_t xstride, double* partial, const int* step,
                         double* c_out, double* lnz_acc,
@@ -232,6 +318,10 @@ cudaError_t launch_step_end(int* step, cudaStream_t st);
 // 2^-14), out[2] = max(out[2], bits of the largest magnitude).
 cudaError_t launch_plane_stats(const void* plane, int64_t nrows, int64_t Kp, int64_t kps, unsigned long long* out,
                                cudaStream_t st);
+// The same over a plane stored by sectors (rows rows, P panels; the new a indices [x0, x0 + nx) of
+// element elem's plan, tensor parity `parity`): the entries left out are counted as zeros.
+cudaError_t launch_sector_stats(const void* plane, const SectorTab& tab, int elem, int parity, int x0, int nx,
+                                int64_t rows, int64_t K, int64_t kps, unsigned long long* out, cudaStream_t st);
 void jacobi_prepare();
 void gemm_prepare();
 template <typename R>
@@ -245,6 +335,14 @@ constexpr int kNormPartials = 2 * 152;
 template <typename R>
 cudaError_t launch_gemm_simt(const R* A, int64_t lda, const R* B, int64_t ldb, R* C, int64_t ldc,
                              int64_t M, int64_t N, int64_t K, double alpha, double beta,
-                             cudaStream_t st);
+                             cudaStream_t st, const OneProduct& one);
+
+void sectors_prepare();
+cudaError_t launch_sector_tables(const SectorArgs& a, int ne, cudaStream_t st);
+template <typename R>
+cudaError_t launch_sector_operand(const R* in, const R* U, R* out, R* out_lo, const SectorOperand& a, int ne, int mode,
+                                  cudaStream_t st);
+template <typename R>
+cudaError_t launch_sector_close(const R* C, const R* U, R* O3, R* T, const SectorClose& a, int ne, cudaStream_t st);
 
 }  // namespace hotrg

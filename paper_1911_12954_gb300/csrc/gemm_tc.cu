@@ -313,6 +313,71 @@ __device__ __forceinline__ float out_alpha(const GemmGroup& g, int pb) {
   return ldexpf(g.p[pb].alpha, -(split_exponent(g.amax_a[e], kF16Top) + split_exponent(g.amax_b[e], kF16Top)));
 }
 
+// Blocks of an output. A dense product has one block, the whole output; a product of tensors
+// that conserve the Z2 charge has one per row charge q: the rows of charge q against the columns
+// of charge q + the output's parity, over the summed indices of charge q + the A operand's parity
+// (their k-blocks, per segment). The extents are read from the element's SectorPlan on the device.
+struct Block {
+  int rows, cols;      // extent
+  int a0, b0;          // first row of the A and of the B operand
+  int c0;              // first output row (columns start at 0: a row belongs to one block)
+  int nk[2];           // k-blocks of the segments
+};
+__device__ __forceinline__ Block sector_block(const SectorPlan& p, const GemmSectors& s, int q, int pa0, int pa1,
+                                              int parity, int BK) {
+  Block b;
+  const int qc = q ^ parity;
+  const int r0 = p.row[0][s.xa + s.na] - p.row[0][s.xa], n0 = p.row[0][s.xb + s.nb] - p.row[0][s.xb];
+  b.rows = q ? p.row[1][s.xa + s.na] - p.row[1][s.xa] : r0;
+  b.cols = qc ? p.row[1][s.xb + s.nb] - p.row[1][s.xb] : n0;
+  if (s.row_limit > 0 && b.rows > s.row_limit) b.rows = (int)s.row_limit;
+  b.a0 = b.c0 = q ? r0 : 0;
+  b.b0 = qc ? n0 : 0;
+  b.nk[0] = (p.K[q ^ pa0] + BK - 1) / BK;
+  b.nk[1] = (p.K[q ^ pa1] + BK - 1) / BK;
+  return b;
+}
+// The blocks of a sector launch and the first tile of each (tiles of TM x TN, blocks one after the
+// other) in shared memory, by all threads of the CTA; the caller synchronises.
+struct BlockList {
+  Block b[2 * kMaxGemmProblems];
+  int first[2 * kMaxGemmProblems + 1];
+};
+__device__ __forceinline__ void list_blocks(const GemmGroup& g, BlockList& l, int BK, int TM, int TN) {
+  const int nb = 2 * g.nprob;
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+    const int pb = i >> 1;
+    const Block b = sector_block(*g.sec.tab.at(pb / g.per_elem).plan, g.sec, i & 1, g.p[pb].pa[0], g.p[pb].pa[1],
+                                 g.p[pb].parity, BK);
+    l.b[i] = b;
+    l.first[i + 1] = ((b.rows + TM - 1) / TM) * ((b.cols + TN - 1) / TN);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    l.first[0] = 0;
+    for (int i = 0; i < nb; ++i) l.first[i + 1] += l.first[i];
+  }
+}
+// Output pb and block of tile t, and its tile coordinates in the block (GM tile rows per group). bi:
+// the caller's current block, 0 at first (t does not decrease). Dense launches compile to plain
+// arithmetic on the kernel's arguments: reading the extents from shared memory there cost 1 %.
+template <bool SECT>
+__device__ __forceinline__ Block tile_at(const GemmGroup& g, const BlockList* l, int t, int& bi, int M, int N, int nkb,
+                                         int TM, int TN, int GM, int& pb, int& tm, int& tn) {
+  if constexpr (SECT) {
+    while (t >= l->first[bi + 1]) ++bi;
+    const Block b = l->b[bi];
+    pb = bi >> 1;
+    tile_coords(t - l->first[bi], (b.rows + TM - 1) / TM, (b.cols + TN - 1) / TN, GM, tm, tn);
+    return b;
+  } else {
+    const int tiles_m = (M + TM - 1) / TM, tiles_n = (N + TN - 1) / TN;
+    pb = t / (tiles_m * tiles_n);
+    tile_coords(t - pb * tiles_m * tiles_n, tiles_m, tiles_n, GM, tm, tn);
+    return Block{M, N, 0, 0, 0, {nkb, nkb}};
+  }
+}
+
 // alpha * acc for one thread's 128 columns of row m (guarded).
 __device__ __forceinline__ void store_row(float* __restrict__ C, int64_t ldc, int M, int N, int64_t m, int n0,
                                           const float* acc, float alpha) {
@@ -329,7 +394,7 @@ __device__ __forceinline__ void store_row(float* __restrict__ C, int64_t ldc, in
   }
 }
 
-template <class CF>
+template <class CF, bool SECT>
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_tf32x3_kernel(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__ CUtensorMap mAlo,
                        const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo,
@@ -348,9 +413,11 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint32_t* tmem_slot = (uint32_t*)(drain + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tiles_m = (M + BM - 1) / BM, tiles_n = (N + BN - 1) / BN;
-  const int ntiles1 = tiles_m * tiles_n;          // tiles of one output
-  const int ntiles = grp.nprob * ntiles1;         // outputs one after the other
+  BlockList* list = nullptr;
+  if constexpr (SECT) {
+    __shared__ BlockList list_mem;
+    list = &list_mem;
+  }
   const int nkbp = (Kp + BK - 1) / BK;   // k-blocks per panel (the last one zero-filled past Kp)
   const int nkb = P * nkbp;              // k-blocks of one segment
 
@@ -372,10 +439,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  if constexpr (SECT) list_blocks(grp, *list, BK, BM, BN);
   fence_before();
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  int ntiles;
+  if constexpr (SECT) ntiles = list->first[2 * grp.nprob];
+  else ntiles = grp.nprob * ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+  int bi = 0;                            // block of the role's current tile
 
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -388,24 +460,24 @@ __global__ void __launch_bounds__(THREADS, 1)
     int nissued = 0;   // k-blocks issued; stage q has been filled (nissued - q + STAGES - 1) / STAGES times
     bool ok = true;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      const int pb = t / ntiles1;
-      int tm, tn;
-      tile_coords(t - pb * ntiles1, tiles_m, tiles_n, GROUP_M, tm, tn);
-      const int nseg = grp.p[pb].nseg;
-      for (int kb = 0; kb < nseg * nkb; ++kb) {
+      int pb, tm, tn;
+      const Block blk = tile_at<SECT>(grp, list, t, bi, M, N, nkb, BM, BN, GROUP_M, pb, tm, tn);
+      const int ya = blk.a0 + tm * BM, yb = blk.b0 + tn * BN;
+      const int nk0 = blk.nk[0], nkbt = nk0 + (grp.p[pb].nseg > 1 ? blk.nk[1] : 0);
+      for (int kb = 0; kb < nkbt; ++kb) {
         if (!mbar_wait(&empty[s], ph ^ 1, status)) {
           ok = false;
           break;
         }
         uint8_t* st = smem + s * STAGE_BYTES;
-        const int sg = kb >= nkb ? 1 : 0, kq = kb - sg * nkb;
+        const int sg = kb >= nk0 ? 1 : 0, kq = kb - sg * nk0;
         const int wa = grp.p[pb].a[sg], wb = grp.p[pb].b[sg];
         const int pn = kq / nkbp, kx = (kq - pn * nkbp) * BK;
         mbar_expect_tx(&full[s], STAGE_BYTES);
-        tma_load(&mAhi, &full[s], st, kx, tm * BM, pn, wa);
-        tma_load(&mAlo, &full[s], st + A_BYTES, kx, tm * BM, pn, wa);
-        tma_load(&mBhi, &full[s], st + 2 * A_BYTES, kx, tn * BN, pn, wb);
-        tma_load(&mBlo, &full[s], st + 2 * A_BYTES + B_BYTES, kx, tn * BN, pn, wb);
+        tma_load(&mAhi, &full[s], st, kx, ya, pn, wa);
+        tma_load(&mAlo, &full[s], st + A_BYTES, kx, ya, pn, wa);
+        tma_load(&mBhi, &full[s], st + 2 * A_BYTES, kx, yb, pn, wb);
+        tma_load(&mBlo, &full[s], st + 2 * A_BYTES + B_BYTES, kx, yb, pn, wb);
         ++nissued;
         if (++s == STAGES) {
           s = 0;
@@ -422,7 +494,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t ph = 0, cph = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      const int nkbt = grp.p[t / ntiles1].nseg * nkb;
+      int pb, tm, tn;
+      const Block blk = tile_at<SECT>(grp, list, t, bi, M, N, nkb, BM, BN, GROUP_M, pb, tm, tn);
+      const int nkbt = blk.nk[0] + (grp.p[pb].nseg > 1 ? blk.nk[1] : 0);
       for (int kb = 0; kb < nkbt; ++kb) {
         const bool first = kb % KPC == 0;
         const bool last = kb % KPC == KPC - 1 || kb == nkbt - 1;
@@ -469,10 +543,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t cph = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      const int pb = t / ntiles1;
-      int tm, tn;
-      tile_coords(t - pb * ntiles1, tiles_m, tiles_n, GROUP_M, tm, tn);
-      const int nchunk = (grp.p[pb].nseg * nkb + KPC - 1) / KPC;
+      int pb, tm, tn;
+      const Block blk = tile_at<SECT>(grp, list, t, bi, M, N, nkb, BM, BN, GROUP_M, pb, tm, tn);
+      const int nchunk = (blk.nk[0] + (grp.p[pb].nseg > 1 ? blk.nk[1] : 0) + KPC - 1) / KPC;
       float acc[BN / 2];
 #pragma unroll
       for (int j = 0; j < BN / 2; ++j) acc[j] = 0.f;
@@ -492,7 +565,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
       if (!ok) break;
-      store_row(grp.p[pb].C, ldc, M, N, (int64_t)tm * BM + row, tn * BN + h * (BN / 2), acc, out_alpha(grp, pb));
+      store_row(grp.p[pb].C + blk.c0 * ldc, ldc, blk.rows, blk.cols, (int64_t)tm * BM + row, tn * BN + h * (BN / 2),
+                acc, out_alpha(grp, pb));
     }
   }
   fence_before();
@@ -509,7 +583,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // CTA) owns the full barriers of the copies, issues every MMA and collects the epilogue's
 // "chunk drained" arrivals of both CTAs; each CTA's empty and chunk-full barriers are
 // arrived at by rank 0's commits, one commit per barrier.
-template <class CF>
+template <class CF, bool SECT>
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__ CUtensorMap mAlo,
                      const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo,
@@ -531,10 +605,12 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const int cid = blockIdx.x / 2, ncl = gridDim.x / 2;
-  const int tiles_m = (M + BM - 1) / BM, tiles_n = (N + BN - 1) / BN;
-  const int tiles_mg = (tiles_m + 1) / 2;               // 256-row tiles
-  const int ntiles1 = tiles_mg * tiles_n;               // tiles of one output
-  const int ntiles = grp.nprob * ntiles1;
+  constexpr int TM = 2 * BM;                            // tile rows of the pair
+  BlockList* list = nullptr;
+  if constexpr (SECT) {
+    __shared__ BlockList list_mem;
+    list = &list_mem;
+  }
   const int nkbp = (Kp + BK - 1) / BK;
   const int nkb = P * nkbp;                             // k-blocks of one segment
 
@@ -557,10 +633,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
+  if constexpr (SECT) list_blocks(grp, *list, BK, TM, BN);
   fence_before();
   cluster_sync_all();   // both CTAs' barriers initialised and TMEM allocated before any use
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  int ntiles;
+  if constexpr (SECT) ntiles = list->first[2 * grp.nprob];
+  else ntiles = grp.nprob * ((M + TM - 1) / TM) * ((N + BN - 1) / BN);
+  int bi = 0;                            // block of the role's current tile
 
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------ TMA producer (both CTAs)
@@ -574,25 +655,24 @@ __global__ void __launch_bounds__(THREADS, 1)
     int nissued = 0;   // k-blocks issued; stage q has been filled (nissued - q + STAGES - 1) / STAGES times
     bool ok = true;
     for (int t = cid; t < ntiles && ok; t += ncl) {
-      const int pb = t / ntiles1;
-      int tg, tn;
-      tile_coords(t - pb * ntiles1, tiles_mg, tiles_n, GROUP_M / 2, tg, tn);
-      const int tm = 2 * tg + (int)rank;
-      const int yb = tn * BN + (int)rank * (BN / 2);
-      const int nseg = grp.p[pb].nseg;
-      for (int kb = 0; kb < nseg * nkb; ++kb) {
+      int pb, tg, tn;
+      const Block blk = tile_at<SECT>(grp, list, t, bi, M, N, nkb, TM, BN, GROUP_M / 2, pb, tg, tn);
+      const int ya = blk.a0 + tg * TM + (int)rank * BM;
+      const int yb = blk.b0 + tn * BN + (int)rank * (BN / 2);
+      const int nk0 = blk.nk[0], nkbt = nk0 + (grp.p[pb].nseg > 1 ? blk.nk[1] : 0);
+      for (int kb = 0; kb < nkbt; ++kb) {
         if (!mbar_wait<true>(&empty[s], ph ^ 1, status)) {
           ok = false;
           break;
         }
         uint8_t* st = smem + s * STAGE_BYTES;
-        const int sg = kb >= nkb ? 1 : 0, kq = kb - sg * nkb;
+        const int sg = kb >= nk0 ? 1 : 0, kq = kb - sg * nk0;
         const int wa = grp.p[pb].a[sg], wb = grp.p[pb].b[sg];
         const int pn = kq / nkbp, kx = (kq - pn * nkbp) * BK;
         if (rank == 0) mbar_expect_tx(&full[s], 2 * STAGE_BYTES);   // this CTA's and the partner's copies
         const uint32_t fb = full0 + (uint32_t)(s * sizeof(uint64_t));
-        tma_load_pair(&mAhi, fb, st, kx, tm * BM, pn, wa);
-        tma_load_pair(&mAlo, fb, st + A_BYTES, kx, tm * BM, pn, wa);
+        tma_load_pair(&mAhi, fb, st, kx, ya, pn, wa);
+        tma_load_pair(&mAlo, fb, st + A_BYTES, kx, ya, pn, wa);
         tma_load_pair(&mBhi, fb, st + 2 * A_BYTES, kx, yb, pn, wb);
         tma_load_pair(&mBlo, fb, st + 2 * A_BYTES + B_BYTES, kx, yb, pn, wb);
         ++nissued;
@@ -614,7 +694,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t ph = 0, cph = 0;
     bool ok = true;
     for (int t = cid; t < ntiles && ok; t += ncl) {
-      const int nkbt = grp.p[t / ntiles1].nseg * nkb;
+      int pb, tg, tn;
+      const Block blk = tile_at<SECT>(grp, list, t, bi, M, N, nkb, TM, BN, GROUP_M / 2, pb, tg, tn);
+      const int nkbt = blk.nk[0] + (grp.p[pb].nseg > 1 ? blk.nk[1] : 0);
       for (int kb = 0; kb < nkbt; ++kb) {
         const bool first = kb % KPC == 0;
         const bool last = kb % KPC == KPC - 1 || kb == nkbt - 1;
@@ -663,11 +745,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t cph = 0;
     bool ok = true;
     for (int t = cid; t < ntiles && ok; t += ncl) {
-      const int pb = t / ntiles1;
-      int tg, tn;
-      tile_coords(t - pb * ntiles1, tiles_mg, tiles_n, GROUP_M / 2, tg, tn);
-      const int tm = 2 * tg + (int)rank;
-      const int nchunk = (grp.p[pb].nseg * nkb + KPC - 1) / KPC;
+      int pb, tg, tn;
+      const Block blk = tile_at<SECT>(grp, list, t, bi, M, N, nkb, TM, BN, GROUP_M / 2, pb, tg, tn);
+      const int nchunk = (blk.nk[0] + (grp.p[pb].nseg > 1 ? blk.nk[1] : 0) + KPC - 1) / KPC;
       float acc[BN / 2];
 #pragma unroll
       for (int j = 0; j < BN / 2; ++j) acc[j] = 0.f;
@@ -687,7 +767,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
       if (!ok) break;
-      store_row(grp.p[pb].C, ldc, M, N, (int64_t)tm * BM + row, tn * BN + h * (BN / 2), acc, out_alpha(grp, pb));
+      store_row(grp.p[pb].C + blk.c0 * ldc, ldc, blk.rows, blk.cols, (int64_t)tg * TM + (int)rank * BM + row,
+                tn * BN + h * (BN / 2), acc, out_alpha(grp, pb));
     }
   }
   fence_before();
@@ -768,7 +849,8 @@ __device__ __forceinline__ void two_sum_into(float& hi, float& lo, float x) {
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     gemm_oz_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB,
                    double* __restrict__ C, int64_t ldc, int M, int N, int Kp, int P, double alpha,
-                   const unsigned* amax_a, const unsigned* amax_b, int accumulate, int* status) {
+                   const unsigned* amax_a, const unsigned* amax_b, int accumulate, int* status,
+                   const __grid_constant__ OneProduct one) {
   using CF = CfgOz;
   constexpr int STAGES = CF::STAGES, BK = CF::BK, STAGE_BYTES = CF::STAGE_BYTES, KPC = CF::KB_PER_CHUNK;
   extern __shared__ uint8_t smem_raw[];
@@ -782,11 +864,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   uint32_t* tmem_slot = (uint32_t*)(drain + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tiles_m = (M + BM - 1) / BM, tiles_n = (N + OZ_BN - 1) / OZ_BN;
-  const int ntiles = tiles_m * tiles_n;
   const int nkbp = (Kp + BK - 1) / BK;
   const int nkb = P * nkbp;
-  const int nchunk = (nkb + KPC - 1) / KPC;
+  // the blocks of the product (see Block): both charges of a sector product, or the whole output
+  __shared__ Block blks[2];
+  if (threadIdx.x < 2) {
+    const int q = threadIdx.x;
+    blks[q] = one.sec.tab.base ? sector_block(*one.sec.tab.at(one.elem).plan, one.sec, q, one.pa, one.pa, one.parity, BK)
+                               : Block{q ? 0 : M, N, 0, 0, 0, {nkb, nkb}};
+  }
+  __syncthreads();
+  const int nt0 = ((blks[0].rows + BM - 1) / BM) * ((blks[0].cols + OZ_BN - 1) / OZ_BN);
+  const int ntiles = nt0 + ((blks[1].rows + BM - 1) / BM) * ((blks[1].cols + OZ_BN - 1) / OZ_BN);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -817,9 +906,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     uint32_t ph = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      const Block& blk = blks[t >= nt0];
       int tm, tn;
-      tile_coords(t, tiles_m, tiles_n, GROUP_M, tm, tn);
-      for (int kb = 0; kb < nkb; ++kb) {
+      tile_coords(t >= nt0 ? t - nt0 : t, (blk.rows + BM - 1) / BM, (blk.cols + OZ_BN - 1) / OZ_BN, GROUP_M, tm, tn);
+      const int nkbt = blk.nk[0];
+      for (int kb = 0; kb < nkbt; ++kb) {
         if (!mbar_wait(&empty[s], ph ^ 1, status)) {
           ok = false;
           break;
@@ -829,8 +920,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         mbar_expect_tx(&full[s], STAGE_BYTES);
 #pragma unroll
         for (int q = 0; q < kOzSlices; ++q) {
-          tma_load(&mA, &full[s], st + q * CF::A_PLANE, kx, tm * BM, pn, q);
-          tma_load(&mB, &full[s], st + kOzSlices * CF::A_PLANE + q * CF::B_PLANE, kx, tn * OZ_BN, pn, q);
+          tma_load(&mA, &full[s], st + q * CF::A_PLANE, kx, blk.a0 + tm * BM, pn, q);
+          tma_load(&mB, &full[s], st + kOzSlices * CF::A_PLANE + q * CF::B_PLANE, kx, blk.b0 + tn * OZ_BN, pn, q);
         }
         ++nissued;
         if (++s == STAGES) {
@@ -847,9 +938,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     uint32_t ph = 0, cph = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-      for (int kb = 0; kb < nkb; ++kb) {
+      const int nkbt = blks[t >= nt0].nk[0];
+      for (int kb = 0; kb < nkbt; ++kb) {
         const bool first = kb % KPC == 0;
-        const bool last = kb % KPC == KPC - 1 || kb == nkb - 1;
+        const bool last = kb % KPC == KPC - 1 || kb == nkbt - 1;
         if ((first && !mbar_wait(cempty, cph ^ 1, status)) || !mbar_wait(&full[s], ph, status)) {
           ok = false;
           break;
@@ -892,8 +984,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     uint32_t cph = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+      const Block& blk = blks[t >= nt0];
+      const int nchunk = (blk.nk[0] + KPC - 1) / KPC;
       int tm, tn;
-      tile_coords(t, tiles_m, tiles_n, GROUP_M, tm, tn);
+      tile_coords(t >= nt0 ? t - nt0 : t, (blk.rows + BM - 1) / BM, (blk.cols + OZ_BN - 1) / OZ_BN, GROUP_M, tm, tn);
       float hi[OZ_COLS], lo[OZ_COLS];
 #pragma unroll
       for (int j = 0; j < OZ_COLS; ++j) hi[j] = lo[j] = 0.f;
@@ -933,14 +1027,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       if (!ok) break;
       const int64_t m = (int64_t)tm * BM + row;
       const int n0 = tn * OZ_BN + cpart * OZ_COLS;
-      if (m < M) {
-        double* crow = C + m * ldc + n0;
+      if (m < blk.rows) {
+        double* crow = C + (blk.c0 + m) * ldc + n0;
         // alpha 2^-16, and 2^-(eA + eB) for the operands' max-norm scales
         const int es = amax_a ? split_exponent(*amax_a, kOzTop) + split_exponent(*amax_b, kOzTop) : 0;
         const double a16 = ldexp(alpha, -16 - es);
 #pragma unroll
         for (int j = 0; j < OZ_COLS; ++j)
-          if (n0 + j < N) crow[j] = a16 * ((double)hi[j] + (double)lo[j]) + (accumulate ? crow[j] : 0.0);
+          if (n0 + j < blk.cols) crow[j] = a16 * ((double)hi[j] + (double)lo[j]) + (accumulate ? crow[j] : 0.0);
       }
     }
   }
@@ -1000,25 +1094,22 @@ const DeviceSetup* device_setup() {
   DeviceSetup& d = g_setup[dev];
   if (d.done) return &d;
   if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return nullptr;
-  bool ok = cudaFuncSetAttribute(gemm_tf32x3_kernel<CfgTF32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)CfgTF32::SMEM_BYTES) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(gemm_tf32x3_kernel<CfgTF32W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)CfgTF32W::SMEM_BYTES) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(gemm_tf32x3_kernel<CfgF16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)CfgF16::SMEM_BYTES) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(gemm_tf32x3_kernel<CfgF16S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)CfgF16S::SMEM_BYTES) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(gemm_tf32x3_kernel<CfgF16L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)CfgF16L::SMEM_BYTES) == cudaSuccess;
-  ok = ok && cudaFuncSetAttribute(gemm_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)CfgOz::SMEM_BYTES) == cudaSuccess;
+  auto smem_ok = [](auto kernel, size_t bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+  };
+  auto single_ok = [&](auto cfg) {
+    using CF = decltype(cfg);
+    return smem_ok(gemm_tf32x3_kernel<CF, false>, CF::SMEM_BYTES) && smem_ok(gemm_tf32x3_kernel<CF, true>, CF::SMEM_BYTES);
+  };
+  const bool ok = single_ok(CfgTF32{}) && single_ok(CfgTF32W{}) && single_ok(CfgF16{}) && single_ok(CfgF16S{}) &&
+                  single_ok(CfgF16L{}) && smem_ok(gemm_oz_kernel, CfgOz::SMEM_BYTES);
   if (!ok) {
     cudaGetLastError();
     return nullptr;
   }
   int n = 0;
-  if (cudaFuncSetAttribute(gemm_pair_kernel<CfgF16P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)CfgF16P::SMEM_BYTES) == cudaSuccess) {
+  if (smem_ok(gemm_pair_kernel<CfgF16P, false>, CfgF16P::SMEM_BYTES) &&
+      smem_ok(gemm_pair_kernel<CfgF16P, true>, CfgF16P::SMEM_BYTES)) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1030,7 +1121,7 @@ const DeviceSetup* device_setup() {
     cfg.dynamicSmemBytes = CfgF16P::SMEM_BYTES;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<CfgF16P>, &cfg) != cudaSuccess) n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<CfgF16P, true>, &cfg) != cudaSuccess) n = 0;
   }
   cudaGetLastError();
   d.pair_grid = 2 * n;
@@ -1046,10 +1137,11 @@ cudaError_t launch_single(const void* Ahi, const void* Alo, const void* Bhi, con
   if (!make_map<CF>(&mAhi, Ahi, M, Kp, kps, P, W, aws, BM) || !make_map<CF>(&mAlo, Alo, M, Kp, kps, P, W, aws, BM) ||
       !make_map<CF>(&mBhi, Bhi, N, Kp, kps, P, W, bws, BN) || !make_map<CF>(&mBlo, Blo, N, Kp, kps, P, W, bws, BN))
     return cudaErrorInvalidValue;
-  const int64_t tiles = g.nprob * ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+  const int64_t more = g.sec.tab.base ? 1 : 0;   // two sectors: at most one more tile row and column
+  const int64_t tiles = g.nprob * ((M + BM - 1) / BM + more) * ((N + BN - 1) / BN + more);
   const int grid = (int)(tiles < dv.sms ? tiles : dv.sms);
-  gemm_tf32x3_kernel<CF><<<grid, THREADS, CF::SMEM_BYTES, st>>>(mAhi, mAlo, mBhi, mBlo, g, ldc, (int)M, (int)N,
-                                                               (int)Kp, (int)P, status);
+  auto kernel = g.sec.tab.base ? gemm_tf32x3_kernel<CF, true> : gemm_tf32x3_kernel<CF, false>;
+  kernel<<<grid, THREADS, CF::SMEM_BYTES, st>>>(mAhi, mAlo, mBhi, mBlo, g, ldc, (int)M, (int)N, (int)Kp, (int)P, status);
   return cudaGetLastError();
 }
 
@@ -1063,7 +1155,8 @@ cudaError_t launch_pair(const void* Ahi, const void* Alo, const void* Bhi, const
       !make_map<CF>(&mBhi, Bhi, N, Kp, kps, P, W, bws, BN / 2) ||
       !make_map<CF>(&mBlo, Blo, N, Kp, kps, P, W, bws, BN / 2))
     return cudaErrorInvalidValue;
-  const int64_t pairs = g.nprob * ((M + 2 * BM - 1) / (2 * BM)) * ((N + BN - 1) / BN);
+  const int64_t more = g.sec.tab.base ? 1 : 0;   // two sectors: at most one more tile row and column
+  const int64_t pairs = g.nprob * ((M + 2 * BM - 1) / (2 * BM) + more) * ((N + BN - 1) / BN + more);
   int grid = dv.pair_grid;
   if (grid / 2 > pairs) grid = (int)(2 * pairs);
   cudaLaunchConfig_t cfg = {};
@@ -1078,7 +1171,7 @@ cudaError_t launch_pair(const void* Ahi, const void* Alo, const void* Bhi, const
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, gemm_pair_kernel<CF>, mAhi, mAlo, mBhi, mBlo, g, ldc, (int)M, (int)N, (int)Kp,
+  return cudaLaunchKernelEx(&cfg, g.sec.tab.base ? gemm_pair_kernel<CF, true> : gemm_pair_kernel<CF, false>, mAhi, mAlo, mBhi, mBlo, g, ldc, (int)M, (int)N, (int)Kp,
                             (int)P, status);
 }
 
@@ -1107,7 +1200,9 @@ cudaError_t launch_gemm_group(const void* Ahi, const void* Alo, const void* Bhi,
     for (int sg = 0; sg < pr.nseg; ++sg)
       if (pr.a[sg] < 0 || pr.a[sg] >= W || pr.b[sg] < 0 || pr.b[sg] >= W) return cudaErrorInvalidValue;
   }
-  if ((g.amax_a == nullptr) != (g.amax_b == nullptr) || (g.amax_a && g.per_elem < 1)) return cudaErrorInvalidValue;
+  if ((g.amax_a == nullptr) != (g.amax_b == nullptr) || ((g.amax_a || g.sec.tab.base) && g.per_elem < 1))
+    return cudaErrorInvalidValue;
+  if (g.sec.tab.base) Kp = kps;   // packed summed indices fill whole panel rows, k-blocks run over the padding
   const bool f16 = variant >= 2 && variant <= 5;
   if ((kps & (variant == 5 ? 63 : (f16 ? 7 : 3))) || kps < Kp) return cudaErrorInvalidValue;
   if ((((uintptr_t)Ahi) | ((uintptr_t)Alo) | ((uintptr_t)Bhi) | ((uintptr_t)Blo)) & 15) return cudaErrorInvalidValue;
@@ -1130,8 +1225,10 @@ cudaError_t launch_gemm_group(const void* Ahi, const void* Alo, const void* Bhi,
 // K panels, plane p of A at A + p aps elements (B: bps); kps % 8 == 0.
 cudaError_t launch_gemm_oz(const void* A, const void* B, int64_t aps, int64_t bps, int64_t Kp, int64_t kps, int64_t P,
                            int64_t M, int64_t N, double* C, int64_t ldc, double alpha, const unsigned* amax_a,
-                           const unsigned* amax_b, bool accumulate, int* status, cudaStream_t st) {
+                           const unsigned* amax_b, bool accumulate, int* status, cudaStream_t st,
+                           const OneProduct& one) {
   using namespace tc;
+  if (one.sec.tab.base) Kp = kps;
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (!A || !B || !C || Kp <= 0 || P <= 0 || M > 0x7fffffff || N > 0x7fffffff || Kp * P > 0x7fffffff || ldc < N ||
       (kps & 7) || kps < Kp || aps < P * M * kps || bps < P * N * kps)
@@ -1143,11 +1240,12 @@ cudaError_t launch_gemm_oz(const void* A, const void* B, int64_t aps, int64_t bp
   if (!make_map<CfgOz>(&mA, A, M, Kp, kps, P, kOzSlices, aps, BM) ||
       !make_map<CfgOz>(&mB, B, N, Kp, kps, P, kOzSlices, bps, OZ_BN))
     return cudaErrorInvalidValue;
-  const int64_t tiles = ((M + BM - 1) / BM) * ((N + OZ_BN - 1) / OZ_BN);
+  const int64_t more = one.sec.tab.base ? 1 : 0;
+  const int64_t tiles = ((M + BM - 1) / BM + more) * ((N + OZ_BN - 1) / OZ_BN + more);
   const int grid = (int)(tiles < dv->sms ? tiles : dv->sms);
   if ((amax_a == nullptr) != (amax_b == nullptr)) return cudaErrorInvalidValue;
   gemm_oz_kernel<<<grid, OZ_THREADS, CfgOz::SMEM_BYTES, st>>>(mA, mB, C, ldc, (int)M, (int)N, (int)Kp, (int)P, alpha,
-                                                              amax_a, amax_b, accumulate ? 1 : 0, status);
+                                                              amax_a, amax_b, accumulate ? 1 : 0, status, one);
   return cudaGetLastError();
 }
 

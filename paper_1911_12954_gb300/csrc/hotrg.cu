@@ -62,6 +62,7 @@ struct StepPlan {
   int Rmax, nmax, nchunks;
   int batch;              // batch elements whose isometry stages run together
   int ne;                 // batch elements contracted together (one group of launches)
+  bool sect;              // contraction by Z2 charge sectors (sectors.cu)
   int gemm_opt;           // tensor-core GEMM pipeline option of this step (-1: the context's)
   bool tuned;             // closing direction and pipeline taken from the autotuner's cache
   double main_flops, total_flops;
@@ -69,7 +70,7 @@ struct StepPlan {
 
 struct Layout {
   // persistent
-  size_t status, step, lnz, cval, trace, rec, beta, hfield, U64, Ur, tensors;
+  size_t status, step, lnz, cval, trace, rec, beta, hfield, sectors, U64, Ur, tensors;
   int64_t cap;            // elements per tensor slot
   size_t persistent_end;
 };
@@ -87,6 +88,7 @@ struct hotrg_ctx {
   Layout L{};
   bool ready = false;        // workspace laid out
   bool initialised = false;  // tensors exist
+  bool sectors = false;      // every element's tensors conserve the Z2 charge (no field)
   int sticky = 0;
   int k = 0;
   int dims[4] = {2, 2, 2, 2};
@@ -362,10 +364,31 @@ int ntensors(int impure) { return (impure & HOTRG_IMPURE_SIGMASIGMA) ? 3 : ((imp
 struct Scratch {
   size_t gpart, npart, gA, G, jwork, lam, eps, degen, Uside;
   size_t O1A, A, Alo, O1B, B, Blo, C, O3;
+  size_t tab;             // sector tables, one set per element of a group
   size_t amax;            // operand magnitude bounds of the current A and B per element (max-norm scaling)
   size_t stats;           // counters of hotrg_split_stats
   size_t total;
 };
+
+// Sector tables of one element (see SectorTables); base is set by the caller.
+SectorTab sector_tab(const StepPlan& p) {
+  SectorTab t{};
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = off;
+    off = align_up(off + bytes, 256);
+    return (int64_t)o;
+  };
+  const int64_t groups = p.rowsA_full / p.D[p.c];
+  t.o_plan = take(sizeof(SectorPlan));
+  t.o_row = take(p.rowsA_full * sizeof(uint32_t));
+  t.o_kA = take(p.K * sizeof(uint2));
+  t.o_kB = take(p.K * sizeof(uint2));
+  t.o_grank = take(groups * sizeof(uint32_t));
+  t.o_grp = take(groups * sizeof(uint32_t));
+  t.stride = (int64_t)off;
+  return t;
+}
 
 Scratch scratch_layout(const StepPlan& p, int xs, int xs2, int prec, int impure, size_t rs) {
   Scratch s{};
@@ -401,6 +424,7 @@ Scratch scratch_layout(const StepPlan& p, int xs, int xs2, int prec, int impure,
   s.Blo = split ? take(ne * nt * p.P * rowsB * p.kps * os) : 0;
   s.C = take(ne * nt * rowsA * rowsB * rs);
   s.O3 = take(ne * (size_t)(rowsA * rowsB / (p.D[p.c] * p.D[p.c]) * p.chi[p.c]) * rs);
+  s.tab = p.sect ? take(ne * sector_tab(p).stride) : 0;
   s.amax = take(2 * ne * nt * sizeof(unsigned));   // A side, then B side: per element (and tensor)
   s.stats = take(4 * 3 * sizeof(unsigned long long));   // hotrg_split_stats counters
   s.total = off;
@@ -423,6 +447,7 @@ Layout persistent_layout(int batch, int64_t cap, int impure, size_t rs) {
   L.rec = take((size_t)batch * kMaxSteps * sizeof(DevRecord));
   L.beta = take(batch * 8);
   L.hfield = take(batch * 8);
+  L.sectors = take(batch * sizeof(SectorState));
   L.U64 = take((size_t)batch * 4 * kMaxGramN * kMaxLeg * 8);
   L.Ur = take((size_t)batch * 4 * kMaxGramN * kMaxLeg * rs);
   L.cap = cap;
@@ -520,10 +545,53 @@ void operand_strides(const StepPlan& p, const std::vector<int64_t>& rn, int64_t 
   }
 }
 
+// Second half-contraction pass of one tensor by charge sectors. O1 is the first pass's output
+// [X, contracted leg, c, c', mu, summed legs] with strides os; side 0: A (contracts b1 of
+// U^b[b1, b2, Y]), 1: B (contracts b2' of U^b[b1', b2', Y']).
+template <typename R>
+hotrg_status sector_operand(hotrg_ctx* ctx, const StepPlan& p, int side, const R* Ub, int x0, int xs, const int64_t* os,
+                            R* O1, R* out, R* out_lo, cudaStream_t st, const ElemStrides& es, unsigned* amax,
+                            int amax_bs, int scale, int phases, const SectorTab& tab, int parity) {
+  const int Db = p.D[p.b], Dc = p.D[p.c], Dm = p.D[p.mu], cb = p.chi[p.b];
+  SectorOperand a{};
+  a.tab = tab;
+  a.sideB = side;
+  a.parity = parity;
+  a.x0 = x0;
+  a.xs = xs;
+  a.cb = cb;
+  a.Db = Db;
+  a.Dc = Dc;
+  a.Dm = Dm;
+  a.nouter = xs * Dc * Dc * Dm;
+  a.in_x = os[0];
+  a.in_j = os[1];
+  a.in_c0 = os[2];
+  a.in_c1 = os[3];
+  a.in_m = os[4];
+  a.u_j = side == 0 ? Db * cb : cb;
+  a.u_r = side == 0 ? cb : Db * cb;
+  a.rows = (int64_t)xs * cb * Dc * Dc * Dm;
+  a.kps = p.kps;
+  a.P = (int)p.P;
+  a.kalign = panel_mode(ctx->prec) ? 128 / (int)operand_size(ctx->prec) : 2;
+  a.in_bs = es.O1;
+  a.u_bs = es.U;
+  a.out_bs = es.op;
+  a.amax = amax;
+  a.amax_mul = 1.0f;
+  a.amax_bs = amax_bs;
+  const int mode = !out_lo ? kTTMStore : split_mode(ctx->prec);
+  if ((phases & kPassMax) && amax && scale == kScaleExact)
+    LK(1, launch_sector_operand<R>(O1, Ub, out, out_lo, a, es.ne, kTTMMaxAbs, st), "sector operand max");
+  if (phases & kPass2) LK(1, launch_sector_operand<R>(O1, Ub, out, out_lo, a, es.ne, mode, st), "sector operand");
+  return HOTRG_OK;
+}
+
 template <typename R>
 hotrg_status build_A(hotrg_ctx* ctx, const StepPlan& p, const R* P, const R* Ua, const R* Ub, int x0, int xs,
                      R* O1, R* A, R* Alo, cudaStream_t st, const ElemStrides& es, unsigned* amax, int amax_bs,
-                     int scale, int phases) {
+                     int scale, int phases, const SectorTab& tab, int parity) {
   const int mu = p.mu, a = p.a, b = p.b, c = p.c;
   const int Da = p.D[a], Db = p.D[b], Dc = p.D[c], Dm = p.D[mu];
   const int ca = p.chi[a], cb = p.chi[b];
@@ -555,6 +623,7 @@ hotrg_status build_A(hotrg_ctx* ctx, const StepPlan& p, const R* P, const R* Ua,
     if (phases & kPass1) LK(1, launch_ttm_r<R>(P, Ua + x0, O1, nullptr, t, bound ? kTTMStoreMax : kTTMStore, st), "ttm A1");
   }
   // A[(X Y c1 c1' mu1), (a2 b2 a1' b1' k)] = sum_b1 U^b[b1, b2, Y] O1[X, b1, ...]
+  if (p.sect) return sector_operand<R>(ctx, p, 0, Ub, x0, xs, os.data(), O1, A, Alo, st, es, amax, amax_bs, scale, phases, tab, parity);
   {
     int64_t o[10];
     operand_strides(p, {xs, cb, Dc, Dc, Dm}, o);
@@ -586,7 +655,7 @@ hotrg_status build_A(hotrg_ctx* ctx, const StepPlan& p, const R* P, const R* Ua,
 template <typename R>
 hotrg_status build_B(hotrg_ctx* ctx, const StepPlan& p, const R* Q, const R* Ua, const R* Ub, int x0, int xs,
                      R* O1, R* B, R* Blo, cudaStream_t st, const ElemStrides& es, unsigned* amax, int amax_bs,
-                     int scale, int phases) {
+                     int scale, int phases, const SectorTab& tab, int parity) {
   const int mu = p.mu, a = p.a, b = p.b, c = p.c;
   const int Da = p.D[a], Db = p.D[b], Dc = p.D[c], Dm = p.D[mu];
   const int ca = p.chi[a], cb = p.chi[b];
@@ -617,6 +686,7 @@ hotrg_status build_B(hotrg_ctx* ctx, const StepPlan& p, const R* Q, const R* Ua,
     }
     if (phases & kPass1) LK(1, launch_ttm_r<R>(Q, Ua + x0, O1, nullptr, t, bound ? kTTMStoreMax : kTTMStore, st), "ttm B1");
   }
+  if (p.sect) return sector_operand<R>(ctx, p, 1, Ub, x0, xs, os.data(), O1, B, Blo, st, es, amax, amax_bs, scale, phases, tab, parity);
   {
     int64_t o[10];
     operand_strides(p, {xs, cb, Dc, Dc, Dm}, o);
@@ -648,10 +718,52 @@ hotrg_status build_B(hotrg_ctx* ctx, const StepPlan& p, const R* Q, const R* Ua,
 // T'[slice] = C x_{(c1 c2)} U^c x_{(c1' c2')} U^c, written into the canonical layout.
 template <typename R>
 hotrg_status close_C(hotrg_ctx* ctx, const StepPlan& p, const R* C, const R* Uc, int x0, int xs, int x20, int xs2,
-                     R* O3, R* Tn, cudaStream_t st, const ElemStrides& es) {
+                     R* O3, R* Tn, cudaStream_t st, const ElemStrides& es, const SectorTab& tab, int parity) {
   const int mu = p.mu, a = p.a, b = p.b, c = p.c;
   const int Dc = p.D[c], Dm = p.D[mu];
   const int cb = p.chi[b], cc = p.chi[c];
+  if (p.sect) {
+    SectorClose s{};
+    s.tab = tab;
+    s.parity = parity;
+    s.x0 = x0;
+    s.xs = xs;
+    s.x20 = x20;
+    s.xs2 = xs2;
+    s.ca = p.chi[a];
+    s.cb = cb;
+    s.cc = cc;
+    s.Dc = Dc;
+    s.Dm = Dm;
+    s.ldc = (int64_t)xs2 * cb * Dc * Dc * Dm;
+    s.c_bs = es.C;
+    s.u_bs = es.U;
+    s.o3_bs = es.O3;
+    s.t_bs = es.T;
+    int64_t tn[8];
+    canon_strides(p.newD, tn);
+    const int gx = cb * Dc * Dm, gy = Dc * Dm;   // strides of X and Y in a row group (X, Y, c', mu)
+    s.nfib = 1;
+    int d = 0;
+    for (int leg = 0; leg < 8; ++leg) {
+      const int n = leg / 2, pr = leg % 2;
+      if (n == c && pr == 1) {
+        s.tz = tn[leg];
+        continue;
+      }
+      s.fd[d] = n == a ? (pr == 0 ? xs : xs2) : p.newD[n];
+      const int g = n == a ? gx : (n == b ? gy : (n == mu ? 1 : 0));
+      s.fm[d] = pr == 0 ? g : 0;
+      s.fn[d] = pr == 1 ? g : 0;
+      s.fz[d] = n == c ? 1 : 0;
+      s.ft[d] = tn[leg];
+      s.nfib *= s.fd[d];
+      ++d;
+    }
+    R* out = Tn + (int64_t)x0 * tn[2 * a] + (int64_t)x20 * tn[2 * a + 1];
+    LK(2, launch_sector_close<R>(C, Uc, O3, out, s, es.ne, st), "sector close");
+    return HOTRG_OK;
+  }
   // C block: rows m = (X, Y, c1, c1', mu1), X in [x0, x0 + xs); columns n = (X', Y', c2, c2', mu2'),
   // X' in [x20, x20 + xs2); row-major with N = its column count
   const int64_t N = (int64_t)xs2 * cb * Dc * Dc * Dm;
@@ -749,12 +861,12 @@ struct GemmTimer {
 // CUDA-core GEMM (FP64 and FP32 modes): C = alpha A B^T + beta C, one product per launch.
 template <typename R>
 hotrg_status gemm_simt(hotrg_ctx* ctx, const R* A, const R* B, const StepPlan& p, R* C, int64_t M, int64_t N,
-                       double alpha, double beta, cudaStream_t st) {
+                       double alpha, double beta, cudaStream_t st, const OneProduct& one) {
   if (p.P != 1) return HOTRG_EUNSUPPORTED;
   GemmTimer tm{ctx, st};
   hotrg_status r = tm.start();
   if (r != HOTRG_OK) return r;
-  CK(launch_gemm_simt<R>(A, p.kps, B, p.kps, C, N, M, N, p.K, alpha, beta, st), "gemm simt");
+  CK(launch_gemm_simt<R>(A, p.kps, B, p.kps, C, N, M, N, p.K, alpha, beta, st, one), "gemm simt");
   return tm.stop(2.0 * (double)M * (double)N * (double)p.K);
 }
 
@@ -895,6 +1007,10 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
     j.rec_b = rec;
     j.step = dstep;
     j.nu = n;
+    j.sectors = ctx->sectors ? (SectorState*)(ctx->ws + ctx->L.sectors) : nullptr;
+    j.cur = ctx->cur;
+    j.mu = mu;
+    j.Dn = p.D[n];
   }
   sp.batch = nb;
   sp.sU = ep.sU;
@@ -987,6 +1103,37 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
     esB.op = nt * Bsz * planes;
     esC.C = nt * Csz;
     esC.O3 = rowsA * rowsB / ((int64_t)p.D[p.c] * p.D[p.c]) * p.chi[p.c];
+    // charge sectors of the group's elements (ranks and extents stay on the device)
+    SectorTab tab{};
+    if (p.sect) {
+      tab = sector_tab(p);
+      tab.base = sb + sc.tab;
+      SectorArgs a{};
+      a.state = (const SectorState*)(ctx->ws + ctx->L.sectors) + e0;
+      a.tab = tab;
+      a.cur = ctx->cur;
+      a.a = p.a;
+      a.b = p.b;
+      a.c = p.c;
+      a.mu = mu;
+      a.Da = p.D[p.a];
+      a.Db = p.D[p.b];
+      a.Dc = p.D[p.c];
+      a.Dm = p.D[mu];
+      a.ca = ca;
+      a.cb = p.chi[p.b];
+      // first passes' summed legs, innermost last: A (a2, a1', b1', k), B (a2, b2, a1', k)
+      const uint32_t Da = a.Da, Db = a.Db, Dm = a.Dm;
+      a.kA[4] = a.kB[4] = 1;
+      a.kA[3] = Dm;
+      a.kA[2] = Db * Dm;
+      a.kA[0] = Da * Db * Dm;
+      a.kB[2] = Dm;
+      a.kB[1] = Da * Dm;
+      a.kB[0] = Db * Da * Dm;
+      LK(1, launch_sector_tables(a, ne, st), "sector tables");
+    }
+    const int parity[3] = {0, 1, 0};   // T, S (one sigma: odd), M (two)
     // Padding columns of a panel (kin >= Kp) are never read: the tensor maps stop at Kp and
     // the CUDA-core GEMM at K, so the operand buffers need no clearing.
     // every tensor's first pass, then (exact scaling) the max pass of every tensor, then the
@@ -1000,7 +1147,7 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
         for (int w = 0; w < nbuild; ++w) {
           hotrg_status s = build_B<R>(ctx, p, src[w], Ua, Ub, x20, xs2, O1B + w * O1Bsz, opnd(Bbuf, w * Bsz * planes),
                                       opnd(Blob, w * Bsz * planes), st, esB, amaxB ? amaxB + (tw > 1 ? w : 0) : nullptr,
-                                      tw, scale, ph);
+                                      tw, scale, ph, tab, parity[w]);
           if (s != HOTRG_OK) return s;
         }
       }
@@ -1015,7 +1162,8 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
     for (int x0 = 0; x0 < xend; x0 += p.xs) {
       const int xs = std::min(p.xs, ca - x0);
       const int64_t rA_full = (int64_t)xs * p.chi[p.b] * p.D[p.c] * p.D[p.c] * p.D[mu];
-      const int64_t rA = pr.gemm_rows > 0 ? std::min(rA_full, pr.gemm_rows) : rA_full;
+      // a probe's rows: the first ones, or (sectors) the first half of them in either sector
+      const int64_t rA = pr.gemm_rows > 0 && !p.sect ? std::min(rA_full, pr.gemm_rows) : rA_full;
       for (int ph : {kPass1, kPassMax, kPass2}) {
         if (!pr.ttm) break;
         if (ph == kPassMax && scale != kScaleExact) continue;
@@ -1023,7 +1171,7 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
         for (int w = 0; w < nbuild; ++w) {
           hotrg_status s = build_A<R>(ctx, p, src[w], Ua, Ub, x0, xs, O1A + w * O1Asz, opnd(Abuf, w * Asz * planes),
                                       opnd(Alob, w * Asz * planes), st, esA, amaxA ? amaxA + (tw > 1 ? w : 0) : nullptr,
-                                      tw, scale, ph);
+                                      tw, scale, ph, tab, parity[w]);
           if (s != HOTRG_OK) return s;
         }
       }
@@ -1035,6 +1183,8 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
           if (s != HOTRG_OK) return s;
         }
         hotrg_status s = HOTRG_OK;
+        GemmSectors sec{};
+        if (p.sect) sec = GemmSectors{tab, x0, xs, x20, xs2, pr.gemm_rows > 0 ? (pr.gemm_rows + 1) / 2 : 0};
         if (!pr.gemm) {
           // tensor-pass probe: no product
         } else if (split) {
@@ -1049,16 +1199,19 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
           g.amax_a = amaxA;
           g.amax_b = amaxB;
           g.per_elem = nt;
+          g.sec = sec;
           g.nprob = nt * ne;
           for (int e = 0; e < ne; ++e) {
             const int w0 = e * nt;
             R* Ce = Cbuf + (int64_t)w0 * Csz;
-            g.p[w0] = GemmProblem{(float*)Ce, (float)un, 1, {w0, 0}, {w0, 0}};
-            if (nt >= 2) g.p[w0 + 1] = GemmProblem{(float*)(Ce + Csz), (float)(0.5 * un), 2, {w0 + 1, w0}, {w0, w0 + 1}};
+            g.p[w0] = GemmProblem{(float*)Ce, (float)un, 1, {w0, 0}, {w0, 0}, {0, 0}, 0};
+            if (nt >= 2)
+              g.p[w0 + 1] = GemmProblem{(float*)(Ce + Csz), (float)(0.5 * un), 2, {w0 + 1, w0}, {w0, w0 + 1}, {1, 0}, 1};
             if (nt >= 3)
-              g.p[w0 + 2] = kstep == 0
-                                ? GemmProblem{(float*)(Ce + 2 * Csz), (float)un, 1, {w0 + 1, 0}, {w0 + 1, 0}}
-                                : GemmProblem{(float*)(Ce + 2 * Csz), (float)(0.5 * un), 2, {w0 + 2, w0}, {w0, w0 + 2}};
+              g.p[w0 + 2] =
+                  kstep == 0
+                      ? GemmProblem{(float*)(Ce + 2 * Csz), (float)un, 1, {w0 + 1, 0}, {w0 + 1, 0}, {1, 1}, 0}
+                      : GemmProblem{(float*)(Ce + 2 * Csz), (float)(0.5 * un), 2, {w0 + 2, w0}, {w0, w0 + 2}, {0, 0}, 0};
           }
           s = gemm_tc(ctx, Abuf, Alob, Bbuf, Blob, nt * ne, Asz, Bsz, p, g, rA, rB, st);
           if (s != HOTRG_OK) return s;
@@ -1073,7 +1226,8 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
                                 Bbuf + (e * esB.op + wb * Bsz * planes) * (int64_t)osz, Asz, Bsz, p.Kp, p.kps, p.P,
                                 rA, rB, (double*)(Cbuf + e * esC.C + out * Csz), rB, alpha, amaxA + e * tw + wa,
                                 amaxB + e * tw + wb,
-                                acc, (int*)(ctx->ws + ctx->L.status), st),
+                                acc, (int*)(ctx->ws + ctx->L.status), st,
+                                OneProduct{sec, e, parity[wa], parity[wa] ^ parity[wb]}),
                  "gemm oz");
               return tm.stop(2.0 * (double)rA * (double)rB * (double)p.K);
             };
@@ -1096,29 +1250,24 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
           R* Cbuf = (R*)(sb + sc.C) + e * esC.C;     // this element's outputs
           auto Ap = [&](int w) { return opnd(Abuf, e * esA.op + w * Asz); };
           auto Bp = [&](int w) { return opnd(Bbuf, e * esB.op + w * Bsz); };
-          // C_T = A(T) B(T)^T
-          s = gemm_simt<R>(ctx, Ap(0), Bp(0), p, Cbuf, rA, rB, 1.0, 0.0, st);
+          // C_out (+)= alpha A(wa) B(wb)^T
+          auto prod = [&](int wa, int wb, int out, double alpha, double beta) {
+            return gemm_simt<R>(ctx, Ap(wa), Bp(wb), p, Cbuf + out * Csz, rA, rB, alpha, beta, st,
+                                OneProduct{sec, e, parity[wa], parity[wa] ^ parity[wb]});
+          };
+          s = prod(0, 0, 0, 1.0, 0.0);                                        // C_T = A(T) B(T)^T
+          if (s == HOTRG_OK && nt >= 2) s = prod(1, 0, 1, 0.5, 0.0);          // C_S = (A(S) B(T)^T + A(T) B(S)^T) / 2
+          if (s == HOTRG_OK && nt >= 2) s = prod(0, 1, 1, 0.5, 1.0);
+          if (nt >= 3 && kstep == 0) {   // M_1 = A(S) B(S)^T: the nearest-neighbour pair inside the first block
+            if (s == HOTRG_OK) s = prod(1, 1, 2, 1.0, 0.0);
+          } else if (nt >= 3) {          // M' = (A(M) B(T)^T + A(T) B(M)^T) / 2
+            if (s == HOTRG_OK) s = prod(2, 0, 2, 0.5, 0.0);
+            if (s == HOTRG_OK) s = prod(0, 2, 2, 0.5, 1.0);
+          }
           if (s != HOTRG_OK) return s;
-          if (nt >= 2) {  // C_S = (A(S) B(T)^T + A(T) B(S)^T) / 2
-            s = gemm_simt<R>(ctx, Ap(1), Bp(0), p, Cbuf + Csz, rA, rB, 0.5, 0.0, st);
-            if (s != HOTRG_OK) return s;
-            s = gemm_simt<R>(ctx, Ap(0), Bp(1), p, Cbuf + Csz, rA, rB, 0.5, 1.0, st);
-            if (s != HOTRG_OK) return s;
-          }
-          if (nt >= 3) {
-            if (kstep == 0) {  // M_1 = A(S) B(S)^T: the nearest-neighbour pair inside the first block
-              s = gemm_simt<R>(ctx, Ap(1), Bp(1), p, Cbuf + 2 * Csz, rA, rB, 1.0, 0.0, st);
-              if (s != HOTRG_OK) return s;
-            } else {           // M' = (A(M) B(T)^T + A(T) B(M)^T) / 2
-              s = gemm_simt<R>(ctx, Ap(2), Bp(0), p, Cbuf + 2 * Csz, rA, rB, 0.5, 0.0, st);
-              if (s != HOTRG_OK) return s;
-              s = gemm_simt<R>(ctx, Ap(0), Bp(2), p, Cbuf + 2 * Csz, rA, rB, 0.5, 1.0, st);
-              if (s != HOTRG_OK) return s;
-            }
-          }
         }
         for (int w = 0; w < nt && pr.ttm; ++w) {
-          s = close_C<R>(ctx, p, Cbuf + w * Csz, Uc, x0, xs, x20, xs2, O3, dst[w], st, esC);
+          s = close_C<R>(ctx, p, Cbuf + w * Csz, Uc, x0, xs, x20, xs2, O3, dst[w], st, esC, tab, parity[w]);
           if (s != HOTRG_OK) return s;
         }
       }
@@ -1225,6 +1374,16 @@ bool choose_slices(const hotrg_ctx* ctx, StepPlan& p) {
   return true;
 }
 
+// Slices of a step of this run: by charge sectors where the tensors conserve the charge and the
+// workspace holds the sector tables too, dense otherwise.
+bool plan_slices(const hotrg_ctx* ctx, StepPlan& p) {
+  p.sect = ctx->sectors;
+  if (choose_slices(ctx, p)) return true;
+  if (!p.sect) return false;
+  p.sect = false;
+  return choose_slices(ctx, p);
+}
+
 // ---------------------------------------------------------------------------- autotuner
 // The plan choices that leave the method's arithmetic unchanged up to rounding are timed on
 // the GPU and the fastest is kept, per device and step shape: the closing direction c (which
@@ -1244,8 +1403,8 @@ std::string tune_key(const hotrg_ctx* ctx, int dir, int dcut) {
   int dev = -1;
   cudaGetDevice(&dev);
   char key[160];
-  snprintf(key, sizeof(key), "dev%d prec%d b%d t%d D%d,%d,%d,%d mu%d cut%d ws%zu", dev, ctx->prec, ctx->batch,
-           ntensors(ctx->impure_active), ctx->dims[0], ctx->dims[1], ctx->dims[2], ctx->dims[3], dir, dcut,
+  snprintf(key, sizeof(key), "dev%d prec%d b%d t%d s%d D%d,%d,%d,%d mu%d cut%d ws%zu", dev, ctx->prec, ctx->batch,
+           ntensors(ctx->impure_active), ctx->sectors ? 1 : 0, ctx->dims[0], ctx->dims[1], ctx->dims[2], ctx->dims[3], dir, dcut,
            ctx->ws_bytes);
   return key;
 }
@@ -1270,7 +1429,7 @@ template <typename R>
 hotrg_status tune_step(hotrg_ctx* ctx, int dir, int dcut, TuneChoice* best_out) {
   cudaStream_t st = ctx->stream;
   StepPlan p0 = make_plan(ctx->dims, dir, dcut, ctx->prec, ctx->batch);
-  if (!choose_slices(ctx, p0)) return HOTRG_EWORKSPACE;
+  if (!plan_slices(ctx, p0)) return HOTRG_EWORKSPACE;
   const Scratch sc0 = scratch_layout(p0, p0.xs, p0.xs2, ctx->prec, ctx->impure_active, ctx->rsize);
   hotrg_status s = isometry_stage<R>(ctx, p0, sc0, ctx->ws + ctx->L.persistent_end, st);
   if (s != HOTRG_OK) return s;
@@ -1299,7 +1458,7 @@ hotrg_status tune_step(hotrg_ctx* ctx, int dir, int dcut, TuneChoice* best_out) 
   for (int c = 0; c < 4 && s == HOTRG_OK; ++c) {
     if (c == dir || c == p0.c) continue;   // the planner's direction last: its operands stay for the GEMM probe
     StepPlan pc = make_plan(ctx->dims, dir, dcut, ctx->prec, ctx->batch, c);
-    if (!choose_slices(ctx, pc)) continue;
+    if (!plan_slices(ctx, pc)) continue;
     Probe pr;
     pr.first_block = true;
     pr.gemm = false;
@@ -1432,6 +1591,7 @@ hotrg_status hotrg_workspace_size(hotrg_ctx* ctx, int nsteps, const int* dirs, c
     int Dm[4] = {ctx->dcut_max, ctx->dcut_max, ctx->dcut_max, ctx->dcut_max};
     StepPlan p = make_plan(Dm, 0, ctx->dcut_max, ctx->prec, ctx->batch);
     p.ne = ne_full;
+    p.sect = true;
     scratch = scratch_layout(p, p.xs, p.xs2, ctx->prec, ctx->impure, ctx->rsize).total;
     cap = std::max(cap, tensor_elems(Dm));
   } else {
@@ -1439,6 +1599,7 @@ hotrg_status hotrg_workspace_size(hotrg_ctx* ctx, int nsteps, const int* dirs, c
       if (dirs[i] < 0 || dirs[i] > 3 || dcuts[i] < 1 || dcuts[i] > ctx->dcut_max) return HOTRG_EINVAL;
       StepPlan p = make_plan(D, dirs[i], dcuts[i], ctx->prec, ctx->batch);
       p.ne = ne_full;
+      p.sect = true;
       scratch = std::max(scratch, scratch_layout(p, p.xs, p.xs2, ctx->prec, ctx->impure, ctx->rsize).total);
       for (int n = 0; n < 4; ++n) {
         D[n] = p.newD[n];
@@ -1464,6 +1625,7 @@ hotrg_status hotrg_set_workspace(hotrg_ctx* ctx, void* dev_ptr, size_t bytes) {
   ctx->drop_graphs();
   jacobi_prepare();
   gemm_prepare();
+  sectors_prepare();
   ctx->ws = (char*)dev_ptr;
   ctx->ws_bytes = bytes;
   ctx->L = L;
@@ -1497,13 +1659,17 @@ hotrg_status hotrg_init_tensor(hotrg_ctx* ctx, const double* beta, const double*
   const double* db = (const double*)(ctx->ws + ctx->L.beta);
   const double* dh = (const double*)(ctx->ws + ctx->L.hfield);
   double* lnz = (double*)(ctx->ws + ctx->L.lnz);
+  // without a field the odd entries of T (and the even ones of S) cancel exactly
+  ctx->sectors = true;
+  for (int b = 0; b < ctx->batch; ++b) ctx->sectors = ctx->sectors && h[b] == 0.0;
+  SectorState* sct = ctx->sectors ? (SectorState*)(ctx->ws + ctx->L.sectors) : nullptr;
   if (f64_store(ctx->prec))
     LK(1, launch_init<double>(db, dh, tensor_ptr<double>(ctx, 0, 0, 0),
-                           ctx->impure ? tensor_ptr<double>(ctx, 1, 0, 0) : nullptr, ctx->L.cap, lnz, ctx->batch, st),
+                           ctx->impure ? tensor_ptr<double>(ctx, 1, 0, 0) : nullptr, ctx->L.cap, lnz, sct, ctx->batch, st),
        "init");
   else
     LK(1, launch_init<float>(db, dh, tensor_ptr<float>(ctx, 0, 0, 0),
-                          ctx->impure ? tensor_ptr<float>(ctx, 1, 0, 0) : nullptr, ctx->L.cap, lnz, ctx->batch, st),
+                          ctx->impure ? tensor_ptr<float>(ctx, 1, 0, 0) : nullptr, ctx->L.cap, lnz, sct, ctx->batch, st),
        "init");
   // the beta/h uploads read host memory that may go away: make them complete now
   CK(cudaStreamSynchronize(st), "init sync");
@@ -1553,6 +1719,7 @@ hotrg_status hotrg_set_tensor(hotrg_ctx* ctx, int b, const int dims[4], const do
   const double lc = log(c);
   CK(cudaMemcpy((double*)(ctx->ws + ctx->L.lnz) + b, &lc, 8, cudaMemcpyHostToDevice), "lnz");
   ctx->impure_active = 0;
+  ctx->sectors = false;
   for (int n = 0; n < 4; ++n) ctx->dims[n] = dims[n];
   ctx->k = 0;
   ctx->sticky = 0;
@@ -1592,7 +1759,7 @@ hotrg_status hotrg_step(hotrg_ctx* ctx, int dir, int dcut) {
     p.gemm_opt = tc.opt;
     p.tuned = hit;
   }
-  if (!choose_slices(ctx, p)) return HOTRG_EWORKSPACE;
+  if (!plan_slices(ctx, p)) return HOTRG_EWORKSPACE;
   hotrg_status s = HOTRG_OK;
   if (!ctx->use_graphs) {
     s = f64_store(ctx->prec) ? do_step<double>(ctx, p) : do_step<float>(ctx, p);
@@ -1602,9 +1769,9 @@ hotrg_status hotrg_step(hotrg_ctx* ctx, int dir, int dcut) {
     // which buffer holds the tensors, whether it is the first step (M_1 = C(S,S)) and the
     // impure tensors in use. ln c / 2^k and the record slot come from the device counter.
     char key[256];
-    snprintf(key, sizeof(key), "%d %d %d %d %d %d %d %d %d %d %d %d %d %d %d", dir, dcut, ctx->dims[0],
+    snprintf(key, sizeof(key), "%d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d", dir, dcut, ctx->dims[0],
              ctx->dims[1], ctx->dims[2], ctx->dims[3], ctx->cur, ctx->k == 0, ctx->impure_active, p.xs, p.xs2,
-             ctx->batch, p.c, p.gemm_opt, p.ne);
+             ctx->batch, p.c, p.gemm_opt, p.ne, ctx->sectors ? 1 : 0, p.sect ? 1 : 0);
     auto it = ctx->graphs.find(key);
     if (it == ctx->graphs.end()) {
       const uint64_t l0 = ctx->launches;
@@ -1866,6 +2033,20 @@ hotrg_status hotrg_split_stats(hotrg_ctx* ctx, hotrg_split_counts* out) {
   for (int e = 0; e < ne; ++e)
     for (int w = 0; w < nbuild; ++w) {
       const int64_t ta = (int64_t)(e * nt + w) * Asz * 2, tb = (int64_t)(e * nt + w) * Bsz * 2;   // bytes
+      if (p.sect) {
+        SectorTab tab = sector_tab(p);
+        tab.base = sb + sc.tab;
+        const int x0 = ca - xs, x20 = ca - xs2, par = w == 1;
+        for (int lo = 0; lo < 2; ++lo) {
+          CK(launch_sector_stats(sb + (lo ? sc.Alo : sc.A) + ta, tab, e, par, x0, xs, xs * per_x, p.K, p.kps,
+                                 cnt + 3 * lo, st),
+             "stats");
+          CK(launch_sector_stats(sb + (lo ? sc.Blo : sc.B) + tb, tab, e, par, x20, xs2, xs2 * per_x, p.K, p.kps,
+                                 cnt + 6 + 3 * lo, st),
+             "stats");
+        }
+        continue;
+      }
       CK(launch_plane_stats(sb + sc.A + ta, p.P * xs * per_x, p.Kp, p.kps, cnt + 0, st), "stats");
       CK(launch_plane_stats(sb + sc.Alo + ta, p.P * xs * per_x, p.Kp, p.kps, cnt + 3, st), "stats");
       CK(launch_plane_stats(sb + sc.B + tb, p.P * xs2 * per_x, p.Kp, p.kps, cnt + 6, st), "stats");

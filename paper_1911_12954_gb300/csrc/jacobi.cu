@@ -394,6 +394,8 @@ __global__ void __launch_bounds__(256) select_kernel(const __grid_constant__ Sel
   jb.U64 += bidx * jobs.sU64;
   jb.Ur = (R*)jb.Ur + bidx * jobs.sUr;
   if (jb.rec_b) jb.rec_b += bidx * jobs.sRec;
+  if (jb.sectors) jb.sectors += bidx;
+  __shared__ int seen[kMaxLeg];      // charges met in each kept column (bit 0: even, bit 1: odd)
   __shared__ double red[8];
   __shared__ int side;
   const int n = jb.n, chi = jb.chi, tid = threadIdx.x;
@@ -436,6 +438,27 @@ __global__ void __launch_bounds__(256) select_kernel(const __grid_constant__ Sel
   }
   R* ur = (R*)jb.Ur;
   for (int e = tid; e < n * chi; e += blockDim.x) ur[e] = (R)jb.U64[e];
+  if (jb.sectors == nullptr) return;
+  // charge of a kept column = charge of the fused indices it is made of; a column that mixes both
+  // drops the element's sectors
+  for (int i = tid; i < chi; i += blockDim.x) seen[i] = 0;
+  __syncthreads();
+  const uint32_t m = jb.sectors->charge[jb.cur][jb.nu];
+  for (int e = tid; e < n * chi; e += blockDim.x)
+    if (jb.U64[e] != 0.0) {
+      const int r = e / chi;
+      atomicOr(&seen[e % chi], 1 << (((m >> (r / jb.Dn)) ^ (m >> (r % jb.Dn))) & 1));
+    }
+  __syncthreads();
+  if (tid == 0) {
+    uint32_t q = 0;
+    for (int i = 0; i < chi; ++i) {
+      if (seen[i] == 3) jb.sectors->dropped = 1;
+      if (seen[i] == 2) q |= 1u << i;
+    }
+    jb.sectors->charge[1 - jb.cur][jb.nu] = q;
+    if (blockIdx.x - bidx * njobs == 0) jb.sectors->charge[1 - jb.cur][jb.mu] = jb.sectors->charge[jb.cur][jb.mu];
+  }
 }
 
 template <typename R>

@@ -18,53 +18,9 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "ttm_device.cuh"
 
 namespace hotrg {
-
-__device__ __forceinline__ float tf32_round(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
-
-// Exact 8-bit slices of x (|x| < 1, FP64): r <- 256 r, v = rint(r), r <- r - v, five times;
-// every step is exact in FP64 and every v an integer fp16 holds exactly (|v| <= 256).
-__device__ __forceinline__ void oz_store(__half* out, int64_t plane, int64_t o, double x) {
-  double r = x;
-#pragma unroll
-  for (int i = 0; i < kOzSlices; ++i) {
-    r *= 256.0;
-    const double v = rint(r);
-    out[o + i * plane] = __float2half_rn((float)v);
-    r -= v;
-  }
-}
-
-// Power-of-two scale of a split pass: from the operand's largest magnitude (a max pass of the
-// same contraction wrote it to amax) or, without one, the fixed 2^14 of the fp16 planes.
-template <int MODE>
-__device__ __forceinline__ double split_scale(const unsigned* amax) {
-  if (MODE == kTTMSplitF16) return amax ? ldexp(1.0, split_exponent(*amax, kF16Top)) : (double)kF16Scale;
-  if (MODE == kTTMSplitOz) return ldexp(1.0, amax ? split_exponent(*amax, kOzTop) : kOzTop);
-  return 1.0;
-}
-
-// Largest magnitude seen by the threads of a block, times mul, merged into *amax (bits of a
-// non-negative float, rounded up, so that the recorded value bounds mul times every output).
-__device__ __forceinline__ void merge_max(unsigned* amax, double m, float mul) {
-  float f = __double2float_ru(m * (double)mul);
-  for (int off = 16; off > 0; off >>= 1) f = fmaxf(f, __shfl_down_sync(0xffffffffu, f, off));
-  if ((threadIdx.x & 31) == 0 && f > 0.f && amax) atomicMax(amax, __float_as_uint(f));
-}
-
-// Output pointer of batch element e: the split modes write fp16 planes, whose strides count
-// fp16 values; the others count elements of the output type.
-template <typename TO, int MODE>
-__device__ __forceinline__ TO* elem_out(TO* p, int64_t off) {
-  if (!p) return p;
-  if (MODE == kTTMSplitF16 || MODE == kTTMSplitOz) return (TO*)((__half*)p + off);
-  return p + off;
-}
 
 template <typename TI, typename TU, typename TO, int MODE>
 __global__ void __launch_bounds__(256) ttm_kernel(const TI* __restrict__ in, const TU* __restrict__ U,
@@ -684,8 +640,14 @@ template cudaError_t launch_ttm<float, double, double>(const float*, const doubl
 // normalised tensors and ln c_0 = ln ||T||_F.
 template <typename R>
 __global__ void __launch_bounds__(256) init_kernel(const double* __restrict__ beta, const double* __restrict__ h,
-                                                   R* T, R* S, int64_t slot, double* lnz_acc) {
+                                                   R* T, R* S, int64_t slot, double* lnz_acc,
+                                                   SectorState* sectors) {
   const int b = blockIdx.x;
+  if (sectors && threadIdx.x == 0) {   // index i of a bond counts the bond's tanh factors: charge i
+    SectorState s = {};
+    for (int n = 0; n < 4; ++n) s.charge[0][n] = s.charge[1][n] = 2u;
+    sectors[b] = s;
+  }
   const double be = beta[b], hb = h[b];
   const double ch = sqrt(cosh(be)), sh = sqrt(sinh(be));
   const int i = threadIdx.x;
@@ -716,14 +678,14 @@ __global__ void __launch_bounds__(256) init_kernel(const double* __restrict__ be
 
 template <typename R>
 cudaError_t launch_init(const double* beta, const double* h, R* T, R* S, int64_t slot, double* lnz_acc,
-                        int batch, cudaStream_t st) {
-  init_kernel<R><<<batch, 256, 0, st>>>(beta, h, T, S, slot, lnz_acc);
+                        SectorState* sectors, int batch, cudaStream_t st) {
+  init_kernel<R><<<batch, 256, 0, st>>>(beta, h, T, S, slot, lnz_acc, sectors);
   return cudaGetLastError();
 }
 template cudaError_t launch_init<double>(const double*, const double*, double*, double*, int64_t, double*,
-                                         int, cudaStream_t);
-template cudaError_t launch_init<float>(const double*, const double*, float*, float*, int64_t, double*, int,
-                                        cudaStream_t);
+                                         SectorState*, int, cudaStream_t);
+template cudaError_t launch_init<float>(const double*, const double*, float*, float*, int64_t, double*, SectorState*,
+                                        int, cudaStream_t);
 
 // ---------------------------------------------------------------------------- norm
 // Pass 1: each block writes the FP64 sum of squares of its grid-stride share.
@@ -817,6 +779,46 @@ cudaError_t launch_plane_stats(const void* plane, int64_t nrows, int64_t Kp, int
   int64_t blocks = (nrows * Kp + 255) / 256;
   if (blocks > 152 * 8) blocks = 152 * 8;
   plane_stats_kernel<<<(unsigned)blocks, 256, 0, st>>>((const __half*)plane, nrows, Kp, kps, out);
+  return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256) sector_stats_kernel(const __half* __restrict__ pl, SectorTab tab, int elem,
+                                                           int parity, int x0, int nx, int64_t rows, int64_t K,
+                                                           int64_t kps, unsigned long long* out) {
+  const SectorPlan& p = *tab.at(elem).plan;
+  const int64_t r0 = p.row[0][x0 + nx] - p.row[0][x0];        // rows of charge 0: first in the plane
+  const int64_t nrow = r0 + p.row[1][x0 + nx] - p.row[1][x0];
+  unsigned long long nz = 0, ns = 0;
+  unsigned mx = 0;
+  const int64_t n = nrow * K;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / K, k = i - r * K;
+    unsigned a = 0u;
+    if (k < p.K[(r < r0 ? 0 : 1) ^ parity])
+      a = __half_as_ushort(pl[(k / kps * rows + r) * kps + k % kps]) & 0x7fffu;
+    nz += a == 0u;
+    ns += (a != 0u && a < 0x0400u);
+    mx = max(mx, a);
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    nz += __shfl_down_sync(0xffffffffu, nz, off);
+    ns += __shfl_down_sync(0xffffffffu, ns, off);
+    mx = max(mx, __shfl_down_sync(0xffffffffu, mx, off));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&out[0], nz);
+    atomicAdd(&out[1], ns);
+    atomicMax(&out[2], (unsigned long long)mx);
+  }
+}
+
+cudaError_t launch_sector_stats(const void* plane, const SectorTab& tab, int elem, int parity, int x0, int nx,
+                                int64_t rows, int64_t K, int64_t kps, unsigned long long* out, cudaStream_t st) {
+  if (rows <= 0 || K <= 0) return cudaSuccess;
+  int64_t blocks = (rows * K + 255) / 256;
+  if (blocks > 152 * 8) blocks = 152 * 8;
+  sector_stats_kernel<<<(unsigned)blocks, 256, 0, st>>>((const __half*)plane, tab, elem, parity, x0, nx, rows, K, kps,
+                                                        out);
   return cudaGetLastError();
 }
 
