@@ -90,6 +90,8 @@ struct GramJob {
   int64_t rst[8];           // summed leg strides
   int64_t K;                // product of rdims
   double* partial;          // [nchunks][R][R]
+  int dir1, dir2, rdir[8];  // directions of the row legs and the summed legs
+  uint32_t rmagic[8];       // reciprocals of the summed leg sizes (filled in by launch_gram)
 };
 
 // One symmetric eigenproblem for the Jacobi kernel.
@@ -210,6 +212,8 @@ constexpr int kMaxSelectJobs = 3;
 struct GramPack {
   GramJob j[kMaxGramJobs];
   int batch = 1;
+  const struct SectorState* sectors = nullptr;   // charges of the tensors (nullptr: none), one per element
+  int cur = 0;              // their buffer
   int64_t sT = 0;           // tensor (storage elements)
   int64_t sPart = 0;        // split-K partials (doubles)
 };

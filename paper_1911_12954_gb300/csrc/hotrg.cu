@@ -338,8 +338,9 @@ StepPlan make_plan(const int D[4], int mu, int dcut, int prec, int batch = 1, in
     }
   }
   const int64_t Kg = p.E / p.Rmax;
-  int64_t nc = (Kg + 511) / 512;
-  if (nc > 256) nc = 256;
+  // split-K chunks of the half-Grams: two CTAs per SM in all (a chunk's set-up, decoding and reduction
+  // cost a few microseconds), of at least 64 summed indices
+  int64_t nc = std::min(2 * 150 * 2 / (12 * (int64_t)batch), (Kg + 63) / 64);
   if (nc < 1) nc = 1;
   // keep the split-K partials of all batch elements under 256 MB
   const int64_t per = (int64_t)batch * kMaxGramJobs * p.Rmax * p.Rmax * 8;
@@ -924,6 +925,8 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
         const int kleg = half == 0 ? 2 * mu + 1 : 2 * mu;
         j.D1 = p.D[n];
         j.D2 = p.D[mu];
+        j.dir1 = n;
+        j.dir2 = mu;
         j.s1 = ts[leg];
         j.s2 = ts[kleg];
         j.nrest = 0;
@@ -932,6 +935,7 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
           if (l == leg || l == kleg) continue;
           j.rdims[j.nrest] = p.D[l / 2];
           j.rst[j.nrest] = ts[l];
+          j.rdir[j.nrest] = l / 2;
           j.K *= p.D[l / 2];
           ++j.nrest;
         }
@@ -941,6 +945,8 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
     }
   }
   gp.batch = nb;
+  gp.sectors = ctx->sectors ? (const SectorState*)(ctx->ws + ctx->L.sectors) : nullptr;
+  gp.cur = ctx->cur;
   gp.sT = ctx->L.cap;                                   // tensor slots of consecutive elements
   gp.sPart = (int64_t)kMaxGramJobs * p.nchunks * RR;
   LK(1, launch_gram<R>(gp, nj, p.Rmax, p.nchunks, st), "gram");

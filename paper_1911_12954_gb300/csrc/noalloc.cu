@@ -37,7 +37,7 @@ namespace hotrg {
 constexpr int kNoAllocMaxLeg = 8;
 constexpr int kNoAllocR = kNoAllocMaxLeg * kNoAllocMaxLeg;   // half-Gram side
 constexpr int kNoAllocN = kNoAllocMaxLeg * kNoAllocMaxLeg;   // Gram side
-constexpr int kNoAllocChunks = 32;                           // split-K chunks per half-Gram
+constexpr int kNoAllocChunks = 38;                           // split-K chunks per half-Gram: 4 x 38 CTAs, one per SM
 constexpr size_t kNoAllocBytes = 8u << 20;                   // 8 MiB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
@@ -117,7 +117,7 @@ extern "C" hotrg_status hotrg_isometry_noalloc(const double* T_dev, const int di
     s *= dims[leg / 2];
   }
   const int64_t E = s;
-  int64_t nch = (E / R + 511) / 512;
+  int64_t nch = (E / R + 127) / 128;
   if (nch > kNoAllocChunks) nch = kNoAllocChunks;
   if (nch < 1) nch = 1;
 
