@@ -13,7 +13,16 @@ constexpr int kMaxLeg = 16;       // largest bond dimension (dcut_max)
 constexpr int kMaxGramN = kMaxLeg * kMaxLeg;  // largest Gram matrix side (D_nu^2)
 constexpr int kMaxSteps = 64;     // steps recorded per batch element
 constexpr int kJacobiMaxSweeps = 60;
-constexpr int kJacobiSmemN = 96;  // the eigensolver keeps A and V in shared memory up to this n (no work buffer)
+constexpr int kJacobiSmemN = 208;    // the eigensolver keeps A (its upper triangle) in shared memory up to this n
+constexpr int kJacobiLogSweeps = 10; // sweeps of rotations the eigensolver logs before it folds them into V
+constexpr int64_t packed_doubles(int n) { return ((int64_t)n * (n + 1) / 2 + 1) / 2 * 2; }   // upper triangle, even
+// Doubles of global work space per matrix (EigJob::work): eigenvector columns, V (used when the log
+// overflows), the upper triangle of matrices that do not fit shared memory, the log of rotations (c, s): a
+// sweep has at most n rounds of at most n pair slots.
+constexpr int64_t jacobi_work_doubles(int n) {
+  return 2 * (int64_t)n * n + (n > kJacobiSmemN ? packed_doubles(n) : 0) +
+         2 * (int64_t)kJacobiLogSweeps * n * n;
+}
 
 // Device-side status words (in the caller's workspace), read back at sync points.
 enum StatusWord { kStNoConv = 0, kStNonFinite = 1, kStTimeout = 2, kStWords = 4 };
@@ -97,7 +106,7 @@ struct GramJob {
 // One symmetric eigenproblem for the Jacobi kernel.
 struct EigJob {
   const double* G;          // n x n, row-major, symmetric
-  double* work;             // 2 n^2 doubles of global scratch (used when n is large)
+  double* work;             // jacobi_work_doubles(n) doubles of global scratch, 16-byte aligned
   double* lam;              // n eigenvalues, descending
   double* U;                // n x chi, first chi eigenvectors in canonical gauge
   double* eps;              // sum of the discarded eigenvalues (index >= chi)

@@ -402,17 +402,22 @@ Scratch scratch_layout(const StepPlan& p, int xs, int xs2, int prec, int impure,
   const int nt = ntensors(impure);
   // isometry stage: one copy per batch element (all elements run it together)
   const size_t nb = (size_t)p.batch;
-  s.gpart = take(nb * kMaxGramJobs * p.nchunks * p.Rmax * p.Rmax * 8);
   s.npart = take(nb * kNormPartials * 8);
   s.gA = take(nb * kMaxGramJobs * p.Rmax * p.Rmax * 8);
   s.G = take(nb * 6 * p.nmax * p.nmax * 8);
-  s.jwork = take(p.nmax > kJacobiSmemN ? nb * 6 * 2 * p.nmax * p.nmax * 8 : 0);
   s.lam = take(nb * 6 * p.nmax * 8);
   s.eps = take(nb * 6 * 8);
   s.degen = take(nb * 6 * 4);
   s.Uside = take(nb * 6 * p.nmax * kMaxLeg * 8);
   const int64_t rowsA = (int64_t)xs * p.chi[p.b] * p.D[p.c] * p.D[p.c] * p.D[p.mu];
   const int64_t rowsB = (int64_t)xs2 * p.chi[p.b] * p.D[p.c] * p.D[p.c] * p.D[p.mu];
+  // the Gram partials and the eigensolver's work are done with before the contraction's buffers are
+  // written: they share that space
+  const size_t shared = off;
+  s.gpart = take(nb * kMaxGramJobs * p.nchunks * p.Rmax * p.Rmax * 8);
+  s.jwork = take(nb * 6 * (size_t)jacobi_work_doubles(p.nmax) * 8);
+  const size_t iso_end = off;
+  off = shared;
   const bool split = tc_mode(prec);
   const size_t os = operand_size(prec) * (prec == HOTRG_FP64OZ ? kOzSlices : 1);   // the slices of one operand
   // contraction: one copy per element of a group (p.ne elements contracted together)
@@ -428,7 +433,7 @@ Scratch scratch_layout(const StepPlan& p, int xs, int xs2, int prec, int impure,
   s.tab = p.sect ? take(ne * sector_tab(p).stride) : 0;
   s.amax = take(2 * ne * nt * sizeof(unsigned));   // A side, then B side: per element (and tensor)
   s.stats = take(4 * 3 * sizeof(unsigned long long));   // hotrg_split_stats counters
-  s.total = off;
+  s.total = std::max(off, iso_end);
   return s;
 }
 
@@ -962,7 +967,7 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
   int* degen = (int*)(sb + sc.degen);
   double* Uside = (double*)(sb + sc.Uside);
   double* jwork = (double*)(sb + sc.jwork);
-  const bool big = p.nmax > kJacobiSmemN;
+  const int64_t jw = jacobi_work_doubles(p.nmax);
   int nmax = 0;
   for (int i = 0; i < 3; ++i) {
     for (int side = 0; side < 2; ++side) {
@@ -971,7 +976,7 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
       j.n = p.D[dirs[i]] * p.D[dirs[i]];
       j.chi = p.chi[dirs[i]];
       j.G = G + (int64_t)e * nn;
-      j.work = big ? jwork + (int64_t)e * 2 * nn : nullptr;
+      j.work = jwork + e * jw;
       j.lam = lam + (int64_t)e * p.nmax;
       j.eps = eps + e;
       j.degenerate = degen + e;
@@ -981,7 +986,7 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
   }
   ep.batch = nb;
   ep.sG = 6 * nn;
-  ep.sWork = big ? 6 * 2 * nn : 0;
+  ep.sWork = 6 * jw;
   ep.sLam = 6 * (int64_t)p.nmax;
   ep.sU = 6 * (int64_t)p.nmax * kMaxLeg;
   ep.sEps = 6;

@@ -51,7 +51,7 @@ constexpr size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Offsets inside the array (bytes).
 struct NoAllocLayout {
-  size_t status, part, half, G, lam, eps, degen, Ucand, recs, U64r, total;
+  size_t status, part, half, G, jwork, lam, eps, degen, Ucand, recs, U64r, total;
 };
 
 constexpr NoAllocLayout layout() {
@@ -61,6 +61,7 @@ constexpr NoAllocLayout layout() {
   L.part = o;    o = up256(o + (size_t)4 * kNoAllocChunks * kNoAllocR * kNoAllocR * sizeof(double));
   L.half = o;    o = up256(o + (size_t)4 * kNoAllocR * kNoAllocR * sizeof(double));
   L.G = o;       o = up256(o + (size_t)2 * kNoAllocN * kNoAllocN * sizeof(double));
+  L.jwork = o;   o = up256(o + (size_t)2 * jacobi_work_doubles(kNoAllocN) * sizeof(double));
   L.lam = o;     o = up256(o + (size_t)2 * kNoAllocN * sizeof(double));
   L.eps = o;     o = up256(o + 2 * sizeof(double));
   L.degen = o;   o = up256(o + 2 * sizeof(int));
@@ -167,7 +168,7 @@ extern "C" hotrg_status hotrg_isometry_noalloc(const double* T_dev, const int di
     j.n = n;
     j.chi = chi;
     j.G = G + (int64_t)side * kNoAllocN * kNoAllocN;
-    j.work = nullptr;  // n <= 64: the eigensolver keeps A and V in shared memory
+    j.work = (double*)(base + L.jwork) + side * jacobi_work_doubles(kNoAllocN);
     j.lam = (double*)(base + L.lam) + side * kNoAllocN;
     j.eps = (double*)(base + L.eps) + side;
     j.degenerate = (int*)(base + L.degen) + side;
