@@ -125,14 +125,15 @@ struct SectorState {          // per batch element, persistent
 struct SectorPlan {           // per batch element of a group and step
   int row[2][kMaxLeg + 1];    // operand rows of charge q with new a index < x
   int grp[2][kMaxLeg + 1];    // row groups (X, Y, c', mu) of charge q with new a index < x
-  int K[2];                   // summed indices (a2, b2, a1', b1', k) of charge q
+  int K[2];                   // summed indices (b2, b1', a2, a1', k) of charge q, fillers included
+  int n3[2];                  // rests (a2, a1', k) of charge q, made even by a filler
   uint32_t na, nb, nc;        // charges of the new a, b, c legs
   uint32_t mb, mc, mm;        // of the old b, c legs and of mu
 };
 struct SectorTables {
   uint32_t* row;              // operand row (X, Y, c, c', mu): rank within its charge, charge in bit 31
-  uint2* kA;                  // summed indices, charge 0 first: offset in A's first pass and leg b2
-  uint2* kB;                  // the same for B: offset and leg b1'
+  uint32_t* kA;               // rests (a2, a1', k) of the summed index, charge 0 first, each charge's list filled up
+  uint32_t* kB;               // to an even length (~0): offsets in A's and in B's first pass
   uint32_t* grank;            // row group: rank, charge in bit 31
   uint32_t* grp;              // row groups, charge 0 first
   SectorPlan* plan;
@@ -142,7 +143,7 @@ struct SectorTab {            // the tables of element e start e * stride bytes 
   int64_t stride, o_row, o_kA, o_kB, o_grank, o_grp, o_plan;
   __host__ __device__ SectorTables at(int e) const {
     char* p = base + e * stride;
-    return SectorTables{(uint32_t*)(p + o_row),   (uint2*)(p + o_kA),     (uint2*)(p + o_kB),
+    return SectorTables{(uint32_t*)(p + o_row),   (uint32_t*)(p + o_kA),  (uint32_t*)(p + o_kB),
                         (uint32_t*)(p + o_grank), (uint32_t*)(p + o_grp), (SectorPlan*)(p + o_plan)};
   }
 };
@@ -152,14 +153,13 @@ struct SectorArgs {           // sector_tables_kernel
   int cur;                    // buffer of the tensors before the step
   int a, b, c, mu;            // directions
   int Da, Db, Dc, Dm, ca, cb;
-  uint32_t kA[5], kB[5];      // strides of the summed legs in the first passes' outputs
 };
 struct SectorOperand {        // second half-contraction pass of one tensor
   SectorTab tab;
   int sideB, parity;          // operand side, the tensor's own parity
   int x0, xs, cb, Db, Dc, Dm;
   int nouter;                 // xs Dc Dc Dm
-  int64_t in_x, in_j, in_c0, in_c1, in_m;   // strides of the first pass's output
+  int64_t in_x, in_j, in_c0, in_c1, in_m, in_seg;   // strides of the first pass's output (in_seg: b1' of A, b2 of B)
   int u_j, u_r;               // U strides of the contracted and the new leg (the column has stride 1)
   int64_t rows, kps;          // panel geometry of the operand
   int P, kalign;              // panels; summed indices are zero filled up to a multiple of kalign

@@ -359,6 +359,15 @@ StepPlan make_plan(const int D[4], int mu, int dcut, int prec, int batch = 1, in
   return p;
 }
 
+// A plan that contracts by charge sectors. Its packed summed indices come in D_b^2 runs (b2, b1') of even length:
+// panels take one more alignment unit where the fillers might not fit (all indices of one charge, odd runs).
+void use_sectors(StepPlan& p, int prec) {
+  p.sect = true;
+  const int64_t run = (int64_t)p.D[p.a] * p.D[p.a] * p.D[p.mu], most = (int64_t)p.D[p.b] * p.D[p.b] * ((run + 2) / 2 * 2);
+  const int64_t al = panel_mode(prec) ? 128 / (int64_t)operand_size(prec) : 4;
+  while (p.P * p.kps < most) p.kps += al;
+}
+
 int ntensors(int impure) { return (impure & HOTRG_IMPURE_SIGMASIGMA) ? 3 : ((impure & HOTRG_IMPURE_SIGMA) ? 2 : 1); }
 
 // Scratch bytes of one step with slice sizes xs (new X) and xs2 (new X').
@@ -383,8 +392,9 @@ SectorTab sector_tab(const StepPlan& p) {
   const int64_t groups = p.rowsA_full / p.D[p.c];
   t.o_plan = take(sizeof(SectorPlan));
   t.o_row = take(p.rowsA_full * sizeof(uint32_t));
-  t.o_kA = take(p.K * sizeof(uint2));
-  t.o_kB = take(p.K * sizeof(uint2));
+  const int64_t rests = (int64_t)p.D[p.a] * p.D[p.a] * p.D[p.mu] + 2;
+  t.o_kA = take(rests * sizeof(uint32_t));
+  t.o_kB = take(rests * sizeof(uint32_t));
   t.o_grank = take(groups * sizeof(uint32_t));
   t.o_grp = take(groups * sizeof(uint32_t));
   t.stride = (int64_t)off;
@@ -575,6 +585,7 @@ hotrg_status sector_operand(hotrg_ctx* ctx, const StepPlan& p, int side, const R
   a.in_c0 = os[2];
   a.in_c1 = os[3];
   a.in_m = os[4];
+  a.in_seg = side == 0 ? os[7] : os[6];   // b1' of A's (a2, a1', b1', k), b2 of B's (a2, b2, a1', k)
   a.u_j = side == 0 ? Db * cb : cb;
   a.u_r = side == 0 ? cb : Db * cb;
   a.rows = (int64_t)xs * cb * Dc * Dc * Dm;
@@ -1133,15 +1144,6 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
       a.Dm = p.D[mu];
       a.ca = ca;
       a.cb = p.chi[p.b];
-      // first passes' summed legs, innermost last: A (a2, a1', b1', k), B (a2, b2, a1', k)
-      const uint32_t Da = a.Da, Db = a.Db, Dm = a.Dm;
-      a.kA[4] = a.kB[4] = 1;
-      a.kA[3] = Dm;
-      a.kA[2] = Db * Dm;
-      a.kA[0] = Da * Db * Dm;
-      a.kB[2] = Dm;
-      a.kB[1] = Da * Dm;
-      a.kB[0] = Db * Da * Dm;
       LK(1, launch_sector_tables(a, ne, st), "sector tables");
     }
     const int parity[3] = {0, 1, 0};   // T, S (one sigma: odd), M (two)
@@ -1388,10 +1390,14 @@ bool choose_slices(const hotrg_ctx* ctx, StepPlan& p) {
 // Slices of a step of this run: by charge sectors where the tensors conserve the charge and the
 // workspace holds the sector tables too, dense otherwise.
 bool plan_slices(const hotrg_ctx* ctx, StepPlan& p) {
-  p.sect = ctx->sectors;
-  if (choose_slices(ctx, p)) return true;
-  if (!p.sect) return false;
-  p.sect = false;
+  if (ctx->sectors) {
+    StepPlan s = p;
+    use_sectors(s, ctx->prec);
+    if (choose_slices(ctx, s)) {
+      p = s;
+      return true;
+    }
+  }
   return choose_slices(ctx, p);
 }
 
@@ -1602,7 +1608,7 @@ hotrg_status hotrg_workspace_size(hotrg_ctx* ctx, int nsteps, const int* dirs, c
     int Dm[4] = {ctx->dcut_max, ctx->dcut_max, ctx->dcut_max, ctx->dcut_max};
     StepPlan p = make_plan(Dm, 0, ctx->dcut_max, ctx->prec, ctx->batch);
     p.ne = ne_full;
-    p.sect = true;
+    use_sectors(p, ctx->prec);
     scratch = scratch_layout(p, p.xs, p.xs2, ctx->prec, ctx->impure, ctx->rsize).total;
     cap = std::max(cap, tensor_elems(Dm));
   } else {
@@ -1610,7 +1616,7 @@ hotrg_status hotrg_workspace_size(hotrg_ctx* ctx, int nsteps, const int* dirs, c
       if (dirs[i] < 0 || dirs[i] > 3 || dcuts[i] < 1 || dcuts[i] > ctx->dcut_max) return HOTRG_EINVAL;
       StepPlan p = make_plan(D, dirs[i], dcuts[i], ctx->prec, ctx->batch);
       p.ne = ne_full;
-      p.sect = true;
+      use_sectors(p, ctx->prec);
       scratch = std::max(scratch, scratch_layout(p, p.xs, p.xs2, ctx->prec, ctx->impure, ctx->rsize).total);
       for (int n = 0; n < 4; ++n) {
         D[n] = p.newD[n];

@@ -21,6 +21,8 @@
 //
 // Sums run over the nonzero terms in the order of the dense passes, so operands, C entries
 // given the same k order, and closed tensors are bit-identical to the dense passes'.
+#include <type_traits>
+
 #include "common.cuh"
 #include "ttm_device.cuh"
 
@@ -87,31 +89,30 @@ __global__ void __launch_bounds__(256) sector_tables_kernel(SectorArgs a) {
   const uint32_t na = qn[a.a] & keep, nb = qn[a.b] & keep, nc = qn[a.c] & keep;
   const int rd[5] = {a.ca, a.cb, a.Dc, a.Dc, a.Dm};
   const uint32_t rm[5] = {na, nb, mc, mc, mm};
-  const int kd[5] = {a.Da, a.Db, a.Da, a.Db, a.Dm};
-  const uint32_t km[5] = {ma, mb, ma, mb, mm};
   const int gd[4] = {a.ca, a.cb, a.Dc, a.Dm};
   const uint32_t gm[4] = {na, nb, mc, mm};
-  const int rows = a.ca * a.cb * a.Dc * a.Dc * a.Dm, K = a.Da * a.Da * a.Db * a.Db * a.Dm;
+  const int sd[3] = {a.Da, a.Da, a.Dm};
+  const uint32_t sm[3] = {ma, ma, mm};
+  const int rows = a.ca * a.cb * a.Dc * a.Dc * a.Dm, rests = a.Da * a.Da * a.Dm;
   const int groups = a.ca * a.cb * a.Dc * a.Dm;
   SectorTables t = a.tab.at(e);
-  const int K0 = even_count(kd, km, 0), G0 = even_count(gd, gm, 0);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < rows + K + groups; i += gridDim.x * blockDim.x) {
+  const int S0 = even_count(sd, sm, 0), G0 = even_count(gd, gm, 0);
+  const int n0 = (S0 + 1) & ~1, n1 = (rests - S0 + 1) & ~1;   // runs of even length
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < rows + rests + groups; i += gridDim.x * blockDim.x) {
     if (i < rows) {
       int idx[5];
       decode(rd, (uint32_t)i, idx);
       t.row[i] = sector_rank(rd, rm, idx);
-    } else if (i < rows + K) {
-      int idx[5];
-      decode(kd, (uint32_t)(i - rows), idx);
-      const uint32_t r = sector_rank(kd, km, idx);
-      const int pos = (int)(r & 0x7fffffffu) + ((r >> 31) ? K0 : 0);
-      // offsets inside one (X, contracted leg, c, c', mu) block of the first pass's output
-      const uint32_t oa = (uint32_t)(idx[0] * a.kA[0] + idx[2] * a.kA[2] + idx[3] * a.kA[3] + idx[4] * a.kA[4]);
-      const uint32_t ob = (uint32_t)(idx[0] * a.kB[0] + idx[1] * a.kB[1] + idx[2] * a.kB[2] + idx[4] * a.kB[4]);
-      t.kA[pos] = make_uint2(oa, (uint32_t)idx[1]);
-      t.kB[pos] = make_uint2(ob, (uint32_t)idx[3]);
+    } else if (i < rows + rests) {
+      // rest (a2, a1', k) of the summed index: offsets in A's (a2, a1', b1', k) and B's (a2, b2, a1', k)
+      int idx[3];
+      decode(sd, (uint32_t)(i - rows), idx);
+      const uint32_t r = sector_rank(sd, sm, idx);
+      const int pos = (int)(r & 0x7fffffffu) + ((r >> 31) ? n0 : 0);
+      t.kA[pos] = (uint32_t)((idx[0] * a.Da + idx[1]) * a.Db * a.Dm + idx[2]);
+      t.kB[pos] = (uint32_t)((idx[0] * a.Db * a.Da + idx[1]) * a.Dm + idx[2]);
     } else {
-      const int g = i - rows - K;
+      const int g = i - rows - rests;
       int idx[4];
       decode(gd, (uint32_t)g, idx);
       const uint32_t r = sector_rank(gd, gm, idx);
@@ -131,8 +132,13 @@ __global__ void __launch_bounds__(256) sector_tables_kernel(SectorArgs a) {
       p.grp[0][x + 1] = p.grp[0][x] + (q ? g1 : g0);
       p.grp[1][x + 1] = p.grp[1][x] + (q ? g0 : g1);
     }
-    p.K[0] = K0;
-    p.K[1] = K - K0;
+    if (S0 & 1) t.kA[S0] = t.kB[S0] = ~0u;                  // fillers
+    if ((rests - S0) & 1) t.kA[n0 + n1 - 1] = t.kB[n0 + n1 - 1] = ~0u;
+    p.n3[0] = n0;
+    p.n3[1] = n1;
+    const int b1 = odd_below(mb, a.Db), b0 = a.Db - b1;
+    p.K[0] = (b0 * b0 + b1 * b1) * n0 + 2 * b0 * b1 * n1;
+    p.K[1] = (b0 * b0 + b1 * b1) * n1 + 2 * b0 * b1 * n0;
     p.na = na;
     p.nb = nb;
     p.nc = nc;
@@ -147,8 +153,7 @@ __global__ void __launch_bounds__(256) sector_tables_kernel(SectorArgs a) {
 constexpr int kSectorSmem = 96 * 1024;
 
 cudaError_t launch_sector_tables(const SectorArgs& a, int ne, cudaStream_t st) {
-  const int64_t n = (int64_t)a.ca * a.cb * a.Dc * a.Dc * a.Dm + (int64_t)a.Da * a.Da * a.Db * a.Db * a.Dm +
-                    (int64_t)a.ca * a.cb * a.Dc * a.Dm;
+  const int64_t n = (int64_t)a.ca * a.cb * a.Dc * a.Dm * (a.Dc + 1) + (int64_t)a.Da * a.Da * a.Dm;
   int64_t blocks = (n + 255) / 256;
   if (blocks > 152 * 8) blocks = 152 * 8;
   sector_tables_kernel<<<dim3((unsigned)blocks, ne), 256, 0, st>>>(a);
@@ -157,18 +162,20 @@ cudaError_t launch_sector_tables(const SectorArgs& a, int ne, cudaStream_t st) {
 
 // ---------------------------------------------------------------------------- operands
 // Second half-contraction pass: operand[row(X, Y, c, c', mu), k] = sum_j U[j, r, Y] O1[X, j, c, c', mu, rest(k)]
-// with k = (r, rest) (r: the new leg b2 of A, b1' of B; j: the contracted leg). A block takes one
-// (X, c, c', mu) and one charge Q of k; its threads walk the packed summed indices two at a time, so
-// stores of a warp are contiguous, and each thread sums only the j whose charge fits. The Y of one
-// charge (the only nonzero rows) are produced four at a time.
+// with j the contracted leg and the summed index k in the order (b2, b1', rest), rest = (a2, a1', k): the new leg
+// r is b2 for A and b1' for B, the other of the two is the segment. For fixed (b2, b1') the rests of one charge
+// are neighbours in the packed operand (a run, of even length: a filler entry where the count is odd). A block
+// takes one (X, c, c', mu); a warp takes 64 rests of one segment and charge, two per lane: their O1 entries are
+// nonzero for the j of one charge only, each is loaded once and serves every r and Y, the coefficients are the
+// same for the whole warp (broadcast reads from shared memory), and the stores are pairs in runs of 64.
+// The writes bound it: at D_cut = 8 one pass writes 2.1 GB and reads 0.5 GB (0.4 ms at the copy rate).
 template <int MODE, typename R>
 __device__ __forceinline__ void sector_store2(R* out, R* out_lo, int64_t o, R v0, R v1) {
   if constexpr (MODE == kTTMSplitF16) {
-    const float f0 = (float)v0, f1 = (float)v1;
-    const __half h0 = __float2half_rn(f0), h1 = __float2half_rn(f1);
-    *(__half2*)((__half*)out + o) = __halves2half2(h0, h1);
-    *(__half2*)((__half*)out_lo + o) =
-        __halves2half2(__float2half_rn(f0 - __half2float(h0)), __float2half_rn(f1 - __half2float(h1)));
+    const __half2 h = __floats2half2_rn((float)v0, (float)v1);
+    const float2 f = __half22float2(h);
+    *(__half2*)((__half*)out + o) = h;
+    *(__half2*)((__half*)out_lo + o) = __floats2half2_rn((float)v0 - f.x, (float)v1 - f.y);
   } else if constexpr (MODE == kTTMSplitTF32) {
     const float f0 = (float)v0, f1 = (float)v1;
     const float h0 = tf32_round(f0), h1 = tf32_round(f1);
@@ -176,17 +183,74 @@ __device__ __forceinline__ void sector_store2(R* out, R* out_lo, int64_t o, R v0
     *(float2*)((float*)out_lo + o) = make_float2(tf32_round(f0 - h0), tf32_round(f1 - h1));
   } else if constexpr (MODE == kTTMSplitOz) {
     oz_store2((__half*)out, (__half*)out_lo - (__half*)out, o, (double)v0, (double)v1);
+  } else if constexpr (sizeof(R) == 8) {
+    *(double2*)(out + o) = make_double2(v0, v1);
   } else {
-    out[o] = v0;
-    out[o + 1] = v1;
+    *(float2*)(out + o) = make_float2(v0, v1);
   }
 }
 
-template <typename R, int MODE>
+// What the blocks of an operand pass keep in shared memory.
+struct OperandShared {
+  int ylist[2][kMaxLeg], jlist[2][kMaxLeg];     // Y and j of either charge
+  int64_t yrow[2][2][kMaxLeg];                  // row offsets of the Y of either charge, double-buffered
+  int base[kMaxLeg][kMaxLeg][2];                // (b2, b1', charge of rest): start of the run
+};
+
+// 64 rests (two per lane: x0, x1; live: in the run) times every r and Y, NJ contracted indices.
+template <typename R, int MODE, int NJ>
+__device__ __forceinline__ void operand_run(const R* x0, const R* x1, bool ok0, bool ok1, bool live, int i, int jc, int sg,
+                                            int g, uint32_t mb, int ny0, int ny1, int NJp, int Yp, int buf, const R* Us,
+                                            const OperandShared& sh, const SectorOperand& a, R* out, R* out_lo,
+                                            unsigned long long& tmax) {
+  R xa[NJ > 0 ? NJ : 1], xb[NJ > 0 ? NJ : 1];
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) {
+    const int64_t o = sh.jlist[jc][j] * a.in_j;
+    xa[j] = ok0 ? x0[o] : (R)0;
+    xb[j] = ok1 ? x1[o] : (R)0;
+  }
+  const R* uj = Us + (size_t)jc * a.Db * NJp * Yp;
+  for (int r = 0; r < a.Db; ++r, uj += (size_t)NJp * Yp) {
+    const int y = jc ^ bit(mb, r), nyy = y ? ny1 : ny0;    // U[j, r, Y] is nonzero for q(j) + q(r) = q(Y)
+    const int k = (a.sideB ? sh.base[sg][r][g] : sh.base[r][sg][g]) + i;
+    const int64_t ocol = k + (int64_t)(a.P > 1 ? k / (int)a.kps : 0) * (a.rows - 1) * a.kps;
+    for (int yb = 0; yb < nyy; yb += 4) {
+      R va[4] = {0, 0, 0, 0}, vb[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const R* u = uj + j * Yp + yb;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          va[s] = fma(u[s], xa[j], va[s]);
+          vb[s] = fma(u[s], xb[j], vb[s]);
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        if (yb + s >= nyy) break;
+        if (MODE == kTTMMaxAbs) {
+          // magnitudes as integers (same order): no FP64 comparisons
+          if constexpr (sizeof(R) == 8) {
+            tmax = max(tmax, (unsigned long long)__double_as_longlong(va[s]) & 0x7fffffffffffffffull);
+            tmax = max(tmax, (unsigned long long)__double_as_longlong(vb[s]) & 0x7fffffffffffffffull);
+          } else {
+            tmax = max(tmax, (unsigned long long)max(__float_as_uint(va[s]) & 0x7fffffffu,
+                                                     __float_as_uint(vb[s]) & 0x7fffffffu));
+          }
+        } else if (live) {
+          sector_store2<MODE>(out, out_lo, sh.yrow[buf][y][yb + s] + ocol, va[s], vb[s]);
+        }
+      }
+    }
+  }
+}
+
+template <typename R, int MODE, int NJM>
 __global__ void __launch_bounds__(256) sector_operand_kernel(const R* __restrict__ in, const R* __restrict__ U,
                                                              R* __restrict__ out, R* __restrict__ out_lo,
                                                              const __grid_constant__ SectorOperand a) {
-  const int e = blockIdx.y, Q = blockIdx.z;
+  const int e = blockIdx.y;
   const SectorTables t = a.tab.at(e);
   const SectorPlan& p = *t.plan;
   in += e * a.in_bs;
@@ -196,108 +260,144 @@ __global__ void __launch_bounds__(256) sector_operand_kernel(const R* __restrict
   unsigned* amax = a.amax ? a.amax + e * a.amax_bs : nullptr;
   const R uscale = (R)split_scale<MODE>(amax);
   extern __shared__ __align__(16) unsigned char fsm[];
-  R* Us = (R*)fsm;                      // [2][Db][Db][Yp]: (charge of Y, j, r, slot of Y), zero past the last slot
-  __shared__ int ny[2], nj[2], ylist[2][kMaxLeg], jlist[2][kMaxLeg];
-  const int Db = a.Db, Yp = (a.cb + 3) / 4 * 4;
+  R* Us = (R*)fsm;      // [2][Db][NJ][Yp]: (charge of j, r, slot of j, slot of Y), zero past the last slots
+  __shared__ OperandShared sh;
+  const int Db = a.Db, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const uint32_t mb = p.mb, nb = p.nb, na = p.na, mc = p.mc, mm = p.mm;
-  if (threadIdx.x < 2) {
-    const int q = threadIdx.x;
-    int n = 0;
-    for (int y = 0; y < a.cb; ++y)
-      if (bit(nb, y) == q) ylist[q][n++] = y;
-    ny[q] = n;
-    n = 0;
-    for (int j = 0; j < Db; ++j)
-      if (bit(mb, j) == q) jlist[q][n++] = j;
-    nj[q] = n;
+  const int ny1 = odd_below(nb, a.cb), ny0 = a.cb - ny1, nj1 = odd_below(mb, Db), nj0 = Db - nj1;
+  // slots of j: the counts that operand_run is built for (see the switch below)
+  int NJp = max(nj0, nj1);
+  if (NJM > 8) NJp = NJp <= 4 ? 4 : (NJp <= 8 ? NJp : (NJp <= 10 ? 10 : (NJp <= 12 ? 12 : 16)));
+  const int Yp = (max(ny0, ny1) + 3) / 4 * 4;
+  const int n0 = p.n3[0], n1 = p.n3[1];
+  if (threadIdx.x < 2 * kMaxLeg) sh.jlist[threadIdx.x / kMaxLeg][threadIdx.x % kMaxLeg] = 0;   // unused slots: any valid j
+  __syncthreads();
+  if (threadIdx.x < kMaxLeg) {
+    const int i = threadIdx.x;
+    if (i < a.cb) sh.ylist[bit(nb, i)][bit(nb, i) ? odd_below(nb, i) : i - odd_below(nb, i)] = i;
+    if (i < Db) sh.jlist[bit(mb, i)][bit(mb, i) ? odd_below(mb, i) : i - odd_below(mb, i)] = i;
+  }
+  for (int i = threadIdx.x; i < Db * Db * 2; i += blockDim.x) {
+    const int g = i & 1, b1 = (i >> 1) % Db, b2 = (i >> 1) / Db;
+    const int o1 = odd_below(mb, b1), o2 = odd_below(mb, b2);
+    const int q1 = g ^ bit(mb, b1), Q = q1 ^ bit(mb, b2);       // charge of (b1', rest), of the summed index
+    const int m0 = nj0 * n0 + nj1 * n1, m1 = nj0 * n1 + nj1 * n0;   // all runs of one b2 by the charge of (b1', rest)
+    sh.base[b2][b1][g] = (b2 - o2) * (Q ? m1 : m0) + o2 * (Q ? m0 : m1) + (b1 - o1) * (q1 ? n1 : n0) + o1 * (q1 ? n0 : n1);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 2 * Db * Db * Yp; i += blockDim.x) {
-    const int sl = i % Yp, r = (i / Yp) % Db, j = (i / (Yp * Db)) % Db, q = i / (Yp * Db * Db);
-    Us[i] = sl < ny[q] ? U[j * a.u_j + r * a.u_r + ylist[q][sl]] * uscale : (R)0;
+  for (int i = threadIdx.x; i < 2 * Db * NJp * Yp; i += blockDim.x) {
+    const int sl = i % Yp, js = (i / Yp) % NJp, r = (i / (Yp * NJp)) % Db, jc = i / (Yp * NJp * Db);
+    const int y = jc ^ bit(mb, r);
+    const bool in_u = sl < (y ? ny1 : ny0) && js < (jc ? nj1 : nj0);
+    Us[i] = in_u ? U[sh.jlist[jc][js] * a.u_j + r * a.u_r + sh.ylist[y][sl]] * uscale : (R)0;
   }
-  __syncthreads();
-  const int KQ = p.K[Q], Kpad = (KQ + a.kalign - 1) / a.kalign * a.kalign;
-  const uint2* kt = (a.sideB ? t.kB : t.kA) + (Q ? p.K[0] : 0);
   const int rows0 = p.row[0][a.x0 + a.xs] - p.row[0][a.x0];   // charge-0 rows of the slice
-  const int rq = Q ^ a.parity;                                // charge of the rows with nonzero entries
-  const int rbase = (rq ? rows0 : 0) - p.row[rq][a.x0];
-  R tmax = 0;
-  for (int o = blockIdx.x; o < a.nouter; o += gridDim.x) {
-    int r = o;
-    const int m = r % a.Dm;
-    r /= a.Dm;
-    const int c1 = r % a.Dc;
-    r /= a.Dc;
-    const int c0 = r % a.Dc;
-    const int X = r / a.Dc;
-    const int y = rq ^ bit(na, a.x0 + X) ^ bit(mc, c0) ^ bit(mc, c1) ^ bit(mm, m);
-    const R* src = in + X * a.in_x + c0 * a.in_c0 + c1 * a.in_c1 + m * a.in_m;
-    const uint32_t* rt = t.row + (((int64_t)(a.x0 + X) * a.cb * a.Dc + c0) * a.Dc + c1) * a.Dm + m;
-    const int64_t ystep = (int64_t)a.Dc * a.Dc * a.Dm;
-    const int nyy = ny[y];
-    const R* Uy = Us + (size_t)y * Db * Db * Yp;
-    for (int k = 2 * threadIdx.x; k < Kpad; k += 2 * blockDim.x) {
-      const int pn = a.P > 1 ? k / a.kps : 0;
-      const int64_t ocol = (int64_t)pn * a.rows * a.kps + (k - pn * a.kps);
-      for (int yb = 0; yb < nyy; yb += 4) {
-        R v[2][4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-#pragma unroll
-          for (int s = 0; s < 4; ++s) v[h][s] = 0;
-          if (k + h < KQ) {
-            const uint2 q = kt[k + h];
-            const R* x = src + q.x;
-            const int jc = y ^ bit(mb, (int)q.y);   // U[j, r, Y] is nonzero for q(j) + q(r) = q(Y)
-            const int n = nj[jc];
-            const R* u = Uy + (size_t)q.y * Yp + yb;
-#pragma unroll 4
-            for (int i = 0; i < n; ++i) {
-              const int j = jlist[jc][i];
-              const R xv = x[(int64_t)j * a.in_j];
-              const R* uj = u + (size_t)j * Db * Yp;
-#pragma unroll
-              for (int s = 0; s < 4; ++s) v[h][s] = fma(uj[s], xv, v[h][s]);
-            }
-          }
-        }
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-          if (yb + s >= nyy) break;
-          if (MODE == kTTMMaxAbs) {
-            tmax = fmax(tmax, fmax(fabs(v[0][s]), fabs(v[1][s])));
-          } else {
-            const int row = (int)(rt[ylist[y][yb + s] * ystep] & 0x7fffffffu) + rbase;
-            sector_store2<MODE>(out, out_lo, (int64_t)row * a.kps + ocol, v[0][s], v[1][s]);
-          }
-        }
+  const int roff0 = -p.row[0][a.x0], roff1 = rows0 - p.row[1][a.x0];
+  const int c0n = (n0 + 63) / 64, per_seg = c0n + (n1 + 63) / 64;
+  const uint32_t* rest = a.sideB ? t.kB : t.kA;
+  const int K0 = p.K[0], K1 = p.K[1];
+  unsigned long long tmax = 0;
+  int buf = 0;
+  for (int o = blockIdx.x; o < a.nouter; o += gridDim.x, buf ^= 1) {
+    int r4 = o;
+    const int m = r4 % a.Dm;
+    r4 /= a.Dm;
+    const int c1 = r4 % a.Dc;
+    r4 /= a.Dc;
+    const int c0 = r4 % a.Dc;
+    const int X = r4 / a.Dc;
+    const int qo = bit(na, a.x0 + X) ^ bit(mc, c0) ^ bit(mc, c1) ^ bit(mm, m) ^ a.parity;
+    if (threadIdx.x < a.cb) {
+      const int Y = threadIdx.x, q = bit(nb, Y);
+      const uint32_t rk = t.row[((((int64_t)(a.x0 + X) * a.cb + Y) * a.Dc + c0) * a.Dc + c1) * a.Dm + m];
+      sh.yrow[buf][q][q ? odd_below(nb, Y) : Y - odd_below(nb, Y)] =
+          ((int64_t)(int)(rk & 0x7fffffffu) + (rk >> 31 ? roff1 : roff0)) * a.kps;
+    }
+    __syncthreads();
+    if (MODE != kTTMMaxAbs && MODE != kTTMStore) {
+      // zeros up to a whole k-block behind every row (a row of charge q holds the k of charge q + parity)
+      for (int i = 2 * threadIdx.x; i < a.cb * a.kalign; i += 2 * blockDim.x) {
+        const int Y = i / a.kalign, q = bit(nb, Y), KQ = (q ^ qo) ? K1 : K0;
+        const int k = KQ + i % a.kalign;
+        if (k >= (KQ + a.kalign - 1) / a.kalign * a.kalign) continue;
+        const int sl = q ? odd_below(nb, Y) : Y - odd_below(nb, Y);
+        sector_store2<MODE>(out, out_lo, sh.yrow[buf][q][sl] + k + (int64_t)(a.P > 1 ? k / (int)a.kps : 0) * (a.rows - 1) * a.kps,
+                            (R)0, (R)0);
       }
     }
+    const R* src = in + X * a.in_x + c0 * a.in_c0 + c1 * a.in_c1 + m * a.in_m;
+    for (int it = warp; it < Db * per_seg; it += nwarp) {
+      const int sg = it / per_seg, w = it - sg * per_seg;
+      const int g = w >= c0n, i = (w - (g ? c0n : 0)) * 64 + 2 * lane;
+      const bool live = i < (g ? n1 : n0);
+      const uint2 ro = live ? *(const uint2*)(rest + (g ? n0 : 0) + i) : make_uint2(~0u, ~0u);
+      const bool ok0 = ro.x != ~0u, ok1 = ro.y != ~0u;
+      const R* xs = src + (int64_t)sg * a.in_seg;
+      const R* x0 = xs + (ok0 ? ro.x : 0u);
+      const R* x1 = xs + (ok1 ? ro.y : 0u);
+      const int jc = qo ^ g ^ bit(mb, sg);                     // charge of the j with nonzero entries
+      const int njc = jc ? nj1 : nj0;
+#define HOTRG_RUN(N)                                                                                                 \
+  operand_run<R, MODE, N>(x0, x1, ok0, ok1, live, i, jc, sg, g, mb, ny0, ny1, NJp, Yp, buf, Us, sh, a, out, out_lo, tmax)
+      if constexpr (NJM <= 8) {
+        switch (njc) {
+          case 0: HOTRG_RUN(0); break;
+          case 1: HOTRG_RUN(1); break;
+          case 2: HOTRG_RUN(2); break;
+          case 3: HOTRG_RUN(3); break;
+          case 4: HOTRG_RUN(4); break;
+          case 5: if constexpr (NJM >= 5) HOTRG_RUN(5); break;
+          case 6: if constexpr (NJM >= 6) HOTRG_RUN(6); break;
+          case 7: if constexpr (NJM >= 7) HOTRG_RUN(7); break;
+          default: if constexpr (NJM >= 8) HOTRG_RUN(8); break;
+        }
+      } else {
+        switch (njc) {
+          case 0: case 1: case 2: case 3: case 4: HOTRG_RUN(4); break;   // unused slots: U is zero there
+          case 5: HOTRG_RUN(5); break;
+          case 6: HOTRG_RUN(6); break;
+          case 7: HOTRG_RUN(7); break;
+          case 8: HOTRG_RUN(8); break;
+          case 9: case 10: HOTRG_RUN(10); break;
+          case 11: case 12: HOTRG_RUN(12); break;
+          default: HOTRG_RUN(16); break;
+        }
+      }
+#undef HOTRG_RUN
+    }
   }
-  if (MODE == kTTMMaxAbs) merge_max(amax, (double)tmax, a.amax_mul);   // every thread gets here
+  if (MODE == kTTMMaxAbs) {   // every thread gets here
+    if constexpr (sizeof(R) == 8) merge_max(amax, __longlong_as_double((long long)tmax), a.amax_mul);
+    else merge_max(amax, (double)__uint_as_float((unsigned)tmax), a.amax_mul);
+  }
 }
 
 template <typename R>
 cudaError_t launch_sector_operand(const R* in, const R* U, R* out, R* out_lo, const SectorOperand& a, int ne, int mode,
                                   cudaStream_t st) {
-  const int Yp = (a.cb + 3) / 4 * 4;
-  const size_t smem = (size_t)2 * a.Db * a.Db * Yp * sizeof(R);
+  const size_t smem = (size_t)2 * a.Db * a.Db * ((a.cb + 3) / 4 * 4 + 4) * sizeof(R);   // a bound for any charges
   if (smem > (size_t)kSectorSmem) return cudaErrorInvalidValue;
   int64_t bx = a.nouter;
-  const int64_t cap = 152 * 32 / ne > 64 ? 152 * 32 / ne : 64;
+  const int64_t cap = 152 * 16 / ne > 32 ? 152 * 16 / ne : 32;
   if (bx > cap) bx = cap;
-  const dim3 g((unsigned)bx, ne, 2);
+  const dim3 g((unsigned)bx, ne);
   auto go = [&](auto kernel) -> cudaError_t {
     kernel<<<g, 256, smem, st>>>(in, U, out, out_lo, a);
     return cudaGetLastError();
   };
+  // the contracted leg's indices of one charge are at most D_b (all of one charge)
+  auto pick = [&](auto mode_const) -> cudaError_t {
+    constexpr int MODE = decltype(mode_const)::value;
+    if (a.Db <= 4) return go(sector_operand_kernel<R, MODE, 4>);
+    if (a.Db <= 8) return go(sector_operand_kernel<R, MODE, 8>);
+    return go(sector_operand_kernel<R, MODE, 16>);
+  };
   switch (mode) {
-    case kTTMStore: return go(sector_operand_kernel<R, kTTMStore>);
-    case kTTMMaxAbs: return go(sector_operand_kernel<R, kTTMMaxAbs>);
-    case kTTMSplitF16: if constexpr (sizeof(R) == 4) return go(sector_operand_kernel<R, kTTMSplitF16>); break;
-    case kTTMSplitTF32: if constexpr (sizeof(R) == 4) return go(sector_operand_kernel<R, kTTMSplitTF32>); break;
-    case kTTMSplitOz: if constexpr (sizeof(R) == 8) return go(sector_operand_kernel<R, kTTMSplitOz>); break;
+    case kTTMStore: return pick(std::integral_constant<int, kTTMStore>{});
+    case kTTMMaxAbs: return pick(std::integral_constant<int, kTTMMaxAbs>{});
+    case kTTMSplitF16: if constexpr (sizeof(R) == 4) return pick(std::integral_constant<int, kTTMSplitF16>{}); break;
+    case kTTMSplitTF32: if constexpr (sizeof(R) == 4) return pick(std::integral_constant<int, kTTMSplitTF32>{}); break;
+    case kTTMSplitOz: if constexpr (sizeof(R) == 8) return pick(std::integral_constant<int, kTTMSplitOz>{}); break;
   }
   return cudaErrorInvalidValue;
 }
@@ -564,13 +664,9 @@ void sectors_prepare() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || done[dev]) return;
   done[dev] = true;
   auto set = [](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSectorSmem); };
-  set(sector_operand_kernel<float, kTTMStore>);
-  set(sector_operand_kernel<float, kTTMMaxAbs>);
-  set(sector_operand_kernel<float, kTTMSplitF16>);
-  set(sector_operand_kernel<float, kTTMSplitTF32>);
-  set(sector_operand_kernel<double, kTTMStore>);
-  set(sector_operand_kernel<double, kTTMMaxAbs>);
-  set(sector_operand_kernel<double, kTTMSplitOz>);
+  set(sector_operand_kernel<double, kTTMStore, 16>);
+  set(sector_operand_kernel<double, kTTMMaxAbs, 16>);
+  set(sector_operand_kernel<double, kTTMSplitOz, 16>);
   set(sector_close1_kernel<float, 16>);
   set(sector_close1_kernel<double, 8>);
   set(sector_close1_kernel<double, 16>);

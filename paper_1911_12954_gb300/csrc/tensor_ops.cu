@@ -788,28 +788,28 @@ __global__ void __launch_bounds__(256) sector_stats_kernel(const __half* __restr
   const SectorPlan& p = *tab.at(elem).plan;
   const int64_t r0 = p.row[0][x0 + nx] - p.row[0][x0];        // rows of charge 0: first in the plane
   const int64_t nrow = r0 + p.row[1][x0 + nx] - p.row[1][x0];
-  unsigned long long nz = 0, ns = 0;
+  unsigned long long nnz = 0, ns = 0;          // what is not stored is zero
   unsigned mx = 0;
-  const int64_t n = nrow * K;
+  const int64_t Kmax = max(p.K[0], p.K[1]), n = nrow * Kmax;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / K, k = i - r * K;
-    unsigned a = 0u;
-    if (k < p.K[(r < r0 ? 0 : 1) ^ parity])
-      a = __half_as_ushort(pl[(k / kps * rows + r) * kps + k % kps]) & 0x7fffu;
-    nz += a == 0u;
+    const int64_t r = i / Kmax, k = i - r * Kmax;
+    if (k >= p.K[(r < r0 ? 0 : 1) ^ parity]) continue;
+    const unsigned a = __half_as_ushort(pl[(k / kps * rows + r) * kps + k % kps]) & 0x7fffu;
+    nnz += a != 0u;
     ns += (a != 0u && a < 0x0400u);
     mx = max(mx, a);
   }
   for (int off = 16; off > 0; off >>= 1) {
-    nz += __shfl_down_sync(0xffffffffu, nz, off);
+    nnz += __shfl_down_sync(0xffffffffu, nnz, off);
     ns += __shfl_down_sync(0xffffffffu, ns, off);
     mx = max(mx, __shfl_down_sync(0xffffffffu, mx, off));
   }
   if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&out[0], nz);
+    atomicAdd(&out[0], 0ull - nnz);
     atomicAdd(&out[1], ns);
     atomicMax(&out[2], (unsigned long long)mx);
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&out[0], (unsigned long long)(nrow * K));
 }
 
 cudaError_t launch_sector_stats(const void* plane, const SectorTab& tab, int elem, int parity, int x0, int nx,
