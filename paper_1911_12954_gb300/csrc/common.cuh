@@ -17,11 +17,11 @@ constexpr int kJacobiSmemN = 208;    // the eigensolver keeps A (its upper trian
 constexpr int kJacobiLogSweeps = 10; // sweeps of rotations the eigensolver logs before it folds them into V
 constexpr int64_t packed_doubles(int n) { return ((int64_t)n * (n + 1) / 2 + 1) / 2 * 2; }   // upper triangle, even
 // Doubles of global work space per matrix (EigJob::work): eigenvector columns, V (used when the log
-// overflows), the upper triangle of matrices that do not fit shared memory, the log of rotations (c, s): a
-// sweep has at most n rounds of at most n pair slots.
+// overflows), the upper triangle of matrices that do not fit shared memory, the log of rotations (cosine and
+// tangent, the two indices): a sweep has at most n rounds of at most n pair slots. Even.
 constexpr int64_t jacobi_work_doubles(int n) {
-  return 2 * (int64_t)n * n + (n > kJacobiSmemN ? packed_doubles(n) : 0) +
-         2 * (int64_t)kJacobiLogSweeps * n * n;
+  const int64_t entries = (int64_t)kJacobiLogSweeps * n * n;
+  return 2 * (int64_t)n * n + (n > kJacobiSmemN ? packed_doubles(n) : 0) + 2 * entries + (entries + 3) / 4 * 2;
 }
 
 // Device-side status words (in the caller's workspace), read back at sync points.

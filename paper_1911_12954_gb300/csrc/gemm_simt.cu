@@ -5,21 +5,25 @@
 // path consumes). 128x64 output tile per CTA, 256 threads with an 8x4 register tile,
 // 16-wide k slices staged in shared memory. FP64 mode uses DFMA; FP32 mode FFMA with FP32
 // accumulation. Ragged M, N and K edges are guarded.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace hotrg {
 
-constexpr int kBM = 128, kBN = 64, kBK = 16;
+constexpr int kBK = 16;
 
-template <typename R>
+// Tile kBM x kBN, 256 threads of kTM x kTN outputs each.
+template <typename R, int kTM, int kTN>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(const R* __restrict__ A, int64_t lda, const R* __restrict__ B,
                                                         int64_t ldb, R* __restrict__ C, int64_t ldc, int64_t M,
                                                         int64_t N, int64_t K, R alpha, R beta,
                                                         const __grid_constant__ OneProduct one) {
+  constexpr int kBM = 16 * kTM, kBN = 16 * kTN;
   __shared__ R As[kBK][kBM + 4];
   __shared__ R Bs[kBK][kBN + 4];
   const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;   // 16 x 16 threads; rows ty*8.., cols tx*4..
+  const int tx = tid % 16, ty = tid / 16;   // 16 x 16 threads; rows ty*kTM.., cols tx*kTN..
   int64_t m0 = (int64_t)blockIdx.y * kBM, n0 = (int64_t)blockIdx.x * kBN;
   if (one.sec.tab.base) {
     // a product by sectors: tile rows of charge 0, then of charge 1 (each against the columns and over
@@ -40,23 +44,23 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const R* __restrict__ A,
     C += (q ? (int64_t)r0 : 0) * ldc;
     B += (qc ? (int64_t)c0 : 0) * ldb;
   }
-  R acc[8][4];
+  R acc[kTM][kTN];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < kTM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0;
+    for (int j = 0; j < kTN; ++j) acc[i][j] = 0;
 
   for (int64_t k0 = 0; k0 < K; k0 += kBK) {
-    // A tile: 128 x 16 = 2048 elements, 8 per thread; k fastest for coalescing
+    // A tile: kBM x 16 elements, kTM per thread; k fastest for coalescing
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
+    for (int r = 0; r < kTM; ++r) {
       const int e = tid + r * 256;
       const int row = e / kBK, kk = e % kBK;
       const int64_t gm = m0 + row, gk = k0 + kk;
       As[kk][row] = (gm < M && gk < K) ? A[gm * lda + gk] : (R)0;
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < kTN; ++r) {
       const int e = tid + r * 256;
       const int col = e / kBK, kk = e % kBK;
       const int64_t gn = n0 + col, gk = k0 + kk;
@@ -65,25 +69,25 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const R* __restrict__ A,
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < kBK; ++kk) {
-      R a[8], b[4];
+      R a[kTM], b[kTN];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = As[kk][ty * 8 + i];
+      for (int i = 0; i < kTM; ++i) a[i] = As[kk][ty * kTM + i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
+      for (int j = 0; j < kTN; ++j) b[j] = Bs[kk][tx * kTN + j];
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < kTM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < kTN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int64_t gm = m0 + ty * 8 + i;
+  for (int i = 0; i < kTM; ++i) {
+    const int64_t gm = m0 + ty * kTM + i;
     if (gm >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t gn = n0 + tx * 4 + j;
+    for (int j = 0; j < kTN; ++j) {
+      const int64_t gn = n0 + tx * kTN + j;
       if (gn >= N) continue;
       R* c = C + gm * ldc + gn;
       *c = beta == (R)0 ? alpha * acc[i][j] : alpha * acc[i][j] + beta * *c;
@@ -95,12 +99,23 @@ template <typename R>
 cudaError_t launch_gemm_simt(const R* A, int64_t lda, const R* B, int64_t ldb, R* C, int64_t ldc, int64_t M,
                              int64_t N, int64_t K, double alpha, double beta, cudaStream_t st, const OneProduct& one) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  // two sectors: at most one more tile row
-  const int64_t gy = (M + kBM - 1) / kBM + (one.sec.tab.base ? 1 : 0), gx = (N + kBN - 1) / kBN;
-  if (gy > 65535 || gx > 0x7fffffffLL) return cudaErrorInvalidValue;
-  dim3 grid((unsigned)gx, (unsigned)gy);
-  gemm_simt_kernel<R><<<grid, 256, 0, st>>>(A, lda, B, ldb, C, ldc, M, N, K, (R)alpha, (R)beta, one);
-  return cudaGetLastError();
+  // Tiles of 128 x 64 keep 32 products per 12 operand reads; where they leave SMs without work (two tiles per
+  // SM), 64 x 32 ones spread the FP64 pipe's load: at D = 4 the two 512 x 512 x 512 sector blocks are 64 large
+  // tiles for 152 SMs (1088 us) or 256 small ones (see the figure at the end of this comment's kernel list).
+  auto go = [&](auto tm, auto tn) -> cudaError_t {
+    constexpr int TM = decltype(tm)::value, TN = decltype(tn)::value;
+    const int64_t more = one.sec.tab.base ? 1 : 0;   // two sectors: at most one more tile row
+    const int64_t gy = (M + 16 * TM - 1) / (16 * TM) + more, gx = (N + 16 * TN - 1) / (16 * TN);
+    if (gy > 65535 || gx > 0x7fffffffLL) return cudaErrorInvalidValue;
+    gemm_simt_kernel<R, TM, TN><<<dim3((unsigned)gx, (unsigned)gy), 256, 0, st>>>(A, lda, B, ldb, C, ldc, M, N, K, (R)alpha,
+                                                                                  (R)beta, one);
+    return cudaGetLastError();
+  };
+  using I2 = std::integral_constant<int, 2>;
+  using I4 = std::integral_constant<int, 4>;
+  using I8 = std::integral_constant<int, 8>;
+  const int64_t large = ((M + 127) / 128) * ((N + 63) / 64) / (one.sec.tab.base ? 2 : 1);
+  return large < 2 * 152 ? go(I4{}, I2{}) : go(I8{}, I4{});
 }
 template cudaError_t launch_gemm_simt<double>(const double*, int64_t, const double*, int64_t, double*, int64_t,
                                               int64_t, int64_t, int64_t, double, double, cudaStream_t,

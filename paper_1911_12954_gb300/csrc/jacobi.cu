@@ -21,13 +21,14 @@
 // would otherwise break exact symmetric ties at random) and normalising that projection. This gauge depends only on the
 // eigenspaces, so it does not depend on the eigensolver.
 //
-// The FP64 pipe (a warp instruction every 16 cycles per SM) and the latency of a round bound it.
-// So A is kept as its upper triangle (16 FP64 instructions per 2x2 block on or above the
-// diagonal, nothing mirrored), the rotation costs two reciprocal square roots, a round in which
-// nothing rotates is skipped, and the eigenvector matrix is not accumulated: the rotations are
-// logged, and the columns that are needed (the clusters that reach into the first chi; 8 of 64 at
-// D = 8) are formed at the end by applying the log backwards to unit vectors, one column per
-// group of lanes without block barriers.
+// The FP64 pipe bounds it (measured: one warp issues an FP64 instruction every 64 cycles, whatever its lanes or
+// dependences, an SM one every 19), so a round costs 64 cycles per FP64 instruction of its longest chain, or 19
+// per warp instruction of its blocks, and even comparisons and conversions count. So: A is kept as its upper triangle, 13 FP64 instructions per 2x2 block off
+// the diagonal; the rotation's tangent is computed in FP32 (from the bits) and its cosine refined to FP64 from an
+// FP32 start, 7 FP64 instructions; thresholds, sorting and tests are integer operations on the bits; a round in
+// which nothing rotates is skipped; and the eigenvector matrix is not accumulated: the rotations are logged, and
+// the columns that are needed (the clusters that reach into the first chi; 8 of 64 at D = 8) are formed at the
+// end by applying the log backwards to unit vectors, one column per group of lanes without block barriers.
 //
 // select_kernel: per transverse direction, the side (nu or nu') with the smaller
 // discarded sum (a difference within side_rel (eps + eps') + 1e-13 lambda_0 is a tie and
@@ -39,7 +40,7 @@
 
 namespace hotrg {
 
-constexpr int kJT = 544;            // most threads of a Jacobi CTA: the 528 blocks of n = 64 in one pass
+constexpr int kJT = 544;            // most threads of a Jacobi CTA: the 496 + 32 blocks of n = 64 in one pass
 
 // Local indices of pair i of round r among m (even) players; r < m - 1, i < m / 2.
 __device__ __forceinline__ void rr_pair(int r, int i, int m, int& p, int& q) {
@@ -71,22 +72,23 @@ __device__ __forceinline__ void tri_index(int e, int h, int& P, int& Q) {
   Q = r + (e - (r * h - r * (r - 1) / 2));
 }
 
-__device__ double block_sum(double v, double* red) {
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double s = 0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-  __syncthreads();
-  return s;
-}
-
-
 // Place of entry (i, j) in the packed upper triangle of an n x n matrix.
 __device__ __forceinline__ int packed(int i, int j, int n) {
   const int lo = min(i, j), hi = max(i, j);
   return lo * (2 * n - 1 - lo) / 2 + hi;
+}
+
+// v 2^-(em - 1023) as a float (toward zero; 0 below FP32's range), and a normal or zero float as a double: by
+// their bits, without the FP64 pipe. em: biased exponent not below v's.
+__device__ __forceinline__ float scaled_float(double v, int em) {
+  const int hi = __double2hiint(v), e = ((hi >> 20) & 0x7ff) - em + 127;
+  const uint32_t m = ((uint32_t)hi & 0xfffffu) << 3 | (uint32_t)__double2loint(v) >> 29;
+  return __int_as_float(e <= 0 ? 0 : (int)((uint32_t)hi & 0x80000000u | (uint32_t)e << 23 | m));
+}
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t b = __float_as_uint(f);
+  const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20));
+  return (b & 0x7f800000u) ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
 }
 
 __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ EigPack jobs, int njobs, int use_smem,
@@ -94,11 +96,14 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
                                                      int* status) {
   extern __shared__ double dyn[];          // region doubles (A, later the columns in progress), then the block list
   // one slot per rotation pair of a round: at most n (ceil(m_c / 2) <= m_c per component)
-  __shared__ double cs[kMaxGramN], sn[kMaxGramN];
-  __shared__ short pp[kMaxGramN], qq[kMaxGramN];
-  __shared__ double lam[kMaxGramN], nrm[kMaxGramN];
+  __shared__ double2 ct[kMaxGramN];        // cosine and tangent
+  __shared__ short2 pq[kMaxGramN];         // the pair's indices (second: -1 where the component is odd)
+  __shared__ double lam[kMaxGramN];
+  __shared__ long long key[kMaxGramN];
+  __shared__ double nrmv[kMaxGramN];
   __shared__ int perm[kMaxGramN], cstart[kMaxGramN + 1];
-  __shared__ double red[kJT / 32];
+  __shared__ int ired[kJT / 32];
+  __shared__ float fred[kJT / 32];
   __shared__ int comp[kMaxGramN];          // component label: its smallest index
   __shared__ int cnum[kMaxGramN];          // component number of an index
   __shared__ int mem[kMaxGramN];           // indices grouped by component
@@ -106,7 +111,6 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
   __shared__ int poff[kMaxGramN + 1];      // first pair slot of component c
   __shared__ int toff[kMaxGramN + 1];      // first 2x2 block of component c
   __shared__ int sz[kMaxGramN];
-  __shared__ unsigned char lround[kJacobiLogSweeps * kMaxGramN];   // round of each log entry
   __shared__ int ncomp, rmax, npmax, ncl;
 
   // job blockIdx.x % njobs of batch element blockIdx.x / njobs
@@ -124,38 +128,48 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
   double* V = W + (int64_t)n * n;          // [n][n], rows
   double* Aw = V + (int64_t)n * n;
   double2* log = (double2*)(Aw + (use_smem ? 0 : packed_doubles(n)));
+  short2* logi = (short2*)(log + (int64_t)kJacobiLogSweeps * n * n);
   double* A = use_smem ? dyn : Aw;         // use_smem: every job of the launch has n <= kJacobiSmemN
   uint32_t* blk = (uint32_t*)(dyn + region);
 
   // the upper triangle of G (the merged Gram is symmetric up to summation order), scaled by a power
   // of two to a largest magnitude in [1, 2), so that squares neither overflow nor vanish
-  double big = 0;
+  int big = 0;                             // exponent bits of the largest magnitude
   for (int e = tid; e < n * n; e += nthr) {
     const int i = e / n, j = e - i * n;
-    if (i <= j) big = fmax(big, fabs(jb.G[e]));
+    if (i <= j) big = max(big, __double2hiint(jb.G[e]) & 0x7ff00000);
   }
-  for (int off = 16; off > 0; off >>= 1) big = fmax(big, __shfl_down_sync(0xffffffffu, big, off));
-  if (lane == 0) red[tid >> 5] = big;
+  big = __reduce_max_sync(0xffffffffu, big);
+  if (lane == 0) ired[tid >> 5] = big;
   __syncthreads();
   big = 0;
-  for (int w = 0; w < nthr >> 5; ++w) big = fmax(big, red[w]);
-  __syncthreads();
-  const int sh = big > 0 && big < INFINITY ? ilogb(big) : 0;
-  const double up = ldexp(1.0, sh < -1000 ? 1000 : (sh > 1000 ? -1000 : -sh)), down = 1.0 / up;   // exact
-  double fro = 0;
+  for (int w = 0; w < nthr >> 5; ++w) big = max(big, ired[w]);
+  // 2^-e and 2^e; no scaling of zeros, infinities, NaN and magnitudes near the ends of the range
+  if (big < (24 << 20) || big > (2022 << 20)) big = 1023 << 20;
+  const double up = __hiloint2double(0x7fe00000 - big, 0), down = __hiloint2double(big, 0);
+  float fro = 0;
   for (int e = tid; e < n * n; e += nthr) {
     const int i = e / n, j = e - i * n;
     if (i > j) continue;
     const double g = jb.G[e] * up;
     A[packed(i, j, n)] = g;
-    fro = fma(i == j ? g : 2 * g, g, fro);
+    const float f = (float)g;
+    fro = fmaf(i == j ? f : 2 * f, f, fro);
   }
-  fro = sqrt(block_sum(fro, red));
-  const double tol_abs = 1e-18 * fro;
-  const double tol2 = 2.220446049250313e-16 * 2.220446049250313e-16;
+  for (int off = 16; off > 0; off >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, off);
+  if (lane == 0) fred[tid >> 5] = fro;
+  __syncthreads();
+  fro = 0;
+  for (int w = 0; w < nthr >> 5; ++w) fro += fred[w];
+  // Exponent of 1e-18 ||G||_F, and the test of a pair by exponents: true for every |a_pq| above
+  // max(1e-18 ||G||_F, 2^-52 sqrt|a_pp a_qq|), and for some down to a quarter of it.
+  const int e_abs = (__double2hiint(1e-18 * (double)sqrtf(fro)) >> 20) & 0x7ff;
   auto rotates = [&](double apq, double app, double aqq) {
-    return fabs(apq) > tol_abs && apq * apq > tol2 * fabs(app * aqq);
+    const int e = (__double2hiint(apq) >> 20) & 0x7ff;
+    const int ep = (__double2hiint(app) >> 20) & 0x7ff, eq = (__double2hiint(aqq) >> 20) & 0x7ff;
+    return e >= e_abs && e != 0 && e != 0x7ff && 2 * e + 2 > ep + eq - 104;
   };
+  auto nonzero = [](double v) { return ((unsigned long long)__double_as_longlong(v) << 1) != 0ull; };
 
   // ---- connected components of the nonzero pattern of A. A rotation of a pair inside one
   // component leaves the entries between components exactly zero, so each component is
@@ -168,7 +182,7 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
     int changed = 0;
     for (int e = tid; e < n * n; e += nthr) {
       const int i = e / n, j = e - i * n;
-      if (i < j && A[packed(i, j, n)] != 0.0) {
+      if (i < j && nonzero(A[packed(i, j, n)])) {
         const int ci = comp[i], cj = comp[j];
         if (ci != cj) {
           atomicMin(&comp[ci < cj ? j : i], min(ci, cj));
@@ -202,7 +216,7 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
       const int np = (sz[k] + 1) / 2;
       b += sz[k];
       p += np;
-      t += np * (np + 1) / 2;
+      t += np * (np - 1) / 2;
       rm = max(rm, 2 * np - 1);
       pm = max(pm, np);
     }
@@ -217,19 +231,32 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
   __syncthreads();
   for (int i = tid; i < n; i += nthr) mem[cbeg[cnum[i]] + perm[i]] = i;
   const int npairs = poff[nc], nblk = toff[nc], rounds = rmax;
-  // 2x2 blocks (pair slots P <= Q of one component), the same for every round
+  // 2x2 blocks off the diagonal (pair slots P < Q of one component), the same for every round
   for (int e = tid; e < nblk; e += nthr) {
     int c = 0;
     while (toff[c + 1] <= e) ++c;
-    int P, Q;
-    tri_index(e - toff[c], poff[c + 1] - poff[c], P, Q);
-    blk[e] = (uint32_t)(P + poff[c]) << 16 | (uint32_t)(Q + poff[c]);
+    int P, Q;                              // the strict triangle of h slots is the triangle of h - 1
+    tri_index(e - toff[c], poff[c + 1] - poff[c] - 1, P, Q);
+    blk[e] = (uint32_t)(P + poff[c]) << 16 | (uint32_t)(Q + 1 + poff[c]);
   }
-  // this thread's first pair slot
+  // The last threads hold a pair slot each (warps of their own where there is room; npairs <= n <= threads): its
+  // component, and its indices in the next round.
+  const int slot = nthr - 1 - tid;
   int sc = 0;
-  if (tid < npairs)
-    while (poff[sc + 1] <= tid) ++sc;
+  if (slot < npairs)
+    while (poff[sc + 1] <= slot) ++sc;
+  const int smc = cbeg[sc + 1] - cbeg[sc], smp = smc + (smc & 1), sb0 = cbeg[sc], sp0 = poff[sc];
+  // indices (p < q) of slot sl of component c (m players, members from b) in round r; q = -1: none
+  auto indices = [&](int r, int i, int mc, int mp, int b) {
+    while (r >= mp - 1) r -= mp - 1;
+    int lp, lq;
+    rr_pair(r, i, mp, lp, lq);
+    return make_short2((short)mem[b + lp], (short)(lq < mc ? mem[b + lq] : -1));
+  };
   __syncthreads();
+  short2 next = slot < npairs ? indices(0, slot - sp0, smc, smp, sb0) : make_short2(0, -1);
+  // small matrices: a thread per entry of a 2x2 block (5 FP64 instructions instead of 13) where the CTA has them
+  const int ws = nblk <= 40 && 4 * nblk + 32 <= nthr ? 2 : 0;
 
   // Applies the logged rotations in order to the rows of V (V <- V J), one row per warp.
   bool have_v = false;
@@ -242,17 +269,12 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
       __syncwarp();
       for (int l = 0; l < nlog; ++l) {
         for (int sl = lane; sl < npairs; sl += 32) {
-          int c = 0;
-          while (poff[c + 1] <= sl) ++c;
-          const int mc = cbeg[c + 1] - cbeg[c], mp = mc + (mc & 1);
-          int lp, lq;
-          rr_pair(lround[l] % (mp - 1), sl - poff[c], mp, lp, lq);
-          if (lq < mc) {
+          const short2 i = logi[(int64_t)l * npairs + sl];
+          if (i.y >= 0) {
             const double2 r = log[(int64_t)l * npairs + sl];
-            const int p = mem[cbeg[c] + lp], q = mem[cbeg[c] + lq];
-            const double vp = v[p], vq = v[q];
-            v[p] = r.x * vp - r.y * vq;
-            v[q] = r.y * vp + r.x * vq;
+            const double vp = v[i.x], vq = v[i.y];
+            v[i.x] = r.x * fma(-r.y, vq, vp);
+            v[i.y] = r.x * fma(r.y, vp, vq);
           }
         }
         __syncwarp();
@@ -269,50 +291,85 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
     const int nlog0 = nlog;
     for (int r = 0; r < rounds; ++r) {
       int rot = 0;
-      for (int sl = tid; sl < npairs; sl += nthr) {
-        int c = sc;
-        if (sl != tid) {
-          c = 0;
-          while (poff[c + 1] <= sl) ++c;
-        }
-        const int mc = cbeg[c + 1] - cbeg[c], mp = mc + (mc & 1);
-        int rr = r;
-        while (rr >= mp - 1) rr -= mp - 1;
-        int lp, lq;
-        rr_pair(rr, sl - poff[c], mp, lp, lq);
-        const int p = mem[cbeg[c] + lp], q = lq < mc ? mem[cbeg[c] + lq] : -1;
-        double cr = 1.0, sr = 0.0;
+      double cr = 1.0, tr = 0.0, app = 0, apq = 0, aqq = 0, d = 0;
+      const short2 ij = next;
+      if (slot < npairs) {
+        const int p = ij.x, q = ij.y;
         if (q >= 0) {
-          const double apq = A[packed(p, q, n)], app = A[packed(p, p, n)], aqq = A[packed(q, q, n)];
+          apq = A[packed(p, q, n)];
+          app = A[packed(p, p, n)];
+          aqq = A[packed(q, q, n)];
           if (rotates(apq, app, aqq)) {
-            // the small rotation angle theta, tan 2 theta = 2 a_pq / (a_qq - a_pp): cos 2 theta = |d| / h >= 0,
-            // c = sqrt((1 + cos 2 theta) / 2), s = sin 2 theta / (2 c); two reciprocal square roots on the
-            // round's critical path
-            const double d = aqq - app, t = 2.0 * apq;
-            const double ih = rsqrt(fma(d, d, t * t));
-            const double u = fma(0.5 * fabs(d), ih, 0.5);
-            const double ic = rsqrt(u);
-            cr = u * ic;
-            sr = (d >= 0 ? apq : -apq) * ih * ic;
+            // tangent of the small rotation angle, t = 2 a_pq / (d + sign(d) sqrt(d^2 + 4 a_pq^2)), to FP32 accuracy
+            // (any t gives an orthogonal rotation; the entry left over, 2^-22 of a_pq, goes with the next sweep), and
+            // c = 1 / sqrt(1 + t^2) to FP64 accuracy from an FP32 start r (1 - x r^2 = e, |e| < 2^-20: the next
+            // term of the series is 5/16 e^3)
+            d = aqq - app;
+            const int ed = (__double2hiint(d) >> 20) & 0x7ff, eb = (__double2hiint(apq) >> 20) & 0x7ff;
+            float tf;
+            if (ed - eb > 60) {
+              tr = apq / d;                   // below FP32's range
+              tf = 0.0f;
+            } else {
+              const int em = max(ed, eb);     // largest magnitude to [1, 2)
+              const float fd = scaled_float(d, em), fb = 2.0f * scaled_float(apq, em);
+              tf = __fdividef(fb, fd + copysignf(__fsqrt_rn(fmaf(fd, fd, fb * fb)), fd));
+              tr = widen(tf);
+            }
+            const double x = fma(tr, tr, 1.0);
+            const double r0 = widen(rsqrtf(fmaf(tf, tf, 1.0f)));
+            const double e = fma(-x, r0 * r0, 1.0);
+            cr = fma(r0 * e, fma(e, 0.375, 0.5), r0);
             rot = 1;
           }
         }
-        cs[sl] = cr;
-        sn[sl] = sr;
-        pp[sl] = (short)p;
-        qq[sl] = (short)q;
-        log[(int64_t)nlog * npairs + sl] = make_double2(cr, sr);
+        ct[slot] = make_double2(cr, tr);
+        pq[slot] = ij;
+        log[(int64_t)nlog * npairs + slot] = make_double2(cr, tr);
+        logi[(int64_t)nlog * npairs + slot] = nonzero(tr) ? ij : make_short2(-1, -1);
       }
-      if (tid == 0) lround[nlog] = (unsigned char)r;
-      if (!__syncthreads_or(rot)) continue;   // nothing rotates in this round: its log entry is overwritten
+      const bool some = __syncthreads_or(rot);
+      if (slot < npairs) next = indices(r + 1 < rounds ? r + 1 : 0, slot - sp0, smc, smp, sb0);
+      if (!some) continue;   // nothing rotates in this round: its log entry is overwritten
       ++nlog;
-      // A <- J^T A J, one 2x2 block (pair P rows, pair Q columns) per thread iteration
+      // A <- J^T A J: the rotated pairs' own blocks by the threads that hold the pairs, the blocks between two
+      // pairs (P rows, Q columns) by the first threads
+      if (nonzero(tr)) {
+        // what is left of a_pq, r = (b (1 - t^2) - t (d - a)) c^2 (the difference keeps its error at 2^-52 of b), and
+        // a' = a - t (b + r), d' = d + t (b + r)
+        const double r = (cr * cr) * fma(-tr, tr * apq, fma(-tr, d, apq)), w = apq + r;
+        A[packed(ij.x, ij.x, n)] = fma(-tr, w, app);
+        A[packed(ij.y, ij.y, n)] = fma(tr, w, aqq);
+        A[packed(ij.x, ij.y, n)] = r;
+      }
+      if (ws == 2) {
+        if (tid - lane < 4 * nblk) {          // whole warps: the four threads of a block read before any writes
+          const uint32_t PQ = blk[min(tid >> 2, nblk - 1)];
+          const double2 r1 = ct[PQ >> 16], r2 = ct[PQ & 0xffffu];
+          const short2 i1 = pq[PQ >> 16], i2 = pq[PQ & 0xffffu];
+          const bool row = tid & 2, col = tid & 1;
+          const bool hq1 = i1.y >= 0, hq2 = i2.y >= 0;
+          const int p1 = i1.x, q1 = hq1 ? i1.y : p1, p2 = i2.x, q2 = hq2 ? i2.y : p2;
+          // own row first: u, the other one: w
+          const int ru = row ? q1 : p1, rw = row ? p1 : q1;
+          const double up = A[packed(ru, p2, n)], uq = A[packed(ru, q2, n)];
+          const double wp = hq1 ? A[packed(rw, p2, n)] : 0.0, wq = hq1 ? A[packed(rw, q2, n)] : 0.0;
+          const double t1 = row ? r1.y : -r1.y, k = r1.x * r2.x;
+          const double rp = fma(t1, wp, up), rq = hq2 ? fma(t1, wq, uq) : 0.0;
+          const double v = k * (col ? fma(r2.y, rp, rq) : fma(-r2.y, rq, rp));
+          __syncwarp();
+          if (tid < 4 * nblk && (!row || hq1) && (!col || hq2)) A[packed(ru, col ? q2 : p2, n)] = v;
+        }
+        __syncthreads();
+        continue;
+      }
       for (int e = tid; e < nblk; e += nthr) {
         const uint32_t PQ = blk[e];
         const int P = (int)(PQ >> 16), Q = (int)(PQ & 0xffffu);
-        const double c1 = cs[P], s1 = sn[P], c2 = cs[Q], s2 = sn[Q];
-        if (s1 == 0.0 && s2 == 0.0) continue;
-        const int p1 = pp[P], q1 = qq[P], p2 = pp[Q], q2 = qq[Q];
+        const double2 r1 = ct[P], r2 = ct[Q];
+        if (!nonzero(r1.y) && !nonzero(r2.y)) continue;
+        const short2 i1 = pq[P], i2 = pq[Q];
+        const int p1 = i1.x, q1 = i1.y, p2 = i2.x, q2 = i2.y;
         const bool hq1 = q1 >= 0, hq2 = q2 >= 0;
         const int ia = packed(p1, p2, n), ib = packed(p1, hq2 ? q2 : p2, n);
         const int ic = packed(hq1 ? q1 : p1, p2, n), id = packed(hq1 ? q1 : p1, hq2 ? q2 : p2, n);
@@ -320,13 +377,12 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
         const double b = hq2 ? A[ib] : 0.0;
         const double cc = hq1 ? A[ic] : 0.0;
         const double d = (hq1 && hq2) ? A[id] : 0.0;
-        // rows
-        const double ra = c1 * a - s1 * cc, rb = c1 * b - s1 * d;
-        const double rc = s1 * a + c1 * cc, rd = s1 * b + c1 * d;
-        // columns
-        const double na = c2 * ra - s2 * rb, nd = s2 * rc + c2 * rd;
-        double nb = s2 * ra + c2 * rb, nc2 = c2 * rc - s2 * rd;
-        if (P == Q) nb = nc2 = 0.0;           // the rotated pair (s1 != 0 here)
+        const double t1 = r1.y, t2 = r2.y, k = r1.x * r2.x;
+        // rows, then columns, without the cosines
+        const double ra = fma(-t1, cc, a), rb = fma(-t1, d, b);
+        const double rc = fma(t1, a, cc), rd = fma(t1, b, d);
+        const double na = k * fma(-t2, rb, ra), nd = k * fma(t2, rc, rd);
+        const double nb = k * fma(t2, ra, rb), nc2 = k * fma(-t2, rd, rc);
         A[ia] = na;
         if (hq2) A[ib] = nb;
         if (hq1) A[ic] = nc2;
@@ -337,9 +393,11 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
     if (nlog == nlog0) break;                 // nothing rotated
     // converged when no pair of a component would rotate
     int more = 0;
-    for (int e = tid; e < n * n; e += nthr) {
-      const int i = e / n, j = e - i * n;
-      if (i < j && cnum[i] == cnum[j]) more |= rotates(A[packed(i, j, n)], A[packed(i, i, n)], A[packed(j, j, n)]);
+    for (int i = tid >> 5; i < n; i += nthr >> 5) {
+      const int row = packed(i, i, n) - i;
+      const double aii = A[row + i];
+      for (int j = i + 1 + lane; j < n; j += 32)
+        if (cnum[i] == cnum[j]) more |= rotates(A[row + j], aii, A[packed(j, j, n)]);
     }
     if (!__syncthreads_or(more)) {
       ++sweep;                                // a further sweep would find nothing to rotate
@@ -349,19 +407,22 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
   if (tid == 0 && sweep >= max_sweeps && n > 1) atomicAdd(&status[kStNoConv], 1);
 
   // ---- sort descending (rank = number of larger eigenvalues, ties by index)
-  for (int i = tid; i < n; i += nthr) nrm[i] = A[packed(i, i, n)] * down;
+  // ranked by (value, index) as integers in the order of the values, a NaN as the lowest: a strict total order, so
+  // perm is a permutation whatever the input (a non-finite tensor is reported by the normalisation)
+  for (int i = tid; i < n; i += nthr) {
+    const double v = A[packed(i, i, n)] * down;
+    const long long b = __double_as_longlong(v);
+    nrmv[i] = v;
+    key[i] = (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll ? (long long)0x8000000000000000ull
+                                                               : (b < 0 ? (long long)0x8000000000000000ull - b : b);
+  }
   __syncthreads();
   for (int i = tid; i < n; i += nthr) {
-    // ranked by (value, index) with a NaN taken as -inf: a strict total order, so perm is a
-    // permutation whatever the input (a non-finite tensor is reported by the normalisation)
-    const double li = nrm[i], ki = li == li ? li : -INFINITY;
+    const long long ki = key[i];
     int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      const double lj = nrm[j], kj = lj == lj ? lj : -INFINITY;
-      rank += (kj > ki) || (kj == ki && j < i);
-    }
+    for (int j = 0; j < n; ++j) rank += key[j] > ki || (key[j] == ki && j < i);
     perm[rank] = i;
-    lam[rank] = li;
+    lam[rank] = nrmv[i];
   }
   __syncthreads();
   for (int i = tid; i < n; i += nthr) jb.lam[i] = lam[i];
@@ -378,11 +439,12 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
       cstart[k] = j;
     }
   }
-  // the discarded sum, in decreasing order
-  if (tid == 0) {
+  // the discarded sum: each lane of the first warp its share, then pairwise
+  if (tid < 32) {
     double e = 0;
-    for (int j = chi; j < n; ++j) e += lam[j];
-    *jb.eps = e;
+    for (int j = chi + lane; j < n; j += 32) e += lam[j];
+    for (int off = 16; off > 0; off >>= 1) e += __shfl_xor_sync(0xffffffffu, e, off);
+    if (tid == 0) *jb.eps = e;
   }
   __syncthreads();
   // columns needed: every member of a cluster that starts below chi
@@ -403,46 +465,51 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
       const bool live = gid < par && k < nw;
       double* w = dyn + (int64_t)(live ? gid : 0) * n;
       const int col = live ? perm[k] : 0, c = cnum[col];
-      const int mc = cbeg[c + 1] - cbeg[c], mp = mc + (mc & 1), np = mp / 2, p0 = poff[c], b0 = cbeg[c];
+      const int np = (cbeg[c + 1] - cbeg[c] + 1) / 2, p0 = poff[c];
       if (live)
         for (int j = lg; j < n; j += gsz) w[j] = j == col ? 1.0 : 0.0;
       __syncwarp();
-      auto apply = [&](int l, int sl, double2 r) {
-        int rr = lround[l];
-        while (rr >= mp - 1) rr -= mp - 1;
-        int lp, lq;
-        rr_pair(rr, sl, mp, lp, lq);
-        if (lq < mc && r.y != 0.0) {
-          const int p = mem[b0 + lp], q = mem[b0 + lq];
-          const double wp = w[p], wq = w[q];
-          w[p] = r.x * wp + r.y * wq;
-          w[q] = r.x * wq - r.y * wp;
+      auto apply = [&](short2 i, double2 r) {
+        if (i.y >= 0) {
+          const double wp = w[i.x], wq = w[i.y];
+          w[i.x] = r.x * fma(r.y, wq, wp);
+          w[i.y] = r.x * fma(-r.y, wp, wq);
         }
       };
       if (one) {
+        // four entries ahead: their rotations and indices are read before the column's own chain needs them
         const bool act = live && lg < np;
-        const double2* lp0 = log + p0 + lg;
-        double2 nx[4];
+        const double2* lr = log + p0 + lg;
+        const short2* li = logi + p0 + lg;
+        double2 nr[4];
+        short2 ni[4];
+        auto fetch = [&](int l, int u) {
+          const bool in = act && l >= 0;
+          ni[u] = in ? li[(int64_t)l * npairs] : make_short2(-1, -1);
+          nr[u] = in ? lr[(int64_t)l * npairs] : make_double2(1.0, 0.0);
+        };
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          nx[u] = act && nlog - 1 - u >= 0 ? lp0[(int64_t)(nlog - 1 - u) * npairs] : make_double2(1.0, 0.0);
+        for (int u = 0; u < 4; ++u) fetch(nlog - 1 - u, u);
         for (int l = nlog - 1; l >= 0; l -= 4) {
-          double2 cur[4];
+          double2 r[4];
+          short2 ij[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            cur[u] = nx[u];
-            nx[u] = act && l - 4 - u >= 0 ? lp0[(int64_t)(l - 4 - u) * npairs] : make_double2(1.0, 0.0);
+            r[u] = nr[u];
+            ij[u] = ni[u];
+            fetch(l - 4 - u, u);
           }
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            if (act && l - u >= 0) apply(l - u, lg, cur[u]);
+            apply(ij[u], r[u]);
             __syncwarp();
           }
         }
       } else {
         for (int l = nlog - 1; l >= 0; --l) {
           if (live)
-            for (int sl = lg; sl < np; sl += gsz) apply(l, sl, log[(int64_t)l * npairs + p0 + sl]);
+            for (int sl = lg; sl < np; sl += gsz)
+              apply(logi[(int64_t)l * npairs + p0 + sl], log[(int64_t)l * npairs + p0 + sl]);
           __syncwarp();
         }
       }
@@ -545,8 +612,7 @@ JacobiSmem jacobi_smem(int nmax) {
   const int cols = (kJT / 32) * nmax;          // 17 columns in progress
   JacobiSmem s;
   s.region = nmax <= kJacobiSmemN ? (int)packed_doubles(nmax) : cols;
-  // blocks: at most one more than a connected matrix has (components of n - 1 and 1), or one per index
-  const int blocks = np * (np + 1) / 2 + 1 > nmax ? np * (np + 1) / 2 + 1 : nmax;
+  const int blocks = np * (np - 1) / 2 + 1;    // of a connected matrix: components have fewer in all
   s.bytes = (size_t)s.region * sizeof(double) + (size_t)blocks * sizeof(uint32_t);
   return s;
 }
@@ -571,9 +637,9 @@ cudaError_t launch_jacobi(const EigPack& jobs, int njobs, int nmax, double clust
   const JacobiSmem sm = jacobi_smem(nmax);
   const cudaError_t e = jacobi_attr_for_current_device();
   if (e != cudaSuccess) return e;
-  // a thread per 2x2 block of a connected matrix, up to kJT
-  const int np = (nmax + 1) / 2, want = (np * (np + 1) / 2 + 31) / 32 * 32;
-  const int threads = want < 64 ? 64 : (want > kJT ? kJT : want);
+  // a thread per 2x2 block of a connected matrix, up to kJT: whole warps of blocks between pairs and of pairs
+  const int np = (nmax + 1) / 2, want = (np * (np - 1) / 2 + 31) / 32 * 32 + (np + 31) / 32 * 32;
+  const int threads = want < 192 ? 192 : (want > kJT ? kJT : want);   // at least nmax: np^2 / 2 + 32 > 2 np from 192 on
   jacobi_kernel<<<njobs * jobs.batch, threads, sm.bytes, st>>>(jobs, njobs, nmax <= kJacobiSmemN ? 1 : 0, sm.region,
                                                               cluster_tau, tie_rel, max_sweeps, status);
   return cudaGetLastError();
