@@ -2,8 +2,8 @@
 //
 // C[m][n] = alpha * sum_k A[m*lda + k] B[n*ldb + k] + beta * C[m*ldc + n]: both operands
 // K-major (the layout the block-spin contraction builds, the same one the tensor-core
-// path consumes). 128x64 output tile per CTA, 256 threads with an 8x4 register tile,
-// 16-wide k slices staged in shared memory. FP64 mode uses DFMA; FP32 mode FFMA with FP32
+// path consumes). 128x64 output tile per CTA (64x32 where that leaves SMs idle), 256 threads
+// with an 8x4 (4x2) register tile, 16-wide k slices staged in shared memory. FP64 mode uses DFMA; FP32 mode FFMA with FP32
 // accumulation. Ragged M, N and K edges are guarded.
 #include <type_traits>
 
@@ -99,9 +99,9 @@ template <typename R>
 cudaError_t launch_gemm_simt(const R* A, int64_t lda, const R* B, int64_t ldb, R* C, int64_t ldc, int64_t M,
                              int64_t N, int64_t K, double alpha, double beta, cudaStream_t st, const OneProduct& one) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  // Tiles of 128 x 64 keep 32 products per 12 operand reads; where they leave SMs without work (two tiles per
-  // SM), 64 x 32 ones spread the FP64 pipe's load: at D = 4 the two 512 x 512 x 512 sector blocks are 64 large
-  // tiles for 152 SMs (1088 us) or 256 small ones (see the figure at the end of this comment's kernel list).
+  // Tiles of 128 x 64 do 32 products per 12 operand reads; below two of them per SM, 64 x 32 tiles share the FP64
+  // pipe's load more evenly: at D = 4 the two 512 x 512 x 512 sector blocks are 64 large tiles for 152 SMs
+  // (1088 us) or 256 small ones (779 us; the pipe's floor is 430).
   auto go = [&](auto tm, auto tn) -> cudaError_t {
     constexpr int TM = decltype(tm)::value, TN = decltype(tn)::value;
     const int64_t more = one.sec.tab.base ? 1 : 0;   // two sectors: at most one more tile row
