@@ -200,8 +200,8 @@ hotrg_status hotrg_step_flops(const hotrg_ctx* ctx, int dir, int dcut, double* m
 /* Tuning and test options of a context (host-side; take effect from the next step).
  * HOTRG_OPT_JACOBI_SWEEPS: sweep limit of the eigensolver, 1..60 (default 60); reaching it
  *   raises HOTRG_ENOCONV at the next synchronising call (used to test that path).
- * HOTRG_OPT_GEMM_VARIANT: tensor-core GEMM pipeline. TF32X3: 0 = 4 stages of 16-wide
- *   k-blocks (default), 1 = 2 stages of 32-wide k-blocks. FP16X3: 0 = partial sums promoted
+ * HOTRG_OPT_GEMM_VARIANT: tensor-core GEMM pipeline. TF32X3: 0 = each 256 x 256
+ *   tile computed by a pair of CTAs on two SMs (default), 1 = one CTA per 128 x 256 tile. FP16X3: 0 = partial sums promoted
  *   from the tensor-core accumulator to FP32 registers every 128 k, each 256 x 256 tile
  *   computed by a pair of CTAs on two SMs (tcgen05.mma.cta_group::2; each CTA loads half of
  *   the B tile) (default); 1 = every 64 k (slower, a smaller truncation bias), 2 = every
@@ -250,7 +250,7 @@ hotrg_status hotrg_set_option(hotrg_ctx* ctx, int option, int value);
  * closing direction (the transverse direction whose isometries are applied last; it sets
  * the shapes of the half contractions and of the block-spin GEMM, Sec. 2) and, in the
  * tensor-core modes, each pipeline that gives the same products (FP16X3: CTA pairs or one
- * CTA per tile; TF32X3: 16- or 32-wide k-blocks). The fastest (ties to the planner's
+ * CTA per tile, TF32X3 too). The fastest (ties to the planner's
  * choice) is cached for this device and step shape (bond dimensions, direction, cut,
  * precision, batch, tensors, workspace size) for the life of the process and used by
  * every context with HOTRG_OPT_AUTOTUNE set. The run does not advance: the current

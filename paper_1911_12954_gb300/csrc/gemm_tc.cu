@@ -105,6 +105,7 @@ using CfgF16 = Cfg<64, true, 128>;      // fp16: 4 stages of 32-wide k-blocks, 1
 using CfgF16S = Cfg<64, true, 64>;      // fp16 with 64-k chunks
 using CfgF16L = Cfg<64, true, 256>;     // fp16 with 256-k chunks
 using CfgF16P = Cfg<128, true, 128, true>;  // fp16, CTA pairs, 3 stages of 64 KB, 128-k chunks
+using CfgTF32P = Cfg<128, false, 32, true>; // tf32, CTA pairs, 3 stages of 64 KB, 32-k chunks
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -232,7 +233,14 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
 
 template <class CF>
 __device__ __forceinline__ void mma(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t accumulate) {
-  if constexpr (CF::kPair) {
+  if constexpr (CF::kPair && !CF::kF16) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
+        "l"(a), "l"(b), "r"(CF::IDESC), "r"(accumulate)
+        : "memory");
+  } else if constexpr (CF::kPair) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
@@ -589,7 +597,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                      const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo,
                      const __grid_constant__ GemmGroup grp, int64_t ldc, int M, int N, int Kp, int P,
                      int* status) {
-  static_assert(CF::kPair && CF::kF16, "pair kernel: fp16 pair configuration");
+  static_assert(CF::kPair, "pair kernel: pair configuration");
   constexpr int STAGES = CF::STAGES, BK = CF::BK, A_BYTES = CF::A_BYTES, B_BYTES = CF::B_BYTES,
                 STAGE_BYTES = CF::STAGE_BYTES, KPC = CF::KB_PER_CHUNK;
   extern __shared__ uint8_t smem_raw[];
@@ -1108,8 +1116,11 @@ const DeviceSetup* device_setup() {
     return nullptr;
   }
   int n = 0;
+  static_assert(CfgF16P::SMEM_BYTES == CfgTF32P::SMEM_BYTES, "one pair grid for both");
   if (smem_ok(gemm_pair_kernel<CfgF16P, false>, CfgF16P::SMEM_BYTES) &&
-      smem_ok(gemm_pair_kernel<CfgF16P, true>, CfgF16P::SMEM_BYTES)) {
+      smem_ok(gemm_pair_kernel<CfgF16P, true>, CfgF16P::SMEM_BYTES) &&
+      smem_ok(gemm_pair_kernel<CfgTF32P, false>, CfgTF32P::SMEM_BYTES) &&
+      smem_ok(gemm_pair_kernel<CfgTF32P, true>, CfgTF32P::SMEM_BYTES)) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1145,10 +1156,10 @@ cudaError_t launch_single(const void* Ahi, const void* Alo, const void* Bhi, con
   return cudaGetLastError();
 }
 
+template <class CF>
 cudaError_t launch_pair(const void* Ahi, const void* Alo, const void* Bhi, const void* Blo, int64_t W, int64_t aws,
                         int64_t bws, int64_t Kp, int64_t kps, int64_t P, int64_t M, int64_t N, int64_t ldc,
                         const GemmGroup& g, int* status, cudaStream_t st, const DeviceSetup& dv) {
-  using CF = CfgF16P;
   CUtensorMap mAhi, mAlo, mBhi, mBlo;
   // each CTA copies its own 128 rows of A and its own 128-row half of the B tile
   if (!make_map<CF>(&mAhi, Ahi, M, Kp, kps, P, W, aws, BM) || !make_map<CF>(&mAlo, Alo, M, Kp, kps, P, W, aws, BM) ||
@@ -1185,7 +1196,9 @@ cudaError_t launch_pair(const void* Ahi, const void* Alo, const void* Bhi, const
 // swizzle, 2 stages; 2: fp16 operands (hi/lo planes of __half), k-blocks of 32, 64-byte
 // swizzle, 4 stages, 128-k promotion chunks (kps % 8 == 0); 3: as 2 with 64-k chunks; 4: as
 // 2 with 256-k chunks; 5: fp16 in CTA pairs (tcgen05.mma.cta_group::2, 256 x 256 tiles),
-// k-blocks of 64 (kps % 64 == 0), 128-k chunks.
+// k-blocks of 64 (kps % 64 == 0), 128-k chunks; 6: tf32 in CTA pairs, k-blocks of 32 (kps % 32 == 0), 32-k chunks
+// (with 64-byte rows one CTA fetches 49 KB per 16 k, more than L2 delivers to 152 SMs at the MMA rate; a pair
+// fetches a third less).
 cudaError_t launch_gemm_group(const void* Ahi, const void* Alo, const void* Bhi, const void* Blo, int W, int64_t aws,
                               int64_t bws, int64_t Kp, int64_t kps, int64_t P, int64_t M, int64_t N, int64_t ldc,
                               const GemmGroup& g, int* status, cudaStream_t st, int variant) {
@@ -1204,14 +1217,16 @@ cudaError_t launch_gemm_group(const void* Ahi, const void* Alo, const void* Bhi,
     return cudaErrorInvalidValue;
   if (g.sec.tab.base) Kp = kps;   // packed summed indices fill whole panel rows, k-blocks run over the padding
   const bool f16 = variant >= 2 && variant <= 5;
-  if ((kps & (variant == 5 ? 63 : (f16 ? 7 : 3))) || kps < Kp) return cudaErrorInvalidValue;
+  if ((kps & (variant == 5 ? 63 : (variant == 6 ? 31 : (f16 ? 7 : 3)))) || kps < Kp) return cudaErrorInvalidValue;
   if ((((uintptr_t)Ahi) | ((uintptr_t)Alo) | ((uintptr_t)Bhi) | ((uintptr_t)Blo)) & 15) return cudaErrorInvalidValue;
   const DeviceSetup* dv = device_setup();
   if (!dv) return cudaErrorInitializationError;
+  if (variant == 6 && dv->pair_grid >= 2)
+    return launch_pair<CfgTF32P>(Ahi, Alo, Bhi, Blo, W, aws, bws, Kp, kps, P, M, N, ldc, g, status, st, *dv);
   if (variant == 5) {
     // a device (or partition) that cannot co-schedule two-CTA clusters runs the same
     // products on single CTAs
-    if (dv->pair_grid >= 2) return launch_pair(Ahi, Alo, Bhi, Blo, W, aws, bws, Kp, kps, P, M, N, ldc, g, status, st, *dv);
+    if (dv->pair_grid >= 2) return launch_pair<CfgF16P>(Ahi, Alo, Bhi, Blo, W, aws, bws, Kp, kps, P, M, N, ldc, g, status, st, *dv);
     return launch_single<CfgF16>(Ahi, Alo, Bhi, Blo, W, aws, bws, Kp, kps, P, M, N, ldc, g, status, st, *dv);
   }
   if (variant == 4) return launch_single<CfgF16L>(Ahi, Alo, Bhi, Blo, W, aws, bws, Kp, kps, P, M, N, ldc, g, status, st, *dv);

@@ -891,6 +891,8 @@ hotrg_status gemm_simt(hotrg_ctx* ctx, const R* A, const R* B, const StepPlan& p
 // 128-k promotion chunks; 1 = one CTA, 64-k chunks; 2 = one CTA, 256-k chunks; 3 = one CTA,
 // 128-k chunks.
 constexpr int kF16Variant[4] = {5, 3, 4, 2};
+// TF32X3: 0 = CTA pairs, 32-wide k-blocks; 1 = one CTA, 32-wide k-blocks.
+constexpr int kTF32Variant[2] = {6, 1};
 
 // Tensor-core modes: every output of the group in one launch. The W operand tensors of a
 // plane start Asz / Bsz operand elements apart.
@@ -901,7 +903,7 @@ hotrg_status gemm_tc(hotrg_ctx* ctx, const void* A, const void* Alo, const void*
   hotrg_status r = tm.start();
   if (r != HOTRG_OK) return r;
   const int opt = p.gemm_opt >= 0 ? p.gemm_opt : ctx->gemm_variant;
-  const int variant = ctx->prec == HOTRG_FP16X3 ? kF16Variant[opt] : opt;
+  const int variant = ctx->prec == HOTRG_FP16X3 ? kF16Variant[opt] : kTF32Variant[opt];
   CK(launch_gemm_group(A, Alo, B, Blo, W, Asz, Bsz, p.Kp, p.kps, p.P, M, N, N, g, (int*)(ctx->ws + ctx->L.status),
                        st, variant),
      ctx->prec == HOTRG_FP16X3 ? "gemm f16x3" : "gemm tf32x3");
@@ -1406,7 +1408,7 @@ bool plan_slices(const hotrg_ctx* ctx, StepPlan& p) {
 // the GPU and the fastest is kept, per device and step shape: the closing direction c (which
 // transverse direction the last two isometry passes close; it fixes the shapes of the half
 // contractions and of the GEMM) and the tensor-core pipeline (FP16X3: CTA pairs or single
-// CTAs, which give bit-identical products; TF32X3: 16- or 32-wide k-blocks). The promotion
+// CTAs, which give bit-identical products; TF32X3: CTA pairs or single CTAs). The promotion
 // chunk changes the truncation bias of the tensor-core accumulator, so it is not a candidate.
 struct TuneChoice {
   int c;
