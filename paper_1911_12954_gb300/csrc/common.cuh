@@ -253,7 +253,9 @@ template <typename R>
 cudaError_t launch_gram(const GramPack& jobs, int njobs, int Rmax, int nchunks, cudaStream_t st);
 cudaError_t launch_gram_reduce(const GramPack& jobs, int njobs, int nchunks, int64_t RRmax, int64_t out_stride,
                                double* out, cudaStream_t st);
-cudaError_t launch_gram_merge(const double* A1, const double* A2, int Dn, int Dk, double* G,
+// `count` Gram matrices of one direction: matrix y from the halves at half + 2 y RRs and half + (2 y + 1) RRs, to
+// G + y nn.
+cudaError_t launch_gram_merge(const double* half, int64_t RRs, int Dn, int Dk, double* G, int64_t nn, int count,
                               cudaStream_t st);
 // The six Gram matrices (3 transverse directions x 2 sides) of each of `batch` elements in
 // one launch: half-Grams at half[((b * 12) + (i * 2 + side) * 2 + h) * RRs] (h = 0: k on

@@ -425,8 +425,12 @@ cudaError_t launch_gram_reduce(const GramPack& jobs, int njobs, int nchunks, int
 }
 
 // G[(a1 a2),(b1 b2)] = sum_{k,k'} A1[(a1,k),(b1,k')] A2[(a2,k),(b2,k')], FP64.
-__global__ void gram_merge_kernel(const double* __restrict__ A1, const double* __restrict__ A2, int Dn, int Dk,
-                                  double* __restrict__ G) {
+// blockIdx.y: the matrix, its halves at half[2 y RRs] and half[(2 y + 1) RRs].
+__global__ void gram_merge_kernel(const double* __restrict__ half, int64_t RRs, int Dn, int Dk, double* __restrict__ G,
+                                  int64_t nn) {
+  const double* A1 = half + 2 * blockIdx.y * RRs;
+  const double* A2 = A1 + RRs;
+  G += blockIdx.y * nn;
   const int n = Dn * Dn;
   const int Rk = Dn * Dk;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * n; e += gridDim.x * blockDim.x) {
@@ -440,9 +444,10 @@ __global__ void gram_merge_kernel(const double* __restrict__ A1, const double* _
   }
 }
 
-cudaError_t launch_gram_merge(const double* A1, const double* A2, int Dn, int Dk, double* G, cudaStream_t st) {
+cudaError_t launch_gram_merge(const double* half, int64_t RRs, int Dn, int Dk, double* G, int64_t nn, int count,
+                              cudaStream_t st) {
   const int n2 = Dn * Dn * Dn * Dn;
-  gram_merge_kernel<<<(n2 + 255) / 256, 256, 0, st>>>(A1, A2, Dn, Dk, G);
+  gram_merge_kernel<<<dim3((n2 + 127) / 128, count), 128, 0, st>>>(half, RRs, Dn, Dk, G, nn);
   return cudaGetLastError();
 }
 

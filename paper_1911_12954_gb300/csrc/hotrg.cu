@@ -338,9 +338,12 @@ StepPlan make_plan(const int D[4], int mu, int dcut, int prec, int batch = 1, in
     }
   }
   const int64_t Kg = p.E / p.Rmax;
-  // split-K chunks of the half-Grams: two CTAs per SM in all (a chunk's set-up, decoding and reduction
-  // cost a few microseconds), of at least 64 summed indices
-  int64_t nc = std::min(2 * 150 * 2 / (12 * (int64_t)batch), (Kg + 63) / 64);
+  // split-K chunks of the half-Grams: one wave of CTAs (two per SM for FP32 tensors, one for FP64), because a
+  // chunk's set-up, decoding and reduction cost a few microseconds (D_cut = 4: 59 -> 38 us against two waves,
+  // FP64 133 -> 41); two waves where chunks are long enough to hide that (D = 8: 804 -> 690); at least 64 summed indices
+  int64_t nc = (f64_store(prec) ? 150 : 300) / (12 * (int64_t)batch);
+  if (nc > 0 && Kg / nc > 8192) nc *= 2;
+  nc = std::min(nc, (Kg + 63) / 64);
   if (nc < 1) nc = 1;
   // keep the split-K partials of all batch elements under 256 MB
   const int64_t per = (int64_t)batch * kMaxGramJobs * p.Rmax * p.Rmax * 8;

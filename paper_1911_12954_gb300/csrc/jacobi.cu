@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(256) select_kernel(const __grid_constant__ Sel
       double q = 0;
       for (int r = lane; r < n; r += 32) q = fma(uj[r], uj[r], q);
       for (int off = 16; off > 0; off >>= 1) q += __shfl_xor_sync(0xffffffffu, q, off);
-      const double inv = 1.0 / sqrt(q);
+      const double inv = rsqrt(q);
       for (int r = lane; r < n; r += 32) uj[r] *= inv;
     }
     __syncthreads();

@@ -157,11 +157,8 @@ extern "C" hotrg_status hotrg_isometry_noalloc(const double* T_dev, const int di
   NA_CK(launch_gram<double>(gp, 4, R, (int)nch, st), "gram");
   NA_CK(launch_gram_reduce(gp, 4, (int)nch, (int64_t)R * R, (int64_t)kNoAllocR * kNoAllocR, half, st), "gram reduce");
   double* G = (double*)(base + L.G);
-  for (int side = 0; side < 2; ++side)
-    NA_CK(launch_gram_merge(half + (int64_t)(side * 2) * kNoAllocR * kNoAllocR,
-                            half + (int64_t)(side * 2 + 1) * kNoAllocR * kNoAllocR, Dn, Dm,
-                            G + (int64_t)side * kNoAllocN * kNoAllocN, st),
-          "gram merge");
+  NA_CK(launch_gram_merge(half, (int64_t)kNoAllocR * kNoAllocR, Dn, Dm, G, (int64_t)kNoAllocN * kNoAllocN, 2, st),
+        "gram merge");
   EigPack ep{};
   for (int side = 0; side < 2; ++side) {
     EigJob& j = ep.j[side];

@@ -688,27 +688,70 @@ template cudaError_t launch_init<float>(const double*, const double*, float*, fl
                                         int, cudaStream_t);
 
 // ---------------------------------------------------------------------------- norm
-// Pass 1: each block writes the FP64 sum of squares of its grid-stride share.
+// Pass 1: each block writes the sum of squares of its grid-stride share, to FP64 accuracy. FP32 entries are
+// squared and summed as pairs of floats (x^2 = p + e exactly, hi + lo += p + e by TwoSum: the pair's own rounding
+// stays near 2^-48), because a conversion and an FMA per entry on the FP64 pipe cost more than reading the tensor
+// (D = 8: 67 us against 10).
 constexpr int kNormBlocks = kNormPartials;
+
+template <typename R>
+struct SumSq {
+  double s;
+  __device__ __forceinline__ void add(R x) { s = fma(x, x, s); }
+  __device__ __forceinline__ void merge(const SumSq& o) { s += o.s; }
+  __device__ __forceinline__ SumSq down(int off) const {
+    SumSq o;
+    o.s = __shfl_down_sync(0xffffffffu, s, off);
+    return o;
+  }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct SumSq<float> {
+  float hi, lo;
+  __device__ __forceinline__ void add(float x) {
+    const float p = x * x;
+    plus(p, fmaf(x, x, -p));
+  }
+  __device__ __forceinline__ void plus(float p, float e) {
+    const float t = hi + p, bp = t - hi;
+    lo += ((hi - (t - bp)) + (p - bp)) + e;
+    hi = t;
+  }
+  __device__ __forceinline__ void merge(const SumSq& o) { plus(o.hi, o.lo); }
+  __device__ __forceinline__ SumSq down(int off) const {
+    SumSq o;
+    o.hi = __shfl_down_sync(0xffffffffu, hi, off);
+    o.lo = __shfl_down_sync(0xffffffffu, lo, off);
+    return o;
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
 
 template <typename R>
 __global__ void __launch_bounds__(256) sumsq_kernel(const R* __restrict__ x, int64_t n, int64_t xstride,
                                                     double* partial) {
   x += blockIdx.y * xstride;                   // batch element blockIdx.y
   partial += blockIdx.y * gridDim.x;
-  double acc = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double v = (double)x[i];
-    acc = fma(v, v, acc);
+  SumSq<R> sum[4] = {};                        // four entries in flight
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += 4 * step) {
+    R v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = i + u * step < n ? x[i + u * step] : (R)0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sum[u].add(v[u]);
   }
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  __shared__ double w[8];
-  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = acc;
+  sum[0].merge(sum[1]);
+  sum[2].merge(sum[3]);
+  sum[0].merge(sum[2]);
+  for (int off = 16; off > 0; off >>= 1) sum[0].merge(sum[0].down(off));
+  __shared__ SumSq<R> w[8];
+  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = sum[0];
   __syncthreads();
   if (threadIdx.x == 0) {
-    double s = 0;
-    for (int j = 0; j < 8; ++j) s += w[j];
-    partial[blockIdx.x] = s;
+    for (int j = 1; j < 8; ++j) sum[0].merge(w[j]);
+    partial[blockIdx.x] = sum[0].value();
   }
 }
 
