@@ -20,6 +20,7 @@
 
 #include <algorithm>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -100,6 +101,7 @@ struct hotrg_ctx {
   int last_Dold[4] = {0, 0, 0, 0};
   int last_mu = -1;
   std::vector<double> h_host;
+  std::vector<char> stage;     // host staging of set_tensor and copy_tensor (see HostStage)
   int jacobi_sweeps = kJacobiMaxSweeps;
   int gemm_variant = 0;
   bool use_graphs = false;
@@ -143,6 +145,23 @@ hotrg_status cuda_fail(hotrg_ctx* ctx, cudaError_t e, const char* where) {
   if (ctx) ctx->sticky = HOTRG_ECUDA;
   return HOTRG_ECUDA;
 }
+
+// Host staging of a tensor on its way to or from the device: the context keeps up to kStageKeep bytes between calls
+// (fresh pages for every call cost more than the copy), larger ones are given back at once.
+constexpr size_t kStageKeep = 64u << 20;
+struct HostStage {
+  std::unique_ptr<char[]> own;
+  char* p;
+  HostStage(hotrg_ctx* ctx, size_t bytes) {
+    if (bytes <= kStageKeep) {
+      if (ctx->stage.size() < bytes) ctx->stage.resize(bytes);
+      p = ctx->stage.data();
+    } else {
+      own.reset(new char[bytes]);
+      p = own.get();
+    }
+  }
+};
 
 #define CK(call, where)                                   \
   do {                                                    \
@@ -1717,9 +1736,13 @@ hotrg_status hotrg_set_tensor(hotrg_ctx* ctx, int b, const int dims[4], const do
   if (b > 0 && ctx->initialised)
     for (int n = 0; n < 4; ++n)
       if (dims[n] != ctx->dims[n]) return HOTRG_EINVAL;
-  double nrm2 = 0;
-  for (int64_t i = 0; i < E; ++i) nrm2 += T_host[i] * T_host[i];
-  const double c = sqrt(nrm2);
+  // eight running sums: one would wait for its own addition at every entry
+  double part[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  int64_t done = 0;
+  for (; done + 8 <= E; done += 8)
+    for (int j = 0; j < 8; ++j) part[j] += T_host[done + j] * T_host[done + j];
+  for (; done < E; ++done) part[0] += T_host[done] * T_host[done];
+  const double c = sqrt(((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7])));
   if (!(c > 0) || !isfinite(c)) return HOTRG_EINVAL;
   cudaStream_t st = ctx->stream;
   CK(cudaStreamSynchronize(st), "set_tensor sync");
@@ -1730,13 +1753,16 @@ hotrg_status hotrg_set_tensor(hotrg_ctx* ctx, int b, const int dims[4], const do
     ctx->cur = 0;
   }
   if (f64_store(ctx->prec)) {
-    std::vector<double> tmp(E);
+    HostStage stage(ctx, E * 8);
+    double* tmp = (double*)stage.p;
     for (int64_t i = 0; i < E; ++i) tmp[i] = T_host[i] / c;
-    CK(cudaMemcpy(tensor_ptr<double>(ctx, 0, ctx->cur, b), tmp.data(), E * 8, cudaMemcpyHostToDevice), "upload");
+    CK(cudaMemcpy(tensor_ptr<double>(ctx, 0, ctx->cur, b), tmp, E * 8, cudaMemcpyHostToDevice), "upload");
   } else {
-    std::vector<float> tmp(E);
-    for (int64_t i = 0; i < E; ++i) tmp[i] = (float)(T_host[i] / c);
-    CK(cudaMemcpy(tensor_ptr<float>(ctx, 0, ctx->cur, b), tmp.data(), E * 4, cudaMemcpyHostToDevice), "upload");
+    HostStage stage(ctx, E * 4);
+    float* tmp = (float*)stage.p;
+    const double inv = 1.0 / c;
+    for (int64_t i = 0; i < E; ++i) tmp[i] = (float)(T_host[i] * inv);
+    CK(cudaMemcpy(tensor_ptr<float>(ctx, 0, ctx->cur, b), tmp, E * 4, cudaMemcpyHostToDevice), "upload");
   }
   const double lc = log(c);
   CK(cudaMemcpy((double*)(ctx->ws + ctx->L.lnz) + b, &lc, 8, cudaMemcpyHostToDevice), "lnz");
@@ -1973,8 +1999,9 @@ hotrg_status hotrg_copy_tensor(hotrg_ctx* ctx, int which, int b, double* host, s
   if (f64_store(ctx->prec)) {
     CK(cudaMemcpy(host, tensor_ptr<double>(ctx, which, ctx->cur, b), E * 8, cudaMemcpyDeviceToHost), "copy");
   } else {
-    std::vector<float> tmp(E);
-    CK(cudaMemcpy(tmp.data(), tensor_ptr<float>(ctx, which, ctx->cur, b), E * 4, cudaMemcpyDeviceToHost), "copy");
+    HostStage stage(ctx, E * 4);
+    float* tmp = (float*)stage.p;
+    CK(cudaMemcpy(tmp, tensor_ptr<float>(ctx, which, ctx->cur, b), E * 4, cudaMemcpyDeviceToHost), "copy");
     for (int64_t i = 0; i < E; ++i) host[i] = tmp[i];
   }
   return HOTRG_OK;
