@@ -249,6 +249,21 @@ template <typename TI, typename TU, typename TO>
 cudaError_t launch_ttm(const TI* in, const TU* U, TO* out, TO* out_lo, const TTMArgs& a, int mode,
                        cudaStream_t st);
 
+// Independent passes of one kind (both operand sides, every tensor of a step), launched together where that is
+// possible; *launches: kernels issued.
+constexpr int kMaxPassJobs = 6;
+template <typename R>
+struct TTMJob {
+  const R* in;
+  const R* U;
+  R* out;
+  R* lo;
+  TTMArgs a;
+  int mode;
+};
+template <typename R>
+cudaError_t launch_ttm_jobs(const TTMJob<R>* jobs, int n, int* launches, cudaStream_t st);
+
 template <typename R>
 cudaError_t launch_gram(const GramPack& jobs, int njobs, int Rmax, int nchunks, cudaStream_t st);
 cudaError_t launch_gram_reduce(const GramPack& jobs, int njobs, int nchunks, int64_t RRmax, int64_t out_stride,
@@ -327,7 +342,6 @@ template <typename R>
 cudaError_t launch_norm(const R* x, int64_t n, int nb, int64_t xstride, double* partial, const int* step,
                         double* c_out, double* lnz_acc,
                         DevRecord* rec_b, int* status, cudaStream_t st);
-cudaError_t launch_step_end(int* step, cudaStream_t st);
 // Counts over one fp16 plane in K panels (nrows rows of kps values, the first Kp of each
 // read): out[0] += zero entries, out[1] += entries in fp16's subnormal range (nonzero, below
 // 2^-14), out[2] = max(out[2], bits of the largest magnitude).
@@ -340,7 +354,8 @@ cudaError_t launch_sector_stats(const void* plane, const SectorTab& tab, int ele
 void jacobi_prepare();
 void gemm_prepare();
 template <typename R>
-cudaError_t launch_scale(R* x, int64_t n, int nb, int64_t xstride, const double* c, cudaStream_t st);
+cudaError_t launch_scale(R* x, int64_t n, int nb, int64_t xstride, int nt, int64_t tstride, const double* c, int* step,
+                         cudaStream_t st);
 template <typename R>
 cudaError_t launch_trace(const R* T, int64_t slot, const int* dims, int batch, double* out, cudaStream_t st);
 template <typename R>
@@ -355,8 +370,15 @@ cudaError_t launch_gemm_simt(const R* A, int64_t lda, const R* B, int64_t ldb, R
 void sectors_prepare();
 cudaError_t launch_sector_tables(const SectorArgs& a, int ne, cudaStream_t st);
 template <typename R>
-cudaError_t launch_sector_operand(const R* in, const R* U, R* out, R* out_lo, const SectorOperand& a, int ne, int mode,
-                                  cudaStream_t st);
+struct SectorJobs {           // the second passes of a phase (blockIdx.z)
+  const R* in[kMaxPassJobs];
+  R* out[kMaxPassJobs];
+  R* lo[kMaxPassJobs];
+  SectorOperand a[kMaxPassJobs];
+  int n;
+};
+template <typename R>
+cudaError_t launch_sector_operand(const SectorJobs<R>& jobs, const R* U, int ne, int mode, cudaStream_t st);
 template <typename R>
 cudaError_t launch_sector_close(const R* C, const R* U, R* O3, R* T, const SectorClose& a, int ne, cudaStream_t st);
 

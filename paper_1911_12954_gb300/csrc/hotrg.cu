@@ -197,7 +197,7 @@ Extent ttm_extent(const TTMArgs& a) {
 thread_local int64_t g_lim_in = -1, g_lim_u = -1, g_lim_out = -1;  // elements available
 
 template <typename R>
-inline cudaError_t launch_ttm_r(const R* in, const R* U, R* out, R* lo, const TTMArgs& a, int mode, cudaStream_t st) {
+inline cudaError_t check_ttm(const R* U, const TTMArgs& a) {
   const Extent e = ttm_extent(a);
   for (int i = 0; i < a.rank; ++i)
     if (a.in_st[i] < 0 || a.u_st[i] < 0 || a.out_st[i] < 0) return cudaErrorInvalidValue;
@@ -210,8 +210,49 @@ inline cudaError_t launch_ttm_r(const R* in, const R* U, R* out, R* lo, const TT
     g_last_error = "TTM launch refused: batch stride shorter than one element's buffer";
     return cudaErrorInvalidValue;
   }
-  return launch_ttm<R, R, R>(in, U, out, lo, a, mode, st);
+  return cudaSuccess;
 }
+template <typename R>
+inline cudaError_t launch_ttm_r(const R* in, const R* U, R* out, R* lo, const TTMArgs& a, int mode, cudaStream_t st) {
+  const cudaError_t e = check_ttm(U, a);
+  return e == cudaSuccess ? launch_ttm<R, R, R>(in, U, out, lo, a, mode, st) : e;
+}
+
+// The passes of one phase of the operand builds, collected and then launched together.
+template <typename R>
+struct PassList {
+  std::vector<TTMJob<R>> ttm;
+  SectorJobs<R> sec{};
+  const R* sec_U = nullptr;
+  int sec_mode = kTTMStore;
+  cudaError_t add(const R* in, const R* U, R* out, R* lo, const TTMArgs& a, int mode) {
+    const cudaError_t e = check_ttm(U, a);
+    if (e == cudaSuccess) ttm.push_back(TTMJob<R>{in, U, out, lo, a, mode});
+    return e;
+  }
+  cudaError_t add(const R* in, const R* U, R* out, R* lo, const SectorOperand& a, int mode) {
+    if (sec.n == kMaxPassJobs || (sec.n > 0 && (U != sec_U || mode != sec_mode))) return cudaErrorInvalidValue;
+    sec.in[sec.n] = in;
+    sec.out[sec.n] = out;
+    sec.lo[sec.n] = lo;
+    sec.a[sec.n++] = a;
+    sec_U = U;
+    sec_mode = mode;
+    return cudaSuccess;
+  }
+  cudaError_t launch(int ne, int* launches, cudaStream_t st) {
+    *launches = 0;
+    if (!ttm.empty()) {
+      const cudaError_t e = launch_ttm_jobs<R>(ttm.data(), (int)ttm.size(), launches, st);
+      if (e != cudaSuccess) return e;
+    }
+    if (sec.n > 0) {
+      *launches += 1;
+      return launch_sector_operand<R>(sec, sec_U, ne, sec_mode, st);
+    }
+    return cudaSuccess;
+  }
+};
 
 // Per-element strides of a group of batch elements contracted together (element e of the
 // group at base + e * stride, in elements of each buffer's type; operand planes in operand
@@ -588,7 +629,7 @@ void operand_strides(const StepPlan& p, const std::vector<int64_t>& rn, int64_t 
 // U^b[b1, b2, Y]), 1: B (contracts b2' of U^b[b1', b2', Y']).
 template <typename R>
 hotrg_status sector_operand(hotrg_ctx* ctx, const StepPlan& p, int side, const R* Ub, int x0, int xs, const int64_t* os,
-                            R* O1, R* out, R* out_lo, cudaStream_t st, const ElemStrides& es, unsigned* amax,
+                            R* O1, R* out, R* out_lo, PassList<R>& list, const ElemStrides& es, unsigned* amax,
                             int amax_bs, int scale, int phases, const SectorTab& tab, int parity) {
   const int Db = p.D[p.b], Dc = p.D[p.c], Dm = p.D[p.mu], cb = p.chi[p.b];
   SectorOperand a{};
@@ -622,14 +663,14 @@ hotrg_status sector_operand(hotrg_ctx* ctx, const StepPlan& p, int side, const R
   a.amax_bs = amax_bs;
   const int mode = !out_lo ? kTTMStore : split_mode(ctx->prec);
   if ((phases & kPassMax) && amax && scale == kScaleExact)
-    LK(1, launch_sector_operand<R>(O1, Ub, out, out_lo, a, es.ne, kTTMMaxAbs, st), "sector operand max");
-  if (phases & kPass2) LK(1, launch_sector_operand<R>(O1, Ub, out, out_lo, a, es.ne, mode, st), "sector operand");
+    CK(list.add(O1, Ub, out, out_lo, a, kTTMMaxAbs), "sector operand max");
+  if (phases & kPass2) CK(list.add(O1, Ub, out, out_lo, a, mode), "sector operand");
   return HOTRG_OK;
 }
 
 template <typename R>
 hotrg_status build_A(hotrg_ctx* ctx, const StepPlan& p, const R* P, const R* Ua, const R* Ub, int x0, int xs,
-                     R* O1, R* A, R* Alo, cudaStream_t st, const ElemStrides& es, unsigned* amax, int amax_bs,
+                     R* O1, R* A, R* Alo, PassList<R>& list, const ElemStrides& es, unsigned* amax, int amax_bs,
                      int scale, int phases, const SectorTab& tab, int parity) {
   const int mu = p.mu, a = p.a, b = p.b, c = p.c;
   const int Da = p.D[a], Db = p.D[b], Dc = p.D[c], Dm = p.D[mu];
@@ -659,10 +700,11 @@ hotrg_status build_A(hotrg_ctx* ctx, const StepPlan& p, const R* P, const R* Ua,
       t.amax_mul = sqrtf((float)Db);
       t.amax_bs = amax_bs;
     }
-    if (phases & kPass1) LK(1, launch_ttm_r<R>(P, Ua + x0, O1, nullptr, t, bound ? kTTMStoreMax : kTTMStore, st), "ttm A1");
+    if (phases & kPass1) CK(list.add(P, Ua + x0, O1, nullptr, t, bound ? kTTMStoreMax : kTTMStore), "ttm A1");
   }
   // A[(X Y c1 c1' mu1), (a2 b2 a1' b1' k)] = sum_b1 U^b[b1, b2, Y] O1[X, b1, ...]
-  if (p.sect) return sector_operand<R>(ctx, p, 0, Ub, x0, xs, os.data(), O1, A, Alo, st, es, amax, amax_bs, scale, phases, tab, parity);
+  if (p.sect) return sector_operand<R>(ctx, p, 0, Ub, x0, xs, os.data(), O1, A, Alo, list, es, amax, amax_bs, scale,
+                                           phases, tab, parity);
   {
     int64_t o[10];
     operand_strides(p, {xs, cb, Dc, Dc, Dm}, o);
@@ -685,15 +727,15 @@ hotrg_status build_A(hotrg_ctx* ctx, const StepPlan& p, const R* P, const R* Ua,
     t.amax = amax;   // max-norm scaling (nullptr: none): the max pass writes it, the split reads it
     t.amax_bs = amax_bs;
     if ((phases & kPassMax) && amax && scale == kScaleExact)
-      LK(1, launch_ttm_r<R>(O1, Ub, A, Alo, t, kTTMMaxAbs, st), "ttm A max");
-    if (phases & kPass2) LK(1, launch_ttm_r<R>(O1, Ub, A, Alo, t, mode, st), "ttm A2");
+      CK(list.add(O1, Ub, A, Alo, t, kTTMMaxAbs), "ttm A max");
+    if (phases & kPass2) CK(list.add(O1, Ub, A, Alo, t, mode), "ttm A2");
   }
   return HOTRG_OK;
 }
 
 template <typename R>
 hotrg_status build_B(hotrg_ctx* ctx, const StepPlan& p, const R* Q, const R* Ua, const R* Ub, int x0, int xs,
-                     R* O1, R* B, R* Blo, cudaStream_t st, const ElemStrides& es, unsigned* amax, int amax_bs,
+                     R* O1, R* B, R* Blo, PassList<R>& list, const ElemStrides& es, unsigned* amax, int amax_bs,
                      int scale, int phases, const SectorTab& tab, int parity) {
   const int mu = p.mu, a = p.a, b = p.b, c = p.c;
   const int Da = p.D[a], Db = p.D[b], Dc = p.D[c], Dm = p.D[mu];
@@ -723,9 +765,10 @@ hotrg_status build_B(hotrg_ctx* ctx, const StepPlan& p, const R* Q, const R* Ua,
       t.amax_mul = sqrtf((float)Db);
       t.amax_bs = amax_bs;
     }
-    if (phases & kPass1) LK(1, launch_ttm_r<R>(Q, Ua + x0, O1, nullptr, t, bound ? kTTMStoreMax : kTTMStore, st), "ttm B1");
+    if (phases & kPass1) CK(list.add(Q, Ua + x0, O1, nullptr, t, bound ? kTTMStoreMax : kTTMStore), "ttm B1");
   }
-  if (p.sect) return sector_operand<R>(ctx, p, 1, Ub, x0, xs, os.data(), O1, B, Blo, st, es, amax, amax_bs, scale, phases, tab, parity);
+  if (p.sect) return sector_operand<R>(ctx, p, 1, Ub, x0, xs, os.data(), O1, B, Blo, list, es, amax, amax_bs, scale,
+                                           phases, tab, parity);
   {
     int64_t o[10];
     operand_strides(p, {xs, cb, Dc, Dc, Dm}, o);
@@ -748,8 +791,8 @@ hotrg_status build_B(hotrg_ctx* ctx, const StepPlan& p, const R* Q, const R* Ua,
     t.amax = amax;   // max-norm scaling (nullptr: none): the max pass writes it, the split reads it
     t.amax_bs = amax_bs;
     if ((phases & kPassMax) && amax && scale == kScaleExact)
-      LK(1, launch_ttm_r<R>(O1, Ub, B, Blo, t, kTTMMaxAbs, st), "ttm B max");
-    if (phases & kPass2) LK(1, launch_ttm_r<R>(O1, Ub, B, Blo, t, mode, st), "ttm B2");
+      CK(list.add(O1, Ub, B, Blo, t, kTTMMaxAbs), "ttm B max");
+    if (phases & kPass2) CK(list.add(O1, Ub, B, Blo, t, mode), "ttm B2");
   }
   return HOTRG_OK;
 }
@@ -1173,25 +1216,38 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
     const int parity[3] = {0, 1, 0};   // T, S (one sigma: odd), M (two)
     // Padding columns of a panel (kin >= Kp) are never read: the tensor maps stop at Kp and
     // the CUDA-core GEMM at K, so the operand buffers need no clearing.
-    // every tensor's first pass, then (exact scaling) the max pass of every tensor, then the
-    // second passes, which read the side's bound; the bound starts from zero before the
-    // passes that record it
-    auto clear_phase = [&](int ph) { return ph == (scale == kScaleBound ? kPass1 : kPassMax); };
-    auto buildB = [&](int x20, int xs2) -> hotrg_status {
+    // Phase by phase: every tensor's first pass, (exact scaling) its max pass, its second pass, which reads the side's
+    // bound; the bound starts from zero before the passes that record it. The passes of a phase, of both sides
+    // where neither is sliced, go out together.
+    auto build = [&](bool sideA, bool sideB, int x0, int xs, int x20, int xs2) -> hotrg_status {
       for (int ph : {kPass1, kPassMax, kPass2}) {
         if (ph == kPassMax && scale != kScaleExact) continue;
-        if (amaxB && clear_phase(ph)) CK(cudaMemsetAsync(amaxB, 0, ne * tw * sizeof(unsigned), st), "amax clear");
+        if (amaxA && ph == (scale == kScaleBound ? kPass1 : kPassMax)) {
+          if (sideA && sideB) CK(cudaMemsetAsync(amaxA, 0, 2 * (size_t)p.ne * tw * sizeof(unsigned), st), "amax clear");
+          else CK(cudaMemsetAsync(sideA ? amaxA : amaxB, 0, (size_t)ne * tw * sizeof(unsigned), st), "amax clear");
+        }
+        PassList<R> list;
         for (int w = 0; w < nbuild; ++w) {
-          hotrg_status s = build_B<R>(ctx, p, src[w], Ua, Ub, x20, xs2, O1B + w * O1Bsz, opnd(Bbuf, w * Bsz * planes),
-                                      opnd(Blob, w * Bsz * planes), st, esB, amaxB ? amaxB + (tw > 1 ? w : 0) : nullptr,
-                                      tw, scale, ph, tab, parity[w]);
+          hotrg_status s = HOTRG_OK;
+          if (sideB)
+            s = build_B<R>(ctx, p, src[w], Ua, Ub, x20, xs2, O1B + w * O1Bsz, opnd(Bbuf, w * Bsz * planes),
+                           opnd(Blob, w * Bsz * planes), list, esB, amaxB ? amaxB + (tw > 1 ? w : 0) : nullptr, tw, scale, ph,
+                           tab, parity[w]);
+          if (s == HOTRG_OK && sideA)
+            s = build_A<R>(ctx, p, src[w], Ua, Ub, x0, xs, O1A + w * O1Asz, opnd(Abuf, w * Asz * planes),
+                           opnd(Alob, w * Asz * planes), list, esA, amaxA ? amaxA + (tw > 1 ? w : 0) : nullptr, tw, scale, ph,
+                           tab, parity[w]);
           if (s != HOTRG_OK) return s;
         }
+        int launched = 0;
+        CK(list.launch(ne, &launched, st), "operand passes");
+        ctx->launches += launched;
       }
       return HOTRG_OK;
     };
+    const bool whole = p.xs >= ca && p.xs2 >= ca;   // neither side sliced
     if (!b_sliced && pr.ttm) {
-      hotrg_status s = buildB(0, ca);
+      hotrg_status s = build(whole, true, 0, ca, 0, ca);
       if (s != HOTRG_OK) return s;
     }
     const int xend = pr.first_block ? std::min(p.xs, ca) : ca;
@@ -1201,22 +1257,15 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
       const int64_t rA_full = (int64_t)xs * p.chi[p.b] * p.D[p.c] * p.D[p.c] * p.D[mu];
       // a probe's rows: the first ones, or (sectors) the first half of them in either sector
       const int64_t rA = pr.gemm_rows > 0 && !p.sect ? std::min(rA_full, pr.gemm_rows) : rA_full;
-      for (int ph : {kPass1, kPassMax, kPass2}) {
-        if (!pr.ttm) break;
-        if (ph == kPassMax && scale != kScaleExact) continue;
-        if (amaxA && clear_phase(ph)) CK(cudaMemsetAsync(amaxA, 0, ne * tw * sizeof(unsigned), st), "amax clear");
-        for (int w = 0; w < nbuild; ++w) {
-          hotrg_status s = build_A<R>(ctx, p, src[w], Ua, Ub, x0, xs, O1A + w * O1Asz, opnd(Abuf, w * Asz * planes),
-                                      opnd(Alob, w * Asz * planes), st, esA, amaxA ? amaxA + (tw > 1 ? w : 0) : nullptr,
-                                      tw, scale, ph, tab, parity[w]);
-          if (s != HOTRG_OK) return s;
-        }
+      if (!whole && pr.ttm) {
+        hotrg_status s = build(true, false, x0, xs, 0, 0);
+        if (s != HOTRG_OK) return s;
       }
       for (int x20 = 0; x20 < x2end; x20 += p.xs2) {
         const int xs2 = std::min(p.xs2, ca - x20);
         const int64_t rB = (int64_t)xs2 * p.chi[p.b] * p.D[p.c] * p.D[p.c] * p.D[mu];
         if (b_sliced && pr.ttm) {
-          hotrg_status s = buildB(x20, xs2);
+          hotrg_status s = build(false, true, 0, 0, x20, xs2);
           if (s != HOTRG_OK) return s;
         }
         hotrg_status s = HOTRG_OK;
@@ -1335,9 +1384,10 @@ hotrg_status do_step(hotrg_ctx* ctx, const StepPlan& p) {
   LK(2, launch_norm<R>(tensor_ptr<R>(ctx, 0, 1 - ctx->cur, 0), p.Enew, ctx->batch, cap, (double*)(sb + sc.npart), dstep,
                        cval, lnz, rec, status, st),
      "norm");
-  for (int w = 0; w < nt; ++w)
-    LK(1, launch_scale<R>(tensor_ptr<R>(ctx, w, 1 - ctx->cur, 0), p.Enew, ctx->batch, cap, cval, st), "scale");
-  LK(1, launch_step_end((int*)(ctx->ws + ctx->L.step), st), "step end");
+  // the tensors' slots: T, S, M, two buffers of every element each
+  LK(1, launch_scale<R>(tensor_ptr<R>(ctx, 0, 1 - ctx->cur, 0), p.Enew, ctx->batch, cap, nt, 2 * ctx->batch * cap, cval,
+                        (int*)(ctx->ws + ctx->L.step), st),
+     "scale");
   return HOTRG_OK;
 }
 

@@ -247,16 +247,16 @@ __device__ __forceinline__ void operand_run(const R* x0, const R* x1, bool ok0, 
 }
 
 template <typename R, int MODE, int NJM>
-__global__ void __launch_bounds__(256) sector_operand_kernel(const R* __restrict__ in, const R* __restrict__ U,
-                                                             R* __restrict__ out, R* __restrict__ out_lo,
-                                                             const __grid_constant__ SectorOperand a) {
+__global__ void __launch_bounds__(256) sector_operand_kernel(const __grid_constant__ SectorJobs<R> jobs,
+                                                             const R* __restrict__ U) {
   const int e = blockIdx.y;
+  const SectorOperand& a = jobs.a[blockIdx.z];
   const SectorTables t = a.tab.at(e);
   const SectorPlan& p = *t.plan;
-  in += e * a.in_bs;
+  const R* __restrict__ in = jobs.in[blockIdx.z] + e * a.in_bs;
   U += e * a.u_bs;
-  out = elem_out<R, MODE>(out, e * a.out_bs);
-  out_lo = elem_out<R, MODE>(out_lo, e * a.out_bs);
+  R* __restrict__ out = elem_out<R, MODE>(jobs.out[blockIdx.z], e * a.out_bs);
+  R* __restrict__ out_lo = elem_out<R, MODE>(jobs.lo[blockIdx.z], e * a.out_bs);
   unsigned* amax = a.amax ? a.amax + e * a.amax_bs : nullptr;
   const R uscale = (R)split_scale<MODE>(amax);
   extern __shared__ __align__(16) unsigned char fsm[];
@@ -373,16 +373,18 @@ __global__ void __launch_bounds__(256) sector_operand_kernel(const R* __restrict
 }
 
 template <typename R>
-cudaError_t launch_sector_operand(const R* in, const R* U, R* out, R* out_lo, const SectorOperand& a, int ne, int mode,
-                                  cudaStream_t st) {
+cudaError_t launch_sector_operand(const SectorJobs<R>& jobs, const R* U, int ne, int mode, cudaStream_t st) {
+  if (jobs.n < 1 || jobs.n > kMaxPassJobs) return cudaErrorInvalidValue;
+  const SectorOperand& a = jobs.a[0];           // every job of a step has the same D_b and chi_b
   const size_t smem = (size_t)2 * a.Db * a.Db * ((a.cb + 3) / 4 * 4 + 4) * sizeof(R);   // a bound for any charges
   if (smem > (size_t)kSectorSmem) return cudaErrorInvalidValue;
-  int64_t bx = a.nouter;
-  const int64_t cap = 152 * 16 / ne > 32 ? 152 * 16 / ne : 32;
+  int64_t bx = 1;
+  for (int i = 0; i < jobs.n; ++i) bx = jobs.a[i].nouter > bx ? jobs.a[i].nouter : bx;
+  const int64_t share = 152 * 16 / ((int64_t)ne * jobs.n), cap = share > 32 ? share : 32;
   if (bx > cap) bx = cap;
-  const dim3 g((unsigned)bx, ne);
+  const dim3 g((unsigned)bx, ne, jobs.n);
   auto go = [&](auto kernel) -> cudaError_t {
-    kernel<<<g, 256, smem, st>>>(in, U, out, out_lo, a);
+    kernel<<<g, 256, smem, st>>>(jobs, U);
     return cudaGetLastError();
   };
   // the contracted leg's indices of one charge are at most D_b (all of one charge)
@@ -401,10 +403,8 @@ cudaError_t launch_sector_operand(const R* in, const R* U, R* out, R* out_lo, co
   }
   return cudaErrorInvalidValue;
 }
-template cudaError_t launch_sector_operand<float>(const float*, const float*, float*, float*, const SectorOperand&, int,
-                                                  int, cudaStream_t);
-template cudaError_t launch_sector_operand<double>(const double*, const double*, double*, double*,
-                                                   const SectorOperand&, int, int, cudaStream_t);
+template cudaError_t launch_sector_operand<float>(const SectorJobs<float>&, const float*, int, int, cudaStream_t);
+template cudaError_t launch_sector_operand<double>(const SectorJobs<double>&, const double*, int, int, cudaStream_t);
 
 // ---------------------------------------------------------------------------- closing passes
 // First closing pass: O3[Z][m][n] = sum_{c1, c2} U[c1, c2, Z] C[row(X, Y, c1, c1', mu1)][col(X', Y', c2, c2', mu2')]

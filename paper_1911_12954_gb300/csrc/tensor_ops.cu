@@ -162,8 +162,8 @@ __device__ __forceinline__ void fiber_store(R* out, R* out_lo, int64_t o, R acc)
 // fibre stay in registers; the new index is produced in blocks of 32 accumulators, each U
 // row of a block read as 16-byte vectors, so an output costs about J FMAs plus its store.
 template <typename R, int MODE>
-__global__ void __launch_bounds__(256) ttm_short_kernel(const R* __restrict__ in, const R* __restrict__ U,
-                                                        R* __restrict__ out, R* __restrict__ out_lo, FiberArgs a) {
+__device__ __forceinline__ void ttm_short(const R* __restrict__ in, const R* __restrict__ U, R* __restrict__ out,
+                                          R* __restrict__ out_lo, const FiberArgs& a) {
   in += blockIdx.y * a.in_bs;                  // batch element blockIdx.y
   U += blockIdx.y * a.u_bs;
   out = elem_out<R, MODE>(out, blockIdx.y * a.out_bs);
@@ -235,6 +235,28 @@ __global__ void __launch_bounds__(256) ttm_short_kernel(const R* __restrict__ in
     }
   }
   if (MODE == kTTMMaxAbs || MODE == kTTMStoreMax) merge_max(amax, (double)tmax, a.amax_mul);   // every thread gets here
+}
+
+template <typename R, int MODE>
+__global__ void __launch_bounds__(256) ttm_short_kernel(const R* __restrict__ in, const R* __restrict__ U,
+                                                        R* __restrict__ out, R* __restrict__ out_lo, FiberArgs a) {
+  ttm_short<R, MODE>(in, U, out, out_lo, a);
+}
+
+// Several contractions of one kind in one launch (blockIdx.z): the first passes of both operand sides and of every
+// tensor are independent, and a small one leaves most of the chip idle (8 temperatures at D_cut = 4: two launches
+// of 13 us).
+template <typename R>
+struct FiberJobs {
+  const R* in[kMaxPassJobs];
+  const R* U[kMaxPassJobs];
+  R* out[kMaxPassJobs];
+  FiberArgs a[kMaxPassJobs];
+};
+template <typename R, int MODE>
+__global__ void __launch_bounds__(256) ttm_short_jobs_kernel(const __grid_constant__ FiberJobs<R> j) {
+  const int z = blockIdx.z;
+  ttm_short<R, MODE>(j.in[z], j.U[z], j.out[z], nullptr, j.a[z]);
 }
 
 // The fp16 split of a short contraction, two fibres per thread: when the innermost fibre leg
@@ -624,6 +646,44 @@ cudaError_t launch_ttm(const TI* in, const TU* U, TO* out, TO* out_lo, const TTM
   return cudaGetLastError();
 }
 
+template <typename R>
+cudaError_t launch_ttm_jobs(const TTMJob<R>* jobs, int n, int* launches, cudaStream_t st) {
+  // one launch where all are plain stores (with or without the maximum) of the short fibre form
+  FiberJobs<R> f{};
+  bool fused = n > 1 && n <= kMaxPassJobs;
+  size_t smem = 0;
+  int64_t blocks = 0;
+  for (int i = 0; i < n && fused; ++i) {
+    const TTMJob<R>& j = jobs[i];
+    fused = j.mode == jobs[0].mode && (j.mode == kTTMStore || j.mode == kTTMStoreMax) && j.U && j.a.nb == jobs[0].a.nb &&
+            j.a.outer > 0 && j.a.inner > 0 && to_fiber(j.a, sizeof(R), f.a[i]) && f.a[i].J1 * f.a[i].J2 <= kShortJ;
+    if (!fused) break;
+    f.in[i] = j.in;
+    f.U[i] = j.U;
+    f.out[i] = j.out;
+    smem = std::max(smem, short_smem(f.a[i].J1 * f.a[i].J2, f.a[i].R1 * f.a[i].R2, sizeof(R)));
+    blocks = std::max(blocks, (f.a[i].nfib + 255) / 256);
+  }
+  if (fused) {
+    const int nb = jobs[0].a.nb;
+    const int64_t cap = std::max<int64_t>(8, 152 * 16 / ((int64_t)nb * n));
+    const dim3 g((unsigned)std::min(blocks, cap), nb, n);
+    if (jobs[0].mode == kTTMStoreMax) ttm_short_jobs_kernel<R, kTTMStoreMax><<<g, 256, smem, st>>>(f);
+    else ttm_short_jobs_kernel<R, kTTMStore><<<g, 256, smem, st>>>(f);
+    *launches = 1;
+    return cudaGetLastError();
+  }
+  *launches = n;
+  for (int i = 0; i < n; ++i) {
+    const TTMJob<R>& j = jobs[i];
+    const cudaError_t e = launch_ttm<R, R, R>(j.in, j.U, j.out, j.lo, j.a, j.mode, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+template cudaError_t launch_ttm_jobs<double>(const TTMJob<double>*, int, int*, cudaStream_t);
+template cudaError_t launch_ttm_jobs<float>(const TTMJob<float>*, int, int*, cudaStream_t);
+
 template cudaError_t launch_ttm<double, double, double>(const double*, const double*, double*, double*,
                                                         const TTMArgs&, int, cudaStream_t);
 template cudaError_t launch_ttm<float, float, float>(const float*, const float*, float*, float*,
@@ -865,20 +925,12 @@ cudaError_t launch_sector_stats(const void* plane, const SectorTab& tab, int ele
   return cudaGetLastError();
 }
 
-// Advances the device step counter at the end of a step.
-__global__ void step_end_kernel(int* step) {
-  if (threadIdx.x == 0) *step += 1;
-}
-
-cudaError_t launch_step_end(int* step, cudaStream_t st) {
-  step_end_kernel<<<1, 32, 0, st>>>(step);
-  return cudaGetLastError();
-}
-
+// Divides the new tensors by c (blockIdx.z: tensor) and advances the device step counter: the last launch of a step.
 template <typename R>
-__global__ void __launch_bounds__(256) scale_kernel(R* __restrict__ x, int64_t n, int64_t xstride,
-                                                    const double* __restrict__ c) {
-  x += blockIdx.y * xstride;                   // batch element blockIdx.y
+__global__ void __launch_bounds__(256) scale_kernel(R* __restrict__ x, int64_t n, int64_t xstride, int64_t tstride,
+                                                    const double* __restrict__ c, int* step) {
+  x += blockIdx.y * xstride + blockIdx.z * tstride;   // batch element blockIdx.y
+  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *step += 1;
   const R inv = (R)(1.0 / c[blockIdx.y]);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     x[i] *= inv;
@@ -892,19 +944,21 @@ cudaError_t launch_norm(const R* x, int64_t n, int nb, int64_t xstride, double* 
   return cudaGetLastError();
 }
 template <typename R>
-cudaError_t launch_scale(R* x, int64_t n, int nb, int64_t xstride, const double* c, cudaStream_t st) {
-  if (n <= 0 || nb <= 0) return cudaSuccess;
+cudaError_t launch_scale(R* x, int64_t n, int nb, int64_t xstride, int nt, int64_t tstride, const double* c, int* step,
+                         cudaStream_t st) {
+  if (n <= 0 || nb <= 0 || nt <= 0) return cudaErrorInvalidValue;
   int64_t blocks = (n + 255) / 256;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  scale_kernel<R><<<dim3((unsigned)blocks, nb), 256, 0, st>>>(x, n, xstride, c);
+  const int64_t cap = std::max<int64_t>(8, 152 * 16 / ((int64_t)nb * nt));
+  if (blocks > cap) blocks = cap;
+  scale_kernel<R><<<dim3((unsigned)blocks, nb, nt), 256, 0, st>>>(x, n, xstride, tstride, c, step);
   return cudaGetLastError();
 }
 template cudaError_t launch_norm<double>(const double*, int64_t, int, int64_t, double*, const int*, double*, double*,
                                          DevRecord*, int*, cudaStream_t);
 template cudaError_t launch_norm<float>(const float*, int64_t, int, int64_t, double*, const int*, double*, double*,
                                         DevRecord*, int*, cudaStream_t);
-template cudaError_t launch_scale<double>(double*, int64_t, int, int64_t, const double*, cudaStream_t);
-template cudaError_t launch_scale<float>(float*, int64_t, int, int64_t, const double*, cudaStream_t);
+template cudaError_t launch_scale<double>(double*, int64_t, int, int64_t, int, int64_t, const double*, int*, cudaStream_t);
+template cudaError_t launch_scale<float>(float*, int64_t, int, int64_t, int, int64_t, const double*, int*, cudaStream_t);
 
 // ---------------------------------------------------------------------------- trace
 // Tr T = sum_{x,y,z,t} T[x,x,y,y,z,z,t,t] in FP64; one block per batch element.
