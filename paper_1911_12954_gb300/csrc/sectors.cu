@@ -408,14 +408,14 @@ template cudaError_t launch_sector_operand<double>(const SectorJobs<double>&, co
 
 // ---------------------------------------------------------------------------- closing passes
 // First closing pass: O3[Z][m][n] = sum_{c1, c2} U[c1, c2, Z] C[row(X, Y, c1, c1', mu1)][col(X', Y', c2, c2', mu2')]
-// with m, n the ranked row groups (X, Y, c1', mu1) and (X', Y', c2', mu2'). A block takes 256 column
+// with m, n the ranked row groups (X, Y, c1', mu1) and (X', Y', c2', mu2'). A block takes NT column
 // groups of one charge t and row groups of one charge r, four at a time: only the pairs (c1, c2) with
 // q(c1) + q(c2) = s (s = r + t + the output's parity) and the Z of charge s are nonzero, the same for
 // the whole block, so no lane is idle; the entries of the other Z are neither written nor read.
-template <typename R, int NZ>
-__global__ void __launch_bounds__(256) sector_close1_kernel(const R* __restrict__ C, const R* __restrict__ U,
-                                                            R* __restrict__ O3,
-                                                            const __grid_constant__ SectorClose a) {
+template <typename R, int NZ, int NT>
+__global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(R) * NZ > 64 ? 2 : 4) : 1)
+    sector_close1_kernel(const R* __restrict__ C, const R* __restrict__ U, R* __restrict__ O3,
+                         const __grid_constant__ SectorClose a) {
   constexpr int RG = 4;
   const int e = blockIdx.z;
   const SectorTables t = a.tab.at(e);
@@ -426,14 +426,14 @@ __global__ void __launch_bounds__(256) sector_close1_kernel(const R* __restrict_
   const int Dc = a.Dc, tid = threadIdx.x;
   const int g0 = p.grp[0][a.x20], n0 = p.grp[0][a.x20 + a.xs2] - g0;
   const int g1 = p.grp[1][a.x20], n1 = p.grp[1][a.x20 + a.xs2] - g1;
-  const int ch0 = (n0 + 255) / 256;
+  const int ch0 = (n0 + NT - 1) / NT;
   const int tq = (int)blockIdx.x < ch0 ? 0 : 1;                 // charge of the column groups
-  const int i0 = (tq ? (int)blockIdx.x - ch0 : (int)blockIdx.x) * 256;
+  const int i0 = (tq ? (int)blockIdx.x - ch0 : (int)blockIdx.x) * NT;
   const int ncol = tq ? n1 : n0;
   if (i0 >= ncol) return;
   extern __shared__ __align__(16) unsigned char fsm[];
   R* Us = (R*)fsm;                                   // [2][Dc][Dc][NZ]: (charge of Z, c1, c2, slot), zero past the last slot
-  int* rks = (int*)(Us + (size_t)2 * Dc * Dc * NZ);  // [Dc][256] column of c2
+  int* rks = (int*)(Us + (size_t)2 * Dc * Dc * NZ);  // [Dc][NT] column of c2
   __shared__ int nz[2], nc[2], zlist[2][kMaxLeg], clist[2][kMaxLeg];
   if (tid < 2) {
     int n = 0;
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(256) sector_close1_kernel(const R* __restrict_
     nc[tid] = n;
   }
   __syncthreads();
-  for (int i = tid; i < 2 * Dc * Dc * NZ; i += 256) {
+  for (int i = tid; i < 2 * Dc * Dc * NZ; i += NT) {
     const int sl = i % NZ, c2 = (i / NZ) % Dc, c1 = (i / (NZ * Dc)) % Dc, q = i / (NZ * Dc * Dc);
     Us[i] = sl < nz[q] ? U[((int64_t)c1 * Dc + c2) * a.cc + zlist[q][sl]] : (R)0;
   }
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(256) sector_close1_kernel(const R* __restrict_
     const uint32_t hi = g / (uint32_t)inner, rem = g - hi * inner;
     for (int c2 = 0; c2 < Dc; ++c2) {
       const uint32_t r = t.row[((int64_t)hi * Dc + c2) * inner + rem];
-      rks[c2 * 256 + tid] = (int)(r & 0x7fffffffu) - p.row[r >> 31][a.x20];
+      rks[c2 * NT + tid] = (int)(r & 0x7fffffffu) - p.row[r >> 31][a.x20];
     }
   }
   __syncthreads();
@@ -502,7 +502,7 @@ __global__ void __launch_bounds__(256) sector_close1_kernel(const R* __restrict_
           R x[4][RG];
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const int col = rks[clist[jc][k + q] * 256 + tid];
+            const int col = rks[clist[jc][k + q] * NT + tid];
 #pragma unroll
             for (int i = 0; i < RG; ++i) x[q][i] = cp[i][col];
           }
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(256) sector_close1_kernel(const R* __restrict_
           }
         }
         for (; k < n; ++k) {
-          const int col = rks[clist[jc][k] * 256 + tid];
+          const int col = rks[clist[jc][k] * NT + tid];
           R x[RG];
 #pragma unroll
           for (int i = 0; i < RG; ++i) x[i] = cp[i][col];
@@ -629,11 +629,14 @@ template <typename R>
 cudaError_t launch_sector_close(const R* C, const R* U, R* O3, R* T, const SectorClose& a, int ne, cudaStream_t st) {
   if (a.nfib > 0x7fffffffLL || a.nfib < 1) return cudaErrorInvalidValue;
   const int NZ = a.cc <= 4 ? 4 : (a.cc <= 8 ? 8 : 16);
-  const size_t s1 = (size_t)2 * a.Dc * a.Dc * NZ * sizeof(R) + (size_t)a.Dc * 256 * sizeof(int);
+  const int64_t cols = (int64_t)a.xs2 * a.cb * a.Dc * a.Dm, rowg = (int64_t)a.xs * a.cb * a.Dc * a.Dm;
+  // 128 threads fill small products and FP64 ones better (D_cut = 4: 20 -> 16 us, D = 6 FP64: 450 -> 330 us), 256
+  // are faster on large FP32 ones (D_cut = 8: 993 us against 1085)
+  const int NT = sizeof(R) == 4 && NZ > 4 && cols > 2048 ? 256 : 128;
+  const size_t s1 = (size_t)2 * a.Dc * a.Dc * NZ * sizeof(R) + (size_t)a.Dc * NT * sizeof(int);
   const size_t s2 = (size_t)a.Dc * a.Dc * NZ * sizeof(R);
   if (s1 > (size_t)kSectorSmem) return cudaErrorInvalidValue;
-  const int64_t cols = (int64_t)a.xs2 * a.cb * a.Dc * a.Dm, rowg = (int64_t)a.xs * a.cb * a.Dc * a.Dm;
-  const int64_t bx = (cols + 255) / 256 + 1;
+  const int64_t bx = (cols + NT - 1) / NT + 1;
   int64_t by = (152 * 12 + bx * ne - 1) / (bx * ne);
   by = by < 1 ? 1 : by;
   by = by > (rowg + 7) / 8 ? (rowg + 7) / 8 : by;      // four row groups of one charge per step
@@ -643,15 +646,21 @@ cudaError_t launch_sector_close(const R* C, const R* U, R* O3, R* T, const Secto
   if (b2 > cap) b2 = cap;
   const dim3 g2((unsigned)b2, ne);
   auto go = [&](auto k1, auto k2) -> cudaError_t {
-    k1<<<g1, 256, s1, st>>>(C, U, O3, a);
+    k1<<<g1, NT, s1, st>>>(C, U, O3, a);
     cudaError_t er = cudaGetLastError();
     if (er != cudaSuccess) return er;
     k2<<<g2, 256, s2, st>>>(O3, U, T, a);
     return cudaGetLastError();
   };
-  if (NZ == 4) return go(sector_close1_kernel<R, 4>, sector_close2_kernel<R, 4>);
-  if (NZ == 8) return go(sector_close1_kernel<R, 8>, sector_close2_kernel<R, 8>);
-  return go(sector_close1_kernel<R, 16>, sector_close2_kernel<R, 16>);
+  if (NZ == 4) return go(sector_close1_kernel<R, 4, 128>, sector_close2_kernel<R, 4>);
+  if (NT == 256) {
+    if constexpr (sizeof(R) == 4) {
+      if (NZ == 8) return go(sector_close1_kernel<R, 8, 256>, sector_close2_kernel<R, 8>);
+      return go(sector_close1_kernel<R, 16, 256>, sector_close2_kernel<R, 16>);
+    }
+  }
+  if (NZ == 8) return go(sector_close1_kernel<R, 8, 128>, sector_close2_kernel<R, 8>);
+  return go(sector_close1_kernel<R, 16, 128>, sector_close2_kernel<R, 16>);
 }
 template cudaError_t launch_sector_close<float>(const float*, const float*, float*, float*, const SectorClose&, int,
                                                 cudaStream_t);
@@ -667,9 +676,10 @@ void sectors_prepare() {
   set(sector_operand_kernel<double, kTTMStore, 16>);
   set(sector_operand_kernel<double, kTTMMaxAbs, 16>);
   set(sector_operand_kernel<double, kTTMSplitOz, 16>);
-  set(sector_close1_kernel<float, 16>);
-  set(sector_close1_kernel<double, 8>);
-  set(sector_close1_kernel<double, 16>);
+  set(sector_close1_kernel<float, 16, 128>);
+  set(sector_close1_kernel<float, 16, 256>);
+  set(sector_close1_kernel<double, 8, 128>);
+  set(sector_close1_kernel<double, 16, 128>);
   set(sector_close2_kernel<double, 16>);
   cudaGetLastError();
 }
