@@ -264,6 +264,28 @@ struct TTMJob {
 template <typename R>
 cudaError_t launch_ttm_jobs(const TTMJob<R>* jobs, int n, int* launches, cudaStream_t st);
 
+// Second half-contraction pass of the dense fp16 planes, range by range of the summed index (tensor_ops.cu).
+struct DenseSplit {
+  int sideB, Da, Db, Dc, Dm, cb;
+  int nouter, n2, P;                        // (X, c, c', mu); values of a2 per block; panels
+  int64_t in_x, in_j, in_c0, in_c1, in_m, in_a;   // strides of the first pass's output
+  int u_j, u_r;                             // U strides of the contracted and the new leg
+  int64_t rows, Kp, kps;
+  int64_t in_bs, u_bs, out_bs;
+  unsigned* amax;
+  int amax_bs;
+};
+struct DenseSplitJobs {
+  const float* in[kMaxPassJobs];
+  float* out[kMaxPassJobs];
+  float* lo[kMaxPassJobs];
+  DenseSplit a[kMaxPassJobs];
+  int n;
+};
+bool dense_split_fits(DenseSplit& a);
+cudaError_t launch_dense_split(const DenseSplitJobs& jobs, const float* U, int ne, cudaStream_t st);
+void tensor_ops_prepare();
+
 template <typename R>
 cudaError_t launch_gram(const GramPack& jobs, int njobs, int Rmax, int nchunks, cudaStream_t st);
 cudaError_t launch_gram_reduce(const GramPack& jobs, int njobs, int nchunks, int64_t RRmax, int64_t out_stride,

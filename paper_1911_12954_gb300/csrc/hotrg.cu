@@ -225,6 +225,17 @@ struct PassList {
   SectorJobs<R> sec{};
   const R* sec_U = nullptr;
   int sec_mode = kTTMStore;
+  DenseSplitJobs split{};
+  const float* split_U = nullptr;
+  cudaError_t add(const float* in, const float* U, float* out, float* lo, const DenseSplit& a) {
+    if (split.n == kMaxPassJobs || (split.n > 0 && U != split_U)) return cudaErrorInvalidValue;
+    split.in[split.n] = in;
+    split.out[split.n] = out;
+    split.lo[split.n] = lo;
+    split.a[split.n++] = a;
+    split_U = U;
+    return cudaSuccess;
+  }
   cudaError_t add(const R* in, const R* U, R* out, R* lo, const TTMArgs& a, int mode) {
     const cudaError_t e = check_ttm(U, a);
     if (e == cudaSuccess) ttm.push_back(TTMJob<R>{in, U, out, lo, a, mode});
@@ -244,6 +255,11 @@ struct PassList {
     *launches = 0;
     if (!ttm.empty()) {
       const cudaError_t e = launch_ttm_jobs<R>(ttm.data(), (int)ttm.size(), launches, st);
+      if (e != cudaSuccess) return e;
+    }
+    if (split.n > 0) {
+      *launches += 1;
+      const cudaError_t e = launch_dense_split(split, split_U, ne, st);
       if (e != cudaSuccess) return e;
     }
     if (sec.n > 0) {
@@ -624,6 +640,44 @@ void operand_strides(const StepPlan& p, const std::vector<int64_t>& rn, int64_t 
   }
 }
 
+// The dense fp16 second pass in the ranged form (dense_split_kernel) where it applies; false: not added.
+template <typename R>
+bool add_dense_split(hotrg_ctx* ctx, const StepPlan& p, int side, const R* Ub, int xs, const int64_t* os, const R* O1,
+                     R* out, R* out_lo, PassList<R>& list, const ElemStrides& es, unsigned* amax, int amax_bs) {
+  if constexpr (sizeof(R) == 4) {
+    if (ctx->prec != HOTRG_FP16X3) return false;
+    const int cb = p.chi[p.b];
+    DenseSplit a{};
+    a.sideB = side;
+    a.Da = p.D[p.a];
+    a.Db = p.D[p.b];
+    a.Dc = p.D[p.c];
+    a.Dm = p.D[p.mu];
+    a.cb = cb;
+    a.nouter = xs * a.Dc * a.Dc * a.Dm;
+    a.P = (int)p.P;
+    a.in_x = os[0];
+    a.in_j = os[1];
+    a.in_c0 = os[2];
+    a.in_c1 = os[3];
+    a.in_m = os[4];
+    a.in_a = os[5];
+    a.u_j = side == 0 ? a.Db * cb : cb;
+    a.u_r = side == 0 ? cb : a.Db * cb;
+    a.rows = (int64_t)xs * cb * a.Dc * a.Dc * a.Dm;
+    a.Kp = p.Kp;
+    a.kps = p.kps;
+    a.in_bs = es.O1;
+    a.u_bs = es.U;
+    a.out_bs = es.op;
+    a.amax = amax;
+    a.amax_bs = amax_bs;
+    if (!dense_split_fits(a)) return false;
+    return list.add(O1, Ub, out, out_lo, a) == cudaSuccess;
+  }
+  return false;
+}
+
 // Second half-contraction pass of one tensor by charge sectors. O1 is the first pass's output
 // [X, contracted leg, c, c', mu, summed legs] with strides os; side 0: A (contracts b1 of
 // U^b[b1, b2, Y]), 1: B (contracts b2' of U^b[b1', b2', Y']).
@@ -728,7 +782,8 @@ hotrg_status build_A(hotrg_ctx* ctx, const StepPlan& p, const R* P, const R* Ua,
     t.amax_bs = amax_bs;
     if ((phases & kPassMax) && amax && scale == kScaleExact)
       CK(list.add(O1, Ub, A, Alo, t, kTTMMaxAbs), "ttm A max");
-    if (phases & kPass2) CK(list.add(O1, Ub, A, Alo, t, mode), "ttm A2");
+    if ((phases & kPass2) && !add_dense_split<R>(ctx, p, 0, Ub, xs, os.data(), O1, A, Alo, list, es, amax, amax_bs))
+      CK(list.add(O1, Ub, A, Alo, t, mode), "ttm A2");
   }
   return HOTRG_OK;
 }
@@ -792,7 +847,8 @@ hotrg_status build_B(hotrg_ctx* ctx, const StepPlan& p, const R* Q, const R* Ua,
     t.amax_bs = amax_bs;
     if ((phases & kPassMax) && amax && scale == kScaleExact)
       CK(list.add(O1, Ub, B, Blo, t, kTTMMaxAbs), "ttm B max");
-    if (phases & kPass2) CK(list.add(O1, Ub, B, Blo, t, mode), "ttm B2");
+    if ((phases & kPass2) && !add_dense_split<R>(ctx, p, 1, Ub, xs, os.data(), O1, B, Blo, list, es, amax, amax_bs))
+      CK(list.add(O1, Ub, B, Blo, t, mode), "ttm B2");
   }
   return HOTRG_OK;
 }
@@ -1717,6 +1773,7 @@ hotrg_status hotrg_set_workspace(hotrg_ctx* ctx, void* dev_ptr, size_t bytes) {
   jacobi_prepare();
   gemm_prepare();
   sectors_prepare();
+  tensor_ops_prepare();
   ctx->ws = (char*)dev_ptr;
   ctx->ws_bytes = bytes;
   ctx->L = L;

@@ -346,6 +346,150 @@ __global__ void __launch_bounds__(256) ttm_pair_f16_kernel(const R* __restrict__
   if (MAXONLY) merge_max(amax, (double)tmax, a.amax_mul);   // every thread of the block gets here
 }
 
+// The fp16 split where neighbouring fibres cannot share a half2 (odd innermost extent): a block takes one operand row
+// group (X, c, c', mu; every Y) and n2 values of a2, keeps the hi and lo outputs of that contiguous range of the
+// summed index in shared memory, shifted so that shared and global 16-byte boundaries agree, and writes whole
+// 16-byte pieces. Same products in the same order as the short form, so the same bits. The two-byte stores of that form
+// into runs that start at any two-byte boundary held it at 1.2 TB/s; here the shared-memory accesses (two stores and
+// two loads an output) bound it at 1.5 TB/s. D = 5, T and S of 4 temperatures, both sides, 8 steps: 3.37 -> 2.64 ms.
+template <int JM>
+__global__ void __launch_bounds__(256) dense_split_kernel(const __grid_constant__ DenseSplitJobs jobs,
+                                                          const float* __restrict__ U) {
+  const DenseSplit& a = jobs.a[blockIdx.z];
+  const int e = blockIdx.y;
+  const float* __restrict__ in = jobs.in[blockIdx.z] + e * a.in_bs;
+  __half* __restrict__ hi = (__half*)jobs.out[blockIdx.z] + e * a.out_bs;
+  __half* __restrict__ lo = (__half*)jobs.lo[blockIdx.z] + e * a.out_bs;
+  U += e * a.u_bs;
+  extern __shared__ __align__(16) unsigned char fsm[];
+  const int J = a.Db, Yp = (a.cb + 3) / 4 * 4, F = a.Da * a.Db * a.Dm, inner = F * a.Db;
+  const int pitch = (a.n2 * inner + 7 + 7) / 8 * 8;
+  float* Us = (float*)fsm;                            // [r][j][Yp], zero past cb
+  __half* Hs = (__half*)(Us + (size_t)a.Db * J * Yp); // [cb][pitch]
+  __half* Ls = Hs + (size_t)a.cb * pitch;
+  const float uscale = (float)split_scale<kTTMSplitF16>(a.amax ? a.amax + e * a.amax_bs : nullptr);
+  for (int i = threadIdx.x; i < a.Db * J * Yp; i += blockDim.x) {
+    const int y = i % Yp, j = (i / Yp) % J, r = i / (Yp * J);
+    Us[i] = y < a.cb ? U[j * a.u_j + r * a.u_r + y] * uscale : 0.f;
+  }
+  const int nchunk = (a.Da + a.n2 - 1) / a.n2;
+  for (int o = blockIdx.x; o < a.nouter * nchunk; o += gridDim.x) {
+    const int a20 = (o % nchunk) * a.n2, n2 = min(a.n2, a.Da - a20);
+    int q = o / nchunk;
+    const int m = q % a.Dm;
+    q /= a.Dm;
+    const int c1 = q % a.Dc;
+    q /= a.Dc;
+    const int c0 = q % a.Dc;
+    const int X = q / a.Dc;
+    // start of the range in row Y: k = a20 inner, whole panels per a2 where a panel is one a2
+    const int64_t k0 = (int64_t)a20 * inner, pn = k0 / a.Kp;
+    const int64_t col0 = pn * a.rows * a.kps + (k0 - pn * a.Kp);
+    const int sft = (int)(col0 & 7);                  // rows start on 128-byte boundaries
+    const float* src = in + X * a.in_x + c0 * a.in_c0 + c1 * a.in_c1 + m * a.in_m + a20 * a.in_a;
+    __syncthreads();
+    for (int f = threadIdx.x; f < n2 * F; f += blockDim.x) {
+      const int a2 = f / F, g = f - a2 * F;
+      const float* xp = src + a2 * a.in_a + g;
+      float x[JM];
+#pragma unroll
+      for (int j = 0; j < JM; ++j) x[j] = j < J ? xp[j * a.in_j] : 0.f;
+      // A: r = b2 comes first in (b2, a1', b1', k); B: r = b1' sits before k
+      const int pos = sft + a2 * inner + (a.sideB ? g / a.Dm * (a.Db * a.Dm) + g % a.Dm : g);
+      const int rstep = a.sideB ? a.Dm : F;
+      for (int r = 0; r < a.Db; ++r) {
+        for (int yb = 0; yb < a.cb; yb += 4) {
+          float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int j = 0; j < JM; ++j) {
+            if (j < J) {
+              const float4 u = *(const float4*)(Us + (r * J + j) * Yp + yb);
+              v[0] = fmaf(u.x, x[j], v[0]);
+              v[1] = fmaf(u.y, x[j], v[1]);
+              v[2] = fmaf(u.z, x[j], v[2]);
+              v[3] = fmaf(u.w, x[j], v[3]);
+            }
+          }
+#pragma unroll
+          for (int s = 0; s < 4; ++s) {
+            if (yb + s < a.cb) {
+              const __half h = __float2half_rn(v[s]);
+              const int at = (yb + s) * pitch + pos + r * rstep;
+              Hs[at] = h;
+              Ls[at] = __float2half_rn(v[s] - __half2float(h));
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();
+    const int n = n2 * inner, pieces = (sft + n + 7) / 8;
+    for (int i = threadIdx.x; i < a.cb * pieces; i += blockDim.x) {
+      const int Y = i / pieces, b = 8 * (i - Y * pieces);
+      const int64_t row = ((((int64_t)X * a.cb + Y) * a.Dc + c0) * a.Dc + c1) * a.Dm + m;
+      const int64_t at = row * a.kps + col0 - sft + b;
+      const __half* hs = Hs + Y * pitch + b;
+      const __half* ls = Ls + Y * pitch + b;
+      if (b >= sft && b + 8 <= sft + n) {
+        *(uint4*)(hi + at) = *(const uint4*)hs;
+        *(uint4*)(lo + at) = *(const uint4*)ls;
+      } else {
+        for (int h = 0; h < 8; ++h)
+          if (b + h >= sft && b + h < sft + n) {
+            hi[at + h] = hs[h];
+            lo[at + h] = ls[h];
+          }
+      }
+    }
+  }
+}
+
+// Shared memory of a block with n2 values of a2.
+size_t dense_split_smem(const DenseSplit& a, int n2) {
+  const int64_t inner = (int64_t)a.Da * a.Db * a.Db * a.Dm, pitch = (n2 * inner + 14) / 8 * 8;
+  return (size_t)a.Db * a.Db * ((a.cb + 3) / 4 * 4) * sizeof(float) + (size_t)2 * a.cb * pitch * sizeof(__half);
+}
+constexpr size_t kDenseSplitSmem = 100 * 1024;   // two blocks per SM
+
+void tensor_ops_prepare() {
+  static bool done[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || done[dev]) return;
+  done[dev] = true;
+  auto set = [](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSplitSmem); };
+  set(dense_split_kernel<4>);
+  set(dense_split_kernel<8>);
+  cudaGetLastError();
+}
+
+// Sets a.n2 and says whether the form applies: an odd extent somewhere in the innermost legs (even ones take the paired
+// form), contraction lengths up to 8, panels of whole a2 ranges, the tile in shared memory.
+bool dense_split_fits(DenseSplit& a) {
+  const int64_t inner = (int64_t)a.Da * a.Db * a.Db * a.Dm;
+  if ((a.Dm & 1) == 0 || a.Db > 8 || a.Kp % inner || (a.P > 1 && a.Kp != inner) || inner > 8192) return false;
+  int n2 = a.P > 1 ? 1 : a.Da;
+  while (n2 > 1 && dense_split_smem(a, n2) > kDenseSplitSmem) --n2;
+  a.n2 = n2;
+  return dense_split_smem(a, n2) <= kDenseSplitSmem;
+}
+
+cudaError_t launch_dense_split(const DenseSplitJobs& jobs, const float* U, int ne, cudaStream_t st) {
+  if (jobs.n < 1 || jobs.n > kMaxPassJobs) return cudaErrorInvalidValue;
+  int64_t tiles = 1;
+  size_t smem = 0;
+  for (int i = 0; i < jobs.n; ++i) {
+    const DenseSplit& a = jobs.a[i];
+    tiles = std::max<int64_t>(tiles, (int64_t)a.nouter * ((a.Da + a.n2 - 1) / a.n2));
+    smem = std::max(smem, dense_split_smem(a, a.n2));
+  }
+  if (smem > kDenseSplitSmem) return cudaErrorInvalidValue;
+  const int64_t cap = std::max<int64_t>(32, 152 * 16 / ((int64_t)ne * jobs.n));
+  const dim3 g((unsigned)std::min(tiles, cap), ne, jobs.n);
+  if (jobs.a[0].Db <= 4) dense_split_kernel<4><<<g, 256, smem, st>>>(jobs, U);
+  else dense_split_kernel<8><<<g, 256, smem, st>>>(jobs, U);
+  return cudaGetLastError();
+}
+
 // Long contractions (J > 16 with a short new index, Rn <= 16: the closing passes with U^c).
 // The outputs of a fibre stay in RB registers; its J inputs stream through in (j1, j2)
 // order, eight loads issued before their FMAs so that several are in flight per thread.
