@@ -10,6 +10,11 @@ hi + lo pair, three products, FP32 accumulation), normalisation and ln Z accumul
 W warm-up steps are steps 1..W of the run (bond dimensions reach 8 at step 3), the K
 timed steps are the steady-state steps W+1..W+K.
 
+At h = 0 the library contracts by Z2 charge sectors: three quarters of the 2 D^15 flops have
+an exactly zero factor and are not executed. "value" counts the whole 2 D^15 product of the
+method, as the host arm's does, and is a measure of time per step, not of the tensor pipe;
+"executed_flops_share" says which part of the product runs, and the roofline counts that part.
+
 Printed (rank 0, one JSON line): algorithmic TFLOP/s of the timed steps (value), the
 block-spin GEMM against its tensor-core roofline, the FP64 GPU path on one
 steady-state step, |Delta ln Z/V| of the mixed path against FP64, the FP64 NumPy oracle
@@ -82,11 +87,11 @@ def parse_args():
     return p.parse_args()
 
 
-# DRAM bytes (read + write) per launch of the block-spin GEMM, from one ncu capture of the
-# kernel as built now (dram__bytes_read.sum + dram__bytes_write.sum, one pass, the steady
-# D_cut = 8 launch: 134.78 GB + 4.71 GB), keyed by (precision, GEMM option, D_cut,
-# temperatures, impure). Workloads without a capture report null.
-GEMM_TRAFFIC = {("fp16x3", 0, 8, 1, False): 139.49e9}
+# DRAM bytes (read + write) per launch of the block-spin GEMM, keyed by (precision, GEMM option,
+# D_cut, temperatures, impure), from an ncu capture of the kernel as built. The sector GEMM of the
+# h = 0 runs has no capture yet; the dense one moved 139.49 GB a launch at D_cut = 8. Workloads
+# without a capture report null.
+GEMM_TRAFFIC = {}
 
 
 # --------------------------------------------------------------------------- helpers
@@ -630,7 +635,10 @@ def main():
 
     peak, peak_src = tensor_peak(args.precision, True)
     peak_burst, _ = tensor_peak(args.precision, False)
-    achieved = prof["gemm_flops"] / (prof["gemm_ms"] * 1e-3) / 1e12 if prof["gemm_ms"] > 0 else None
+    # without a field only the nonzero charge blocks of the product run: rows, columns and summed
+    # indices split in halves (to within a few percent), two blocks of an eighth
+    executed = 0.25 if hfield == 0.0 else 1.0
+    achieved = executed * prof["gemm_flops"] / (prof["gemm_ms"] * 1e-3) / 1e12 if prof["gemm_ms"] > 0 else None
     traffic = GEMM_TRAFFIC.get((args.precision, args.gemm_variant, D, args.batch, bool(impure)))
     line = {
         "metric": METRIC, "value": value, "unit": "TFLOP/s", "n_gpus": world, "steps": args.steps,
@@ -647,11 +655,12 @@ def main():
                      "frac": (achieved / peak) if achieved else None, "traffic": traffic,
                      "algorithmic_bytes": (2 * (4 if args.precision == "fp16x3" else 8) + 4) * float(D) ** 10,
                      "kernel": " + ".join(sorted({kernel_name(args.precision, pl["gemm_option"]) for pl in plans}))
-                               + " (block-spin contraction, 2 M N K algorithmic flops per launch)",
+                               + " (block-spin contraction, 2 M N K x executed_flops_share flops per launch)",
                      "peak_source": peak_src, "launches": prof["gemm_launches"],
                      "avg_launch_ms": prof["gemm_ms"] / max(1, prof["gemm_launches"]),
                      "tensor_pipe_flops_frac": (3 * achieved / peak) if achieved else None,
                      "peak_burst": peak_burst, "frac_of_burst": (achieved / peak_burst) if achieved else None},
+        "executed_flops_share": executed,
         "gpu_launches": prof["launches"],
         "plans": plans, "autotuner": tune,
         "clocks": clk.summary(),
