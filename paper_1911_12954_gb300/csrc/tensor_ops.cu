@@ -896,70 +896,45 @@ template cudaError_t launch_init<float>(const double*, const double*, float*, fl
                                         int, cudaStream_t);
 
 // ---------------------------------------------------------------------------- norm
-// Pass 1: each block writes the sum of squares of its grid-stride share, to FP64 accuracy. FP32 entries are
-// squared and summed as pairs of floats (x^2 = p + e exactly, hi + lo += p + e by TwoSum: the pair's own rounding
-// stays near 2^-48), because a conversion and an FMA per entry on the FP64 pipe cost more than reading the tensor
-// (D = 8: 67 us against 10).
+// Pass 1: each block writes the FP64 sum of squares of its grid-stride share. The FP64 pipe bounds it for FP32 entries
+// (a conversion and an FMA per entry, 67 us at D = 8 against 10 to read the tensor), so they are widened by their bits;
+// only infinities, NaN and subnormal entries take the conversion.
 constexpr int kNormBlocks = kNormPartials;
 
-template <typename R>
-struct SumSq {
-  double s;
-  __device__ __forceinline__ void add(R x) { s = fma(x, x, s); }
-  __device__ __forceinline__ void merge(const SumSq& o) { s += o.s; }
-  __device__ __forceinline__ SumSq down(int off) const {
-    SumSq o;
-    o.s = __shfl_down_sync(0xffffffffu, s, off);
-    return o;
-  }
-  __device__ __forceinline__ double value() const { return s; }
-};
-template <>
-struct SumSq<float> {
-  float hi, lo;
-  __device__ __forceinline__ void add(float x) {
-    const float p = x * x;
-    plus(p, fmaf(x, x, -p));
-  }
-  __device__ __forceinline__ void plus(float p, float e) {
-    const float t = hi + p, bp = t - hi;
-    lo += ((hi - (t - bp)) + (p - bp)) + e;
-    hi = t;
-  }
-  __device__ __forceinline__ void merge(const SumSq& o) { plus(o.hi, o.lo); }
-  __device__ __forceinline__ SumSq down(int off) const {
-    SumSq o;
-    o.hi = __shfl_down_sync(0xffffffffu, hi, off);
-    o.lo = __shfl_down_sync(0xffffffffu, lo, off);
-    return o;
-  }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
+__device__ __forceinline__ double exact_double(double x) { return x; }
+__device__ __forceinline__ double exact_double(float x) {
+  const uint32_t b = __float_as_uint(x), e = b >> 23 & 0xffu;
+  if (e == 0xffu || (e == 0u && (b << 1) != 0u)) return (double)x;
+  const uint32_t hi = (b & 0x80000000u) | (e ? ((b & 0x7fffffffu) >> 3) + (896u << 20) : 0u);   // 896 = 1023 - 127
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
 
 template <typename R>
 __global__ void __launch_bounds__(256) sumsq_kernel(const R* __restrict__ x, int64_t n, int64_t xstride,
                                                     double* partial) {
   x += blockIdx.y * xstride;                   // batch element blockIdx.y
   partial += blockIdx.y * gridDim.x;
-  SumSq<R> sum[4] = {};                        // four entries in flight
+  double sum[4] = {0, 0, 0, 0};                // four entries in flight
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += 4 * step) {
     R v[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) v[u] = i + u * step < n ? x[i + u * step] : (R)0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) sum[u].add(v[u]);
+    for (int u = 0; u < 4; ++u) {
+      const double d = exact_double(v[u]);
+      sum[u] = fma(d, d, sum[u]);
+    }
   }
-  sum[0].merge(sum[1]);
-  sum[2].merge(sum[3]);
-  sum[0].merge(sum[2]);
-  for (int off = 16; off > 0; off >>= 1) sum[0].merge(sum[0].down(off));
-  __shared__ SumSq<R> w[8];
-  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = sum[0];
+  double acc = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+  __shared__ double w[8];
+  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = acc;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int j = 1; j < 8; ++j) sum[0].merge(w[j]);
-    partial[blockIdx.x] = sum[0].value();
+    double s = 0;
+    for (int j = 0; j < 8; ++j) s += w[j];
+    partial[blockIdx.x] = s;
   }
 }
 
