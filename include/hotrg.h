@@ -234,6 +234,13 @@ hotrg_status hotrg_step_flops(const hotrg_ctx* ctx, int dir, int dcut, double* m
  *   that computes the second pass's outputs once more (largest entry in [2^14, 2^15)).
  *   0 = the fixed 2^14 of every operand. Other precisions ignore it (FP64OZ always scales
  *   by the exact largest magnitude, from a max pass).
+ * HOTRG_OPT_CHARGES: test option of runs without a field, whose bond indices carry a Z2 charge
+ *   (synchronises the stream; the next step sees the change). Bits 0..3: flip the charge of
+ *   every index of direction n's bond, a relabelling that moves no zero of the tensors (a
+ *   bond has two legs). Bit 4: drop the charges of every batch element, as an isometry column
+ *   that mixed them would: the contraction has one sector from then on, the dense product.
+ *   Either way the results stay the same up to rounding. Errors: ESTATE before
+ *   hotrg_init_tensor or with a field, ECUDA.
  * Errors: EINVAL. */
 enum {
   HOTRG_OPT_JACOBI_SWEEPS = 1,
@@ -241,7 +248,8 @@ enum {
   HOTRG_OPT_GRAPHS = 3,
   HOTRG_OPT_AUTOTUNE = 4,
   HOTRG_OPT_GROUP = 5,
-  HOTRG_OPT_MAXNORM = 6
+  HOTRG_OPT_MAXNORM = 6,
+  HOTRG_OPT_CHARGES = 7
 };
 hotrg_status hotrg_set_option(hotrg_ctx* ctx, int option, int value);
 

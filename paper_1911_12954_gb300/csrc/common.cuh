@@ -129,6 +129,7 @@ struct SectorPlan {           // per batch element of a group and step
   int n3[2];                  // rests (a2, a1', k) of charge q, made even by a filler
   uint32_t na, nb, nc;        // charges of the new a, b, c legs
   uint32_t mb, mc, mm;        // of the old b, c legs and of mu
+  int odd;                    // mask of every parity: 0 where the charges are dropped (one sector, the dense product)
 };
 struct SectorTables {
   uint32_t* row;              // operand row (X, Y, c, c', mu): rank within its charge, charge in bit 31

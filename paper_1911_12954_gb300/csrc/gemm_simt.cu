@@ -34,11 +34,11 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const R* __restrict__ A,
     const int c0 = p.row[0][s.xb + s.nb] - p.row[0][s.xb], c1 = p.row[1][s.xb + s.nb] - p.row[1][s.xb];
     const int64_t lim = s.row_limit > 0 ? s.row_limit : 0x7fffffff;
     const int64_t t0 = (min((int64_t)r0, lim) + kBM - 1) / kBM;
-    const int q = (int64_t)blockIdx.y >= t0, qc = q ^ one.parity;
+    const int q = (int64_t)blockIdx.y >= t0, qc = q ^ (one.parity & p.odd);
     if (q) m0 -= t0 * kBM;
     M = min((int64_t)(q ? r1 : r0), lim);
     N = qc ? c1 : c0;
-    K = p.K[q ^ one.pa];
+    K = p.K[q ^ (one.pa & p.odd)];
     if (m0 >= M || n0 >= N) return;
     A += (q ? (int64_t)r0 : 0) * lda;
     C += (q ? (int64_t)r0 : 0) * ldc;

@@ -334,15 +334,15 @@ struct Block {
 __device__ __forceinline__ Block sector_block(const SectorPlan& p, const GemmSectors& s, int q, int pa0, int pa1,
                                               int parity, int BK) {
   Block b;
-  const int qc = q ^ parity;
+  const int qc = q ^ (parity & p.odd);
   const int r0 = p.row[0][s.xa + s.na] - p.row[0][s.xa], n0 = p.row[0][s.xb + s.nb] - p.row[0][s.xb];
   b.rows = q ? p.row[1][s.xa + s.na] - p.row[1][s.xa] : r0;
   b.cols = qc ? p.row[1][s.xb + s.nb] - p.row[1][s.xb] : n0;
   if (s.row_limit > 0 && b.rows > s.row_limit) b.rows = (int)s.row_limit;
   b.a0 = b.c0 = q ? r0 : 0;
   b.b0 = qc ? n0 : 0;
-  b.nk[0] = (p.K[q ^ pa0] + BK - 1) / BK;
-  b.nk[1] = (p.K[q ^ pa1] + BK - 1) / BK;
+  b.nk[0] = (p.K[q ^ (pa0 & p.odd)] + BK - 1) / BK;
+  b.nk[1] = (p.K[q ^ (pa1 & p.odd)] + BK - 1) / BK;
   return b;
 }
 // The blocks of a sector launch and the first tile of each (tiles of TM x TN, blocks one after the

@@ -2160,6 +2160,23 @@ hotrg_status hotrg_set_option(hotrg_ctx* ctx, int option, int value) {
       ctx->maxnorm = value;
       ctx->drop_graphs();
       return HOTRG_OK;
+    case HOTRG_OPT_CHARGES: {
+      if (value < 0 || value > 31) return HOTRG_EINVAL;
+      if (!ctx->ready || !ctx->initialised || !ctx->sectors) return HOTRG_ESTATE;
+      std::vector<SectorState> s(ctx->batch);
+      SectorState* dev = (SectorState*)(ctx->ws + ctx->L.sectors);
+      const size_t bytes = s.size() * sizeof(SectorState);
+      CK(cudaMemcpyAsync(s.data(), dev, bytes, cudaMemcpyDeviceToHost, ctx->stream), "charges read");
+      CK(cudaStreamSynchronize(ctx->stream), "charges sync");
+      for (SectorState& e : s) {
+        for (int n = 0; n < 4; ++n)
+          if ((value >> n) & 1) e.charge[ctx->cur][n] ^= (1u << ctx->dims[n]) - 1u;
+        if (value & 16) e.dropped = 1;
+      }
+      CK(cudaMemcpyAsync(dev, s.data(), bytes, cudaMemcpyHostToDevice, ctx->stream), "charges write");
+      CK(cudaStreamSynchronize(ctx->stream), "charges sync");
+      return HOTRG_OK;
+    }
     default:
       return HOTRG_EINVAL;
   }

@@ -17,7 +17,7 @@
 // nonzero summed indices packed to the front of its K panels (zero filled up to a k-block), so
 // the buffers, the tensor maps and the GEMM pipelines are those of the dense product.
 // An isometry column that mixes charges (which exact arithmetic excludes) drops the element to
-// "every charge 0" (SectorState::dropped): one sector, the dense product.
+// "every charge 0, every parity 0" (SectorState::dropped, SectorPlan::odd): one sector, the dense product.
 //
 // Sums run over the nonzero terms in the order of the dense passes, so operands, C entries
 // given the same k order, and closed tensors are bit-identical to the dense passes'.
@@ -145,6 +145,7 @@ __global__ void __launch_bounds__(256) sector_tables_kernel(SectorArgs a) {
     p.mb = mb;
     p.mc = mc;
     p.mm = mm;
+    p.odd = st.dropped ? 0 : 1;
   }
 }
 
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(256) sector_operand_kernel(const __grid_consta
     r4 /= a.Dc;
     const int c0 = r4 % a.Dc;
     const int X = r4 / a.Dc;
-    const int qo = bit(na, a.x0 + X) ^ bit(mc, c0) ^ bit(mc, c1) ^ bit(mm, m) ^ a.parity;
+    const int qo = bit(na, a.x0 + X) ^ bit(mc, c0) ^ bit(mc, c1) ^ bit(mm, m) ^ (a.parity & p.odd);
     if (threadIdx.x < a.cb) {
       const int Y = threadIdx.x, q = bit(nb, Y);
       const uint32_t rk = t.row[((((int64_t)(a.x0 + X) * a.cb + Y) * a.Dc + c0) * a.Dc + c1) * a.Dm + m];
@@ -470,7 +471,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(R) * NZ > 64 ? 2 : 4) 
   const int64_t ocol = (tq ? n0 : 0) + gi;
   for (int rq = 0; rq < 2; ++rq) {
     const int gbase = p.grp[rq][a.x0], nrow = p.grp[rq][a.x0 + a.xs] - gbase;
-    const int s = rq ^ tq ^ a.parity;
+    const int s = rq ^ tq ^ (a.parity & p.odd);
     const int nzs = nz[s];
     if (nzs == 0) continue;
     for (int b = blockIdx.y * RG; b < nrow; b += gridDim.y * RG) {
@@ -600,7 +601,7 @@ __global__ void __launch_bounds__(256) sector_close2_kernel(const R* __restrict_
     for (int z = 0; z < NZ; ++z) acc[z] = 0;
     // charge of (c1', c2') that reaches a nonzero entry
     const int qm = (int)(t.grank[mg] >> 31) ^ bit(mc, 0), qn = (int)(t.grank[ng] >> 31) ^ bit(mc, 0);
-    const int s = qm ^ qn ^ bit(p.nc, Z) ^ a.parity;
+    const int s = qm ^ qn ^ bit(p.nc, Z) ^ (a.parity & p.odd);
     const R* o3 = O3 + (int64_t)Z * GR * GC;
     for (int c1 = 0; c1 < Dc; ++c1) {
       const uint32_t gr = t.grank[mg + c1 * a.Dm];

@@ -1019,7 +1019,7 @@ __global__ void __launch_bounds__(256) sector_stats_kernel(const __half* __restr
   const int64_t Kmax = max(p.K[0], p.K[1]), n = nrow * Kmax;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = i / Kmax, k = i - r * Kmax;
-    if (k >= p.K[(r < r0 ? 0 : 1) ^ parity]) continue;
+    if (k >= p.K[(r < r0 ? 0 : 1) ^ (parity & p.odd)]) continue;
     const unsigned a = __half_as_ushort(pl[(k / kps * rows + r) * kps + k % kps]) & 0x7fffu;
     nnz += a != 0u;
     ns += (a != 0u && a < 0x0400u);

@@ -18,7 +18,7 @@ from . import build as _build
 FP64, FP32, TF32X3, FP16X3, FP64OZ = 0, 1, 2, 3, 4
 PRECISIONS = {"fp64": FP64, "fp32": FP32, "tf32x3": TF32X3, "fp16x3": FP16X3, "fp64oz": FP64OZ}
 IMPURE_NONE, IMPURE_SIGMA, IMPURE_SIGMASIGMA = 0, 1, 2
-OPT_JACOBI_SWEEPS, OPT_GEMM_VARIANT, OPT_GRAPHS, OPT_AUTOTUNE, OPT_GROUP, OPT_MAXNORM = 1, 2, 3, 4, 5, 6
+OPT_JACOBI_SWEEPS, OPT_GEMM_VARIANT, OPT_GRAPHS, OPT_AUTOTUNE, OPT_GROUP, OPT_MAXNORM, OPT_CHARGES = 1, 2, 3, 4, 5, 6, 7
 
 STATUS = {0: "ok", -1: "EINVAL", -2: "EWORKSPACE", -3: "ECUDA", -4: "ENOCONV", -5: "ENONFINITE",
           -6: "ETIMEOUT", -7: "ESTATE", -8: "EUNSUPPORTED"}
