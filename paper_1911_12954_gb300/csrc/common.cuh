@@ -100,7 +100,8 @@ struct GramJob {
   int64_t K;                // product of rdims
   double* partial;          // [nchunks][R][R]
   int dir1, dir2, rdir[8];  // directions of the row legs and the summed legs
-  uint32_t rmagic[8];       // reciprocals of the summed leg sizes (filled in by launch_gram)
+  uint32_t rmagic[8];       // reciprocals of the summed leg sizes, and the directions of an odd number of summed
+  uint32_t unit;            // legs of one value (bit n: direction n; both filled in by launch_gram)
 };
 
 // One symmetric eigenproblem for the Jacobi kernel.

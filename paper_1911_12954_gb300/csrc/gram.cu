@@ -188,6 +188,10 @@ __global__ void __launch_bounds__(kGramThreads<R>, sizeof(R) == 8 ? 1 : 2)
   uint32_t rmask[8];
 #pragma unroll
   for (int d = 0; d < 8; ++d) rmask[d] = d < jb.nrest ? gram_mask(jobs, bidx, jb.rdir[d]) : 0u;
+  uint32_t unit = 0;                          // charge of the summed legs of one value
+#pragma unroll
+  for (int n = 0; n < 4; ++n)
+    if ((jb.unit >> n) & 1u) unit ^= gram_mask(jobs, bidx, n);
 
   for (int64_t kb = k0; kb < k1; kb += kGList) {
     // offsets of the indices of charge q among the next kGList, in increasing order (K <= 16^6 < 2^32: 32-bit
@@ -201,7 +205,7 @@ __global__ void __launch_bounds__(kGramThreads<R>, sizeof(R) == 8 ? 1 : 2)
     for (int it = 0; it < kIter; ++it) {
       const int64_t k = kb + it * kGThreads + tid;
       bool in = it * kGThreads + tid < kGList && k < k1;
-      uint32_t r = (uint32_t)k, o = 0, c = 0;
+      uint32_t r = (uint32_t)k, o = 0, c = unit;
 #pragma unroll
       for (int d = 7; d >= 0; --d) {
         if (d < jb.nrest) {
@@ -355,11 +359,16 @@ template <typename R>
 cudaError_t launch_gram(const GramPack& jobs, int njobs, int Rmax, int nchunks, cudaStream_t st) {
   GramPack p = jobs;
   for (int i = 0; i < njobs; ++i) {
-    // summed legs of one value leave; reciprocals ceil(2^32 / n) of the others (exact quotients below 2^28)
+    // summed legs of one value leave, but for their charge (unit); reciprocals ceil(2^32 / n) of the others (exact
+    // quotients below 2^28)
     GramJob& j = p.j[i];
     int n = 0;
+    j.unit = 0;
     for (int d = 0; d < j.nrest; ++d) {
-      if (j.rdims[d] == 1) continue;
+      if (j.rdims[d] == 1) {
+        j.unit ^= 1u << j.rdir[d];
+        continue;
+      }
       j.rdims[n] = j.rdims[d];
       j.rst[n] = j.rst[d];
       j.rdir[n] = j.rdir[d];
