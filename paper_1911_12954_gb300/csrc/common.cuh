@@ -18,9 +18,9 @@ constexpr int kJacobiLogSweeps = 10; // sweeps of rotations the eigensolver logs
 constexpr int64_t packed_doubles(int n) { return ((int64_t)n * (n + 1) / 2 + 1) / 2 * 2; }   // upper triangle, even
 // Doubles of global work space per matrix (EigJob::work): eigenvector columns, V (used when the log
 // overflows), the upper triangle of matrices that do not fit shared memory, the log of rotations (cosine and
-// tangent, the two indices): a sweep has at most n rounds of at most n pair slots. Even.
-constexpr int64_t jacobi_work_doubles(int n) {
-  const int64_t entries = (int64_t)kJacobiLogSweeps * n * n;
+// tangent, the two indices) of `sweeps` sweeps: a sweep has at most n rounds of at most n pair slots. Even.
+constexpr int64_t jacobi_work_doubles(int n, int sweeps = kJacobiLogSweeps) {
+  const int64_t entries = (int64_t)sweeps * n * n;
   return 2 * (int64_t)n * n + (n > kJacobiSmemN ? packed_doubles(n) : 0) + 2 * entries + (entries + 3) / 4 * 2;
 }
 
@@ -107,7 +107,7 @@ struct GramJob {
 // One symmetric eigenproblem for the Jacobi kernel.
 struct EigJob {
   const double* G;          // n x n, row-major, symmetric
-  double* work;             // jacobi_work_doubles(n) doubles of global scratch, 16-byte aligned
+  double* work;             // jacobi_work_doubles(n, EigPack::log_sweeps) doubles of global scratch, 16-byte aligned
   double* lam;              // n eigenvalues, descending
   double* U;                // n x chi, first chi eigenvectors in canonical gauge
   double* eps;              // sum of the discarded eigenvalues (index >= chi)
@@ -231,6 +231,7 @@ struct GramPack {
 struct EigPack {
   EigJob j[kMaxEigJobs];
   int batch = 1;
+  int log_sweeps = kJacobiLogSweeps;   // at least 1: what the work space holds
   int64_t sG = 0, sWork = 0, sLam = 0, sU = 0, sEps = 0, sDeg = 0;
 };
 struct SelectPack {

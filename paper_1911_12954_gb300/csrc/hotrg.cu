@@ -61,6 +61,7 @@ struct StepPlan {
   // Gram
   int R[4];               // rows of the half-Gram per direction = D_nu D_mu
   int Rmax, nmax, nchunks;
+  bool lean;              // isometry stage in the least space (see use_less)
   int batch;              // batch elements whose isometry stages run together
   int ne;                 // batch elements contracted together (one group of launches)
   bool sect;              // contraction by Z2 charge sectors (sectors.cu)
@@ -447,6 +448,16 @@ void use_sectors(StepPlan& p, int prec) {
   while (p.P * p.kps < most) p.kps += al;
 }
 
+// A plan whose isometry stage takes the least space, for workspaces that do not hold the ordinary one: a chunk of the
+// half-Grams per 512 summed indices, the eigenproblems one after the other with one sweep of logged rotations.
+void use_less(StepPlan& p) {
+  p.lean = true;
+  int64_t nc = std::min<int64_t>((p.E / p.Rmax + 511) / 512, 256);
+  const int64_t per = (int64_t)p.batch * kMaxGramJobs * p.Rmax * p.Rmax * 8;
+  while (nc > 1 && nc * per > (256LL << 20)) nc /= 2;
+  p.nchunks = (int)std::min<int64_t>(p.nchunks, nc);
+}
+
 int ntensors(int impure) { return (impure & HOTRG_IMPURE_SIGMASIGMA) ? 3 : ((impure & HOTRG_IMPURE_SIGMA) ? 2 : 1); }
 
 // Scratch bytes of one step with slice sizes xs (new X) and xs2 (new X').
@@ -456,6 +467,7 @@ struct Scratch {
   size_t tab;             // sector tables, one set per element of a group
   size_t amax;            // operand magnitude bounds of the current A and B per element (max-norm scaling)
   size_t stats;           // counters of hotrg_split_stats
+  int jne, jsweeps;       // elements whose eigenproblems run together (0: one matrix at a time), sweeps of their log
   size_t total;
 };
 
@@ -500,13 +512,10 @@ Scratch scratch_layout(const StepPlan& p, int xs, int xs2, int prec, int impure,
   s.Uside = take(nb * 6 * p.nmax * kMaxLeg * 8);
   const int64_t rowsA = (int64_t)xs * p.chi[p.b] * p.D[p.c] * p.D[p.c] * p.D[p.mu];
   const int64_t rowsB = (int64_t)xs2 * p.chi[p.b] * p.D[p.c] * p.D[p.c] * p.D[p.mu];
-  // the Gram partials and the eigensolver's work are done with before the contraction's buffers are
-  // written: they share that space
+  // the Gram partials, then the eigensolver's work, then the contraction's buffers share one space, each being
+  // done with before the next is written
   const size_t shared = off;
-  s.gpart = take(nb * kMaxGramJobs * p.nchunks * p.Rmax * p.Rmax * 8);
-  s.jwork = take(nb * 6 * (size_t)jacobi_work_doubles(p.nmax) * 8);
-  const size_t iso_end = off;
-  off = shared;
+  s.gpart = s.jwork = shared;
   const bool split = tc_mode(prec);
   const size_t os = operand_size(prec) * (prec == HOTRG_FP64OZ ? kOzSlices : 1);   // the slices of one operand
   // contraction: one copy per element of a group (p.ne elements contracted together)
@@ -522,7 +531,20 @@ Scratch scratch_layout(const StepPlan& p, int xs, int xs2, int prec, int impure,
   s.tab = p.sect ? take(ne * sector_tab(p).stride) : 0;
   s.amax = take(2 * ne * nt * sizeof(unsigned));   // A side, then B side: per element (and tensor)
   s.stats = take(4 * 3 * sizeof(unsigned long long));   // hotrg_split_stats counters
-  s.total = std::max(off, iso_end);
+  // as many elements' eigenproblems at a time as the others leave room for (1 MB where they are smaller: 50 elements
+  // at D = 2, two CTAs for every SM)
+  const size_t gbytes = nb * kMaxGramJobs * p.nchunks * p.Rmax * p.Rmax * 8;
+  size_t jbytes;
+  if (p.lean) {
+    s.jsweeps = 1;
+    jbytes = (size_t)jacobi_work_doubles(p.nmax, 1) * 8;
+  } else {
+    s.jsweeps = kJacobiLogSweeps;
+    const size_t one = 6 * (size_t)jacobi_work_doubles(p.nmax) * 8, room = std::max<size_t>(std::max(off - shared, gbytes), 1 << 20);
+    s.jne = (int)std::min(nb, std::max<size_t>(room / one, 1));
+    jbytes = s.jne * one;
+  }
+  s.total = std::max(off, shared + align_up(std::max(gbytes, jbytes), 256));
   return s;
 }
 
@@ -1101,7 +1123,7 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
   int* degen = (int*)(sb + sc.degen);
   double* Uside = (double*)(sb + sc.Uside);
   double* jwork = (double*)(sb + sc.jwork);
-  const int64_t jw = jacobi_work_doubles(p.nmax);
+  const int64_t jw = jacobi_work_doubles(p.nmax, sc.jsweeps);
   int nmax = 0;
   for (int i = 0; i < 3; ++i) {
     for (int side = 0; side < 2; ++side) {
@@ -1110,7 +1132,7 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
       j.n = p.D[dirs[i]] * p.D[dirs[i]];
       j.chi = p.chi[dirs[i]];
       j.G = G + (int64_t)e * nn;
-      j.work = jwork + e * jw;
+      j.work = jwork + (sc.jne > 0 ? e * jw : 0);
       j.lam = lam + (int64_t)e * p.nmax;
       j.eps = eps + e;
       j.degenerate = degen + e;
@@ -1118,7 +1140,7 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
       nmax = std::max(nmax, j.n);
     }
   }
-  ep.batch = nb;
+  ep.log_sweeps = sc.jsweeps;
   ep.sG = 6 * nn;
   ep.sWork = 6 * jw;
   ep.sLam = 6 * (int64_t)p.nmax;
@@ -1126,8 +1148,25 @@ hotrg_status isometry_stage(hotrg_ctx* ctx, const StepPlan& p, const Scratch& sc
   ep.sEps = 6;
   ep.sDeg = 6;
   const bool fp64 = f64_store(ctx->prec);
-  LK(1, launch_jacobi(ep, 6, nmax, fp64 ? 1e-10 : 1e-6, status, st, ctx->jacobi_sweeps, fp64 ? 1e-8 : 1e-4),
-     "jacobi");
+  // jobs [j0, j0 + njobs) of ne elements from e0 on
+  auto jacobi = [&](int e0, int ne, int j0, int njobs) {
+    EigPack q = ep;
+    q.batch = ne;
+    for (int i = 0; i < njobs; ++i) {
+      EigJob& j = q.j[i] = ep.j[j0 + i];
+      j.G += e0 * ep.sG;
+      j.lam += e0 * ep.sLam;
+      j.U += e0 * ep.sU;
+      j.eps += e0 * ep.sEps;
+      j.degenerate += e0 * ep.sDeg;
+    }
+    return launch_jacobi(q, njobs, nmax, fp64 ? 1e-10 : 1e-6, status, st, ctx->jacobi_sweeps, fp64 ? 1e-8 : 1e-4);
+  };
+  if (sc.jne > 0) {
+    for (int e0 = 0; e0 < nb; e0 += sc.jne) LK(1, jacobi(e0, std::min(sc.jne, nb - e0), 0, 6), "jacobi");
+  } else {
+    for (int q = 0; q < 6 * nb; ++q) LK(1, jacobi(q / 6, 1, q % 6, 1), "jacobi");
+  }
   SelectPack sp{};
   double* U64 = (double*)(ctx->ws + ctx->L.U64);
   R* Ur = (R*)(ctx->ws + ctx->L.Ur);
@@ -1518,17 +1557,22 @@ bool choose_slices(const hotrg_ctx* ctx, StepPlan& p) {
 }
 
 // Slices of a step of this run: by charge sectors where the tensors conserve the charge and the
-// workspace holds the sector tables too, dense otherwise.
+// workspace holds the sector tables too, dense otherwise; either with the ordinary isometry stage
+// where the workspace holds that.
 bool plan_slices(const hotrg_ctx* ctx, StepPlan& p) {
-  if (ctx->sectors) {
-    StepPlan s = p;
-    use_sectors(s, ctx->prec);
-    if (choose_slices(ctx, s)) {
-      p = s;
-      return true;
+  for (const bool sect : {true, false}) {
+    if (sect && !ctx->sectors) continue;
+    for (const bool lean : {false, true}) {
+      StepPlan s = p;
+      if (sect) use_sectors(s, ctx->prec);
+      if (lean) use_less(s);
+      if (choose_slices(ctx, s)) {
+        p = s;
+        return true;
+      }
     }
   }
-  return choose_slices(ctx, p);
+  return false;
 }
 
 // ---------------------------------------------------------------------------- autotuner
@@ -1924,9 +1968,9 @@ hotrg_status hotrg_step(hotrg_ctx* ctx, int dir, int dcut) {
     // which buffer holds the tensors, whether it is the first step (M_1 = C(S,S)) and the
     // impure tensors in use. ln c / 2^k and the record slot come from the device counter.
     char key[256];
-    snprintf(key, sizeof(key), "%d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d", dir, dcut, ctx->dims[0],
+    snprintf(key, sizeof(key), "%d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d", dir, dcut, ctx->dims[0],
              ctx->dims[1], ctx->dims[2], ctx->dims[3], ctx->cur, ctx->k == 0, ctx->impure_active, p.xs, p.xs2,
-             ctx->batch, p.c, p.gemm_opt, p.ne, ctx->sectors ? 1 : 0, p.sect ? 1 : 0);
+             ctx->batch, p.c, p.gemm_opt, p.ne, ctx->sectors ? 1 : 0, p.sect ? 1 : 0, p.lean ? 1 : 0);
     auto it = ctx->graphs.find(key);
     if (it == ctx->graphs.end()) {
       const uint64_t l0 = ctx->launches;

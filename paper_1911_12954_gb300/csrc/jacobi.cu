@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
   double* V = W + (int64_t)n * n;          // [n][n], rows
   double* Aw = V + (int64_t)n * n;
   double2* log = (double2*)(Aw + (use_smem ? 0 : packed_doubles(n)));
-  short2* logi = (short2*)(log + (int64_t)kJacobiLogSweeps * n * n);
+  short2* logi = (short2*)(log + (int64_t)jobs.log_sweeps * n * n);
   double* A = use_smem ? dyn : Aw;         // use_smem: every job of the launch has n <= kJacobiSmemN
   uint32_t* blk = (uint32_t*)(dyn + region);
 
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
 
   int sweep = 0;
   for (; sweep < max_sweeps && n > 1; ++sweep) {
-    if (nlog + rounds > kJacobiLogSweeps * n) fold_log();
+    if (nlog + rounds > jobs.log_sweeps * n) fold_log();
     const int nlog0 = nlog;
     for (int r = 0; r < rounds; ++r) {
       int rot = 0;
