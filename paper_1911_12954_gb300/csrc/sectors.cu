@@ -21,6 +21,7 @@
 //
 // Sums run over the nonzero terms in the order of the dense passes, so operands, C entries
 // given the same k order, and closed tensors are bit-identical to the dense passes'.
+#include <mutex>
 #include <type_traits>
 
 #include "common.cuh"
@@ -668,21 +669,23 @@ template cudaError_t launch_sector_close<float>(const float*, const float*, floa
 template cudaError_t launch_sector_close<double>(const double*, const double*, double*, double*, const SectorClose&, int,
                                                  cudaStream_t);
 
+// Once per device; a thread that finds another one at it waits until the attributes are set.
 void sectors_prepare() {
-  static bool done[64] = {};
+  static std::once_flag once[64];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || done[dev]) return;
-  done[dev] = true;
-  auto set = [](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSectorSmem); };
-  set(sector_operand_kernel<double, kTTMStore, 16>);
-  set(sector_operand_kernel<double, kTTMMaxAbs, 16>);
-  set(sector_operand_kernel<double, kTTMSplitOz, 16>);
-  set(sector_close1_kernel<float, 16, 128>);
-  set(sector_close1_kernel<float, 16, 256>);
-  set(sector_close1_kernel<double, 8, 128>);
-  set(sector_close1_kernel<double, 16, 128>);
-  set(sector_close2_kernel<double, 16>);
-  cudaGetLastError();
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+  std::call_once(once[dev], [] {
+    auto set = [](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSectorSmem); };
+    set(sector_operand_kernel<double, kTTMStore, 16>);
+    set(sector_operand_kernel<double, kTTMMaxAbs, 16>);
+    set(sector_operand_kernel<double, kTTMSplitOz, 16>);
+    set(sector_close1_kernel<float, 16, 128>);
+    set(sector_close1_kernel<float, 16, 256>);
+    set(sector_close1_kernel<double, 8, 128>);
+    set(sector_close1_kernel<double, 16, 128>);
+    set(sector_close2_kernel<double, 16>);
+    cudaGetLastError();
+  });
 }
 
 }  // namespace hotrg

@@ -15,6 +15,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <mutex>
 #include <type_traits>
 
 #include "common.cuh"
@@ -451,15 +452,17 @@ size_t dense_split_smem(const DenseSplit& a, int n2) {
 }
 constexpr size_t kDenseSplitSmem = 100 * 1024;   // two blocks per SM
 
+// Once per device; a thread that finds another one at it waits until the attributes are set.
 void tensor_ops_prepare() {
-  static bool done[64] = {};
+  static std::once_flag once[64];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || done[dev]) return;
-  done[dev] = true;
-  auto set = [](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSplitSmem); };
-  set(dense_split_kernel<4>);
-  set(dense_split_kernel<8>);
-  cudaGetLastError();
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+  std::call_once(once[dev], [] {
+    auto set = [](auto k) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSplitSmem); };
+    set(dense_split_kernel<4>);
+    set(dense_split_kernel<8>);
+    cudaGetLastError();
+  });
 }
 
 // Sets a.n2 and says whether the form applies: an odd extent somewhere in the innermost legs (even ones take the paired
