@@ -176,6 +176,12 @@ hotrg_status hotrg_x_indicator(hotrg_ctx* ctx, int nu, double* X);
 /* Record of step `step` (1-based, <= steps done) of batch element b. Synchronises. */
 hotrg_status hotrg_step_info(hotrg_ctx* ctx, int b, int step, hotrg_step_record* rec);
 
+/* Share of the multiply-adds of step `step`'s block-spin products (2 M N K flops each, of batch
+ * element b, over every tensor) that the step executes: 1 for a dense contraction; where the
+ * contraction ran by Z2 charge sectors, the blocks that are not zero by the charge, from the
+ * sizes of the sectors (near 1/4). Tile padding is not counted. Synchronises. */
+hotrg_status hotrg_product_share(hotrg_ctx* ctx, int b, int step, double* share);
+
 /* Number of steps done since the last init/set_tensor; current bond dimensions. */
 hotrg_status hotrg_state(const hotrg_ctx* ctx, int* steps_done, int dims[4]);
 
@@ -284,7 +290,8 @@ typedef struct {
   uint64_t launches;      /* CUDA kernels this context launched since the last reset         */
   uint64_t gemm_launches; /* launches of the block-spin GEMM (the O(D^15) product)            */
   double gemm_ms;         /* their summed device time, CUDA events on the context's stream   */
-  double gemm_flops;      /* their summed algorithmic flops, 2 M N K each                    */
+  double gemm_flops;      /* their summed algorithmic flops, 2 M N K each, of which a step by
+                             charge sectors executes hotrg_product_share                     */
 } hotrg_profile;
 
 /* enable != 0: from now on record a CUDA event pair around every GEMM launch (host-side

@@ -155,6 +155,13 @@ struct SectorArgs {           // sector_tables_kernel
   int cur;                    // buffer of the tensors before the step
   int a, b, c, mu;            // directions
   int Da, Db, Dc, Dm, ca, cb;
+  struct DevRecord* rec;      // of the group's first element: record *step takes the sizes of the sectors
+  const int* step;
+};
+struct SectorCount {          // sizes of a step's sectors (DevRecord::eps[mu])
+  int rows0, rests0;          // operand rows and rests (a2, a1', k) of charge 0
+  int odd_b;                  // indices of the old b leg of charge 1
+  int odd;                    // SectorPlan::odd
 };
 struct SectorOperand {        // second half-contraction pass of one tensor
   SectorTab tab;
@@ -206,7 +213,7 @@ struct SelectJob {
 
 // Step record as kept on the device for each batch element and step.
 struct DevRecord {
-  double eps[4][2];
+  double eps[4][2];   // of direction mu: the step's SectorCount
   double ln_c;
   int primed[4];
   int degen[4];

@@ -115,6 +115,10 @@ struct hotrg_ctx {
   int c_hist[kMaxSteps];       // closing direction of each step
   int opt_hist[kMaxSteps];     // GEMM pipeline option of each step (-1: CUDA cores)
   int tuned_hist[kMaxSteps];   // plan from the autotuner's cache
+  struct ProductSize {
+    int rows, rests, Db, nt;   // rests: (a2, a1', k); nt: tensors (0: a dense contraction)
+  };
+  ProductSize size_hist[kMaxSteps];   // of the contraction by charge sectors of each step
   uint64_t tune_timed = 0;     // step shapes timed by this context
   uint64_t tune_hits = 0;      // steps whose plan came from the cache
   struct GraphEntry {
@@ -1306,6 +1310,8 @@ hotrg_status contract_group(hotrg_ctx* ctx, const StepPlan& p, int e0, int ne, c
       a.Dm = p.D[mu];
       a.ca = ca;
       a.cb = p.chi[p.b];
+      a.rec = (DevRecord*)(ctx->ws + ctx->L.rec) + (int64_t)e0 * kMaxSteps;
+      a.step = (const int*)(ctx->ws + ctx->L.step);
       LK(1, launch_sector_tables(a, ne, st), "sector tables");
     }
     const int parity[3] = {0, 1, 0};   // T, S (one sigma: odd), M (two)
@@ -2000,6 +2006,7 @@ hotrg_status hotrg_step(hotrg_ctx* ctx, int dir, int dcut) {
   ctx->opt_hist[ctx->k] = tc_mode(ctx->prec) ? (p.gemm_opt >= 0 ? p.gemm_opt : ctx->gemm_variant) : -1;
   ctx->tuned_hist[ctx->k] = p.tuned ? 1 : 0;
   ctx->group_hist[ctx->k] = p.ne;
+  ctx->size_hist[ctx->k] = {(int)p.rowsA_full, p.D[p.a] * p.D[p.a] * p.D[dir], p.D[p.b], p.sect ? ntensors(ctx->impure_active) : 0};
   ctx->slices_hist[ctx->k][0] = (p.chi[p.a] + p.xs - 1) / p.xs;
   ctx->slices_hist[ctx->k][1] = (p.chi[p.a] + p.xs2 - 1) / p.xs2;
   for (int n = 0; n < 4; ++n) {
@@ -2117,6 +2124,7 @@ hotrg_status hotrg_step_info(hotrg_ctx* ctx, int b, int step, hotrg_step_record*
     rec->dims[n] = ctx->dims_hist[step - 1][n];
     rec->primed[n] = d.primed[n];
     rec->degenerate[n] = d.degen[n];
+    if (n == rec->mu) continue;   // (holds hotrg_product_share)
     rec->eps[n][0] = d.eps[n][0];
     rec->eps[n][1] = d.eps[n][1];
   }
@@ -2127,6 +2135,34 @@ hotrg_status hotrg_step_info(hotrg_ctx* ctx, int b, int step, hotrg_step_record*
   rec->gemm_option = ctx->opt_hist[step - 1];
   rec->tuned = ctx->tuned_hist[step - 1];
   rec->group = ctx->group_hist[step - 1];
+  return HOTRG_OK;
+}
+
+hotrg_status hotrg_product_share(hotrg_ctx* ctx, int b, int step, double* share) {
+  hotrg_status r = check_ready(ctx);
+  if (r != HOTRG_OK) return r;
+  if (!share || b < 0 || b >= ctx->batch || step < 1 || step > ctx->k) return HOTRG_EINVAL;
+  *share = 1.0;
+  const hotrg_ctx::ProductSize& z = ctx->size_hist[step - 1];
+  if (z.nt == 0) return HOTRG_OK;
+  SectorCount c;
+  const DevRecord* rec = (const DevRecord*)(ctx->ws + ctx->L.rec) + (int64_t)b * kMaxSteps + (step - 1);
+  CK(cudaMemcpyAsync(&c, rec->eps[ctx->mu_hist[step - 1]], sizeof(c), cudaMemcpyDeviceToHost, ctx->stream), "share read");
+  CK(cudaStreamSynchronize(ctx->stream), "sync");
+  // rows of charge q against columns of charge q + the output's parity over the summed indices of charge q + A's
+  // parity, for T, S (two products) and M (one at the first step, then two)
+  const double R[2] = {(double)c.rows0, (double)(z.rows - c.rows0)}, S[2] = {(double)c.rests0, (double)(z.rests - c.rests0)};
+  const double b0 = z.Db - c.odd_b, b1 = c.odd_b, even = b0 * b0 + b1 * b1, odd = 2 * b0 * b1;
+  const double K[2] = {even * S[0] + odd * S[1], even * S[1] + odd * S[0]};
+  auto part = [&](int pa, int par) {
+    pa &= c.odd;
+    par &= c.odd;
+    return R[0] * R[par] * K[pa] + R[1] * R[1 ^ par] * K[1 ^ pa];
+  };
+  double sum = part(0, 0), n = 1;
+  if (z.nt >= 2) sum += part(1, 1) + part(0, 1), n += 2;
+  if (z.nt >= 3) sum += step == 1 ? part(1, 0) : 2 * part(0, 0), n += step == 1 ? 1 : 2;
+  *share = sum / (n * z.rows * z.rows * (K[0] + K[1]));
   return HOTRG_OK;
 }
 

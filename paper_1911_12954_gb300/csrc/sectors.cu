@@ -147,6 +147,8 @@ __global__ void __launch_bounds__(256) sector_tables_kernel(SectorArgs a) {
     p.mc = mc;
     p.mm = mm;
     p.odd = st.dropped ? 0 : 1;
+    const int k = *a.step;
+    if (k < kMaxSteps) *(SectorCount*)a.rec[(int64_t)e * kMaxSteps + k].eps[a.mu] = SectorCount{p.row[0][a.ca], S0, b1, p.odd};
   }
 }
 

@@ -53,7 +53,7 @@ class SplitStats(ctypes.Structure):
 _LIB = None
 SYMBOLS = ["hotrg_create", "hotrg_destroy", "hotrg_workspace_size", "hotrg_set_workspace", "hotrg_set_stream",
            "hotrg_init_tensor", "hotrg_set_tensor", "hotrg_step", "hotrg_lnZ", "hotrg_impure_magnetization",
-           "hotrg_impure_energy", "hotrg_x_indicator", "hotrg_step_info", "hotrg_state", "hotrg_copy_tensor",
+           "hotrg_impure_energy", "hotrg_x_indicator", "hotrg_step_info", "hotrg_product_share", "hotrg_state", "hotrg_copy_tensor",
            "hotrg_copy_isometry", "hotrg_step_flops", "hotrg_set_option", "hotrg_selftest_wait", "hotrg_profile_enable",
            "hotrg_profile_read", "hotrg_isometry_noalloc", "hotrg_autotune", "hotrg_tune_stats", "hotrg_split_stats",
            "hotrg_status_string", "hotrg_last_error"]
@@ -86,6 +86,7 @@ def _lib():
         "hotrg_impure_energy": (c_int, [c_void_p, P(c_double), P(c_double)]),
         "hotrg_x_indicator": (c_int, [c_void_p, c_int, P(c_double)]),
         "hotrg_step_info": (c_int, [c_void_p, c_int, c_int, P(StepRecord)]),
+        "hotrg_product_share": (c_int, [c_void_p, c_int, c_int, P(c_double)]),
         "hotrg_state": (c_int, [c_void_p, P(c_int), P(c_int)]),
         "hotrg_copy_tensor": (c_int, [c_void_p, c_int, c_int, P(c_double), c_size_t]),
         "hotrg_copy_isometry": (c_int, [c_void_p, c_int, c_int, P(c_double), c_size_t]),
@@ -254,6 +255,12 @@ class HOTRG:
                     eps=tuple(tuple(r.eps[n]) for n in range(4)), ln_c=r.ln_c,
                     degenerate=tuple(r.degenerate), slices=tuple(r.slices), closing=r.closing,
                     gemm_option=r.gemm_option, tuned=bool(r.tuned), group=r.group)
+
+    def product_share(self, step: int, b: int = 0) -> float:
+        """Share of step's block-spin product that was executed: 1 dense, near 1/4 by charge sectors."""
+        out = ctypes.c_double()
+        _check(self.lib.hotrg_product_share(self.ctx, b, step, ctypes.byref(out)), "product_share")
+        return out.value
 
     def tensor(self, which: int = 0, b: int = 0) -> np.ndarray:
         _, dims = self.state()
