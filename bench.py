@@ -119,7 +119,8 @@ def kernel_name(precision: str, option: int) -> str:
         return {0: "gemm_pair_kernel<CfgF16P> (CTA pairs, tcgen05.mma.cta_group::2)",
                 1: "gemm_tf32x3_kernel<CfgF16S>", 2: "gemm_tf32x3_kernel<CfgF16L>",
                 3: "gemm_tf32x3_kernel<CfgF16>"}[option]
-    return {0: "gemm_tf32x3_kernel<CfgTF32>", 1: "gemm_tf32x3_kernel<CfgTF32W>"}.get(option, "gemm_simt_kernel")
+    return {0: "gemm_pair_kernel<CfgTF32P> (CTA pairs, tcgen05.mma.cta_group::2)",
+            1: "gemm_tf32x3_kernel<CfgTF32W>"}.get(option, "gemm_simt_kernel")
 
 
 class ClockSampler:
@@ -436,6 +437,8 @@ def main():
     plans = [{"step": k, **{f: run.step_info(k)[f] for f in ("mu", "closing", "gemm_option", "tuned", "group")}}
              for k in range(args.warmup + 1, nsteps + 1)]
     tune = run.tune_stats()
+    shares = [run.product_share(k, b) for k in range(args.warmup + 1, nsteps + 1) for b in range(args.batch)]
+    executed = sum(shares) / len(shares) if shares else 1.0
     # --steps 0: the warm-up steps and the accuracy runs only (no timed region, no throughput)
     value, ms_max = sync.throughput(flops, start.elapsed_time(stop)) if args.steps > 0 else (None, None)
     lnz_run = [float(x) for x in run.lnZ()]
@@ -635,9 +638,8 @@ def main():
 
     peak, peak_src = tensor_peak(args.precision, True)
     peak_burst, _ = tensor_peak(args.precision, False)
-    # without a field only the nonzero charge blocks of the product run: rows, columns and summed
-    # indices split in halves (to within a few percent), two blocks of an eighth
-    executed = 0.25 if hfield == 0.0 else 1.0
+    # without a field only the nonzero charge blocks of the product run; `executed` is their share of the timed
+    # steps' products, from the sizes of the sectors (1: dense contractions)
     achieved = executed * prof["gemm_flops"] / (prof["gemm_ms"] * 1e-3) / 1e12 if prof["gemm_ms"] > 0 else None
     traffic = GEMM_TRAFFIC.get((args.precision, args.gemm_variant, D, args.batch, bool(impure)))
     line = {
@@ -653,7 +655,9 @@ def main():
                              f"{(4 if args.precision == 'fp16x3' else 8) * D ** 10 / 1e9:.1f} GB per step, hi + lo)"},
         "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": (achieved / peak) if achieved else None, "traffic": traffic,
-                     "algorithmic_bytes": (2 * (4 if args.precision == "fp16x3" else 8) + 4) * float(D) ** 10,
+                     # of one product; by sectors about half of every operand and of C is not zero
+                     "algorithmic_bytes": ((2 * (4 if args.precision == "fp16x3" else 8) + 4) * float(D) ** 10
+                                           * (0.5 if executed < 0.9 else 1.0)),
                      "kernel": " + ".join(sorted({kernel_name(args.precision, pl["gemm_option"]) for pl in plans}))
                                + " (block-spin contraction, 2 M N K x executed_flops_share flops per launch)",
                      "peak_source": peak_src, "launches": prof["gemm_launches"],
