@@ -1902,27 +1902,31 @@ hotrg_status hotrg_set_tensor(hotrg_ctx* ctx, int b, const int dims[4], const do
   const double c = sqrt(((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7])));
   if (!(c > 0) || !isfinite(c)) return HOTRG_EINVAL;
   cudaStream_t st = ctx->stream;
-  CK(cudaStreamSynchronize(st), "set_tensor sync");
+  // on the context's own stream, which need not wait for work on the default one
   if (b == 0) {
-    CK(cudaMemset(ctx->ws + ctx->L.status, 0, kStWords * 4), "status");
-    CK(cudaMemset(ctx->ws + ctx->L.step, 0, sizeof(int)), "step");
-    CK(cudaMemset(ctx->ws + ctx->L.rec, 0, (size_t)ctx->batch * kMaxSteps * sizeof(DevRecord)), "rec");
+    CK(cudaMemsetAsync(ctx->ws + ctx->L.status, 0, kStWords * 4, st), "status");
+    CK(cudaMemsetAsync(ctx->ws + ctx->L.step, 0, sizeof(int), st), "step");
+    CK(cudaMemsetAsync(ctx->ws + ctx->L.rec, 0, (size_t)ctx->batch * kMaxSteps * sizeof(DevRecord), st),
+       "rec");
     ctx->cur = 0;
   }
   if (f64_store(ctx->prec)) {
     HostStage stage(ctx, E * 8);
     double* tmp = (double*)stage.p;
     for (int64_t i = 0; i < E; ++i) tmp[i] = T_host[i] / c;
-    CK(cudaMemcpy(tensor_ptr<double>(ctx, 0, ctx->cur, b), tmp, E * 8, cudaMemcpyHostToDevice), "upload");
+    CK(cudaMemcpyAsync(tensor_ptr<double>(ctx, 0, ctx->cur, b), tmp, E * 8, cudaMemcpyHostToDevice, st), "upload");
+    CK(cudaStreamSynchronize(st), "upload sync");
   } else {
     HostStage stage(ctx, E * 4);
     float* tmp = (float*)stage.p;
     const double inv = 1.0 / c;
     for (int64_t i = 0; i < E; ++i) tmp[i] = (float)(T_host[i] * inv);
-    CK(cudaMemcpy(tensor_ptr<float>(ctx, 0, ctx->cur, b), tmp, E * 4, cudaMemcpyHostToDevice), "upload");
+    CK(cudaMemcpyAsync(tensor_ptr<float>(ctx, 0, ctx->cur, b), tmp, E * 4, cudaMemcpyHostToDevice, st), "upload");
+    CK(cudaStreamSynchronize(st), "upload sync");
   }
   const double lc = log(c);
-  CK(cudaMemcpy((double*)(ctx->ws + ctx->L.lnz) + b, &lc, 8, cudaMemcpyHostToDevice), "lnz");
+  CK(cudaMemcpyAsync((double*)(ctx->ws + ctx->L.lnz) + b, &lc, 8, cudaMemcpyHostToDevice, st), "lnz");
+  CK(cudaStreamSynchronize(st), "set_tensor sync");
   ctx->impure_active = 0;
   ctx->sectors = false;
   for (int n = 0; n < 4; ++n) ctx->dims[n] = dims[n];
