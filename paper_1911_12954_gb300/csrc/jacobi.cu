@@ -302,8 +302,8 @@ __global__ void __launch_bounds__(kJT) jacobi_kernel(const __grid_constant__ Eig
           if (rotates(apq, app, aqq)) {
             // tangent of the small rotation angle, t = 2 a_pq / (d + sign(d) sqrt(d^2 + 4 a_pq^2)), to FP32 accuracy
             // (any t gives an orthogonal rotation; the entry left over, 2^-22 of a_pq, goes with the next sweep), and
-            // c = 1 / sqrt(1 + t^2) to FP64 accuracy from an FP32 start r (1 - x r^2 = e, |e| < 2^-20: the next
-            // term of the series is 5/16 e^3)
+            // c = 1 / sqrt(1 + t^2) to FP64 accuracy from an FP32 start r by the binomial series of (1 - e)^(-1/2) =
+            // 1 + e/2 + 3/8 e^2 + 5/16 e^3 + ..., 1 - e = (1 + t^2) r^2, |e| < 2^-20: two terms are enough
             d = aqq - app;
             const int ed = (__double2hiint(d) >> 20) & 0x7ff, eb = (__double2hiint(apq) >> 20) & 0x7ff;
             float tf;
