@@ -26,3 +26,20 @@ def test_ln_c_of_a_tiny_coarse_tensor(precision, eps):
     g.x_indicator()                          # raises if the norm was found not finite or zero
     assert abs(g.step_info(1)["ln_c"] - want) < 1e-5
     assert np.linalg.norm(g.tensor()) == pytest.approx(1.0, abs=1e-5)
+
+
+@pytest.mark.parametrize("eps", [1e-36, 1e-37])
+def test_ln_c_with_subnormal_entries(eps):
+    """The same with entries of T' below FP32's normal range (eps / 100 of 2^-149 = 1.4e-45): 60 roundings of
+    half a quantum are 3e-5 of such an entry, 1e-4 on ln c."""
+    from paper_1911_12954_gb300 import HOTRG
+
+    R = np.random.default_rng(2).uniform(0.5, 1.5, (2,) * 6)
+    T = np.zeros((2,) * 8)
+    T[0, 1], T[1, 0] = R, eps * R
+    T /= np.linalg.norm(T)
+    want = np.log(np.linalg.norm(np.tensordot(T, T, axes=(1, 0))))
+    g = HOTRG(batch=1, dcut_max=4, precision="fp32", schedule=[(0, 4)], dims0=(2, 2, 2, 2))
+    g.set_tensor(T)
+    g.step(0, 4)
+    assert abs(g.step_info(1)["ln_c"] - want) < 1e-4
