@@ -121,6 +121,12 @@ __global__ void __launch_bounds__(256) sector_tables_kernel(SectorArgs a) {
       t.grp[(int)(r & 0x7fffffffu) + ((r >> 31) ? G0 : 0)] = (uint32_t)g;
     }
   }
+  if (blockIdx.x == 0 && threadIdx.x == 32) {
+    const int k = *a.step;
+    if (k < kMaxSteps)
+      *(SectorCount*)a.rec[(int64_t)e * kMaxSteps + k].eps[a.mu] =
+          SectorCount{even_count(rd, rm, 0), S0, odd_below(mb, a.Db), st.dropped ? 0 : 1};
+  }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     SectorPlan& p = *t.plan;
     const int r0 = even_count(rd, rm, 1), r1 = rows / a.ca - r0;   // rows of one X by the other legs' charge
@@ -147,8 +153,6 @@ __global__ void __launch_bounds__(256) sector_tables_kernel(SectorArgs a) {
     p.mc = mc;
     p.mm = mm;
     p.odd = st.dropped ? 0 : 1;
-    const int k = *a.step;
-    if (k < kMaxSteps) *(SectorCount*)a.rec[(int64_t)e * kMaxSteps + k].eps[a.mu] = SectorCount{p.row[0][a.ca], S0, b1, p.odd};
   }
 }
 
@@ -268,6 +272,7 @@ __global__ void __launch_bounds__(256) sector_operand_kernel(const __grid_consta
   __shared__ OperandShared sh;
   const int Db = a.Db, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const uint32_t mb = p.mb, nb = p.nb, na = p.na, mc = p.mc, mm = p.mm;
+  const int parity = a.parity & p.odd;
   const int ny1 = odd_below(nb, a.cb), ny0 = a.cb - ny1, nj1 = odd_below(mb, Db), nj0 = Db - nj1;
   // slots of j: the counts that operand_run is built for (see the switch below)
   int NJp = max(nj0, nj1);
@@ -310,7 +315,7 @@ __global__ void __launch_bounds__(256) sector_operand_kernel(const __grid_consta
     r4 /= a.Dc;
     const int c0 = r4 % a.Dc;
     const int X = r4 / a.Dc;
-    const int qo = bit(na, a.x0 + X) ^ bit(mc, c0) ^ bit(mc, c1) ^ bit(mm, m) ^ (a.parity & p.odd);
+    const int qo = bit(na, a.x0 + X) ^ bit(mc, c0) ^ bit(mc, c1) ^ bit(mm, m) ^ parity;
     if (threadIdx.x < a.cb) {
       const int Y = threadIdx.x, q = bit(nb, Y);
       const uint32_t rk = t.row[((((int64_t)(a.x0 + X) * a.cb + Y) * a.Dc + c0) * a.Dc + c1) * a.Dm + m];
@@ -472,9 +477,10 @@ __global__ void __launch_bounds__(NT, NT == 128 ? (sizeof(R) * NZ > 64 ? 2 : 4) 
   const int mg0 = p.grp[0][a.x0 + a.xs] - p.grp[0][a.x0];   // charge-0 row groups of the slice
   const int64_t GR = (int64_t)a.xs * a.cb * inner, GC = (int64_t)a.xs2 * a.cb * inner;
   const int64_t ocol = (tq ? n0 : 0) + gi;
+  const int parity = a.parity & p.odd;
   for (int rq = 0; rq < 2; ++rq) {
     const int gbase = p.grp[rq][a.x0], nrow = p.grp[rq][a.x0 + a.xs] - gbase;
-    const int s = rq ^ tq ^ (a.parity & p.odd);
+    const int s = rq ^ tq ^ parity;
     const int nzs = nz[s];
     if (nzs == 0) continue;
     for (int b = blockIdx.y * RG; b < nrow; b += gridDim.y * RG) {
@@ -584,7 +590,8 @@ __global__ void __launch_bounds__(256) sector_close2_kernel(const R* __restrict_
   const int m0 = p.grp[0][a.x0 + a.xs] - p.grp[0][a.x0], n0 = p.grp[0][a.x20 + a.xs2] - p.grp[0][a.x20];
   const int moff[2] = {-p.grp[0][a.x0], m0 - p.grp[1][a.x0]};
   const int noff[2] = {-p.grp[0][a.x20], n0 - p.grp[1][a.x20]};
-  const uint32_t mc = p.mc;
+  const uint32_t mc = p.mc, nc = p.nc;
+  const int parity = a.parity & p.odd;
   for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < a.nfib; f += (int64_t)gridDim.x * blockDim.x) {
     uint32_t r = (uint32_t)f;
     int mg = a.x0 * a.cb * inner, ng = a.x20 * a.cb * inner, Z = 0;
@@ -604,7 +611,7 @@ __global__ void __launch_bounds__(256) sector_close2_kernel(const R* __restrict_
     for (int z = 0; z < NZ; ++z) acc[z] = 0;
     // charge of (c1', c2') that reaches a nonzero entry
     const int qm = (int)(t.grank[mg] >> 31) ^ bit(mc, 0), qn = (int)(t.grank[ng] >> 31) ^ bit(mc, 0);
-    const int s = qm ^ qn ^ bit(p.nc, Z) ^ (a.parity & p.odd);
+    const int s = qm ^ qn ^ bit(nc, Z) ^ parity;
     const R* o3 = O3 + (int64_t)Z * GR * GC;
     for (int c1 = 0; c1 < Dc; ++c1) {
       const uint32_t gr = t.grank[mg + c1 * a.Dm];
