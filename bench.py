@@ -10,8 +10,8 @@ hi + lo pair, three products, FP32 accumulation), normalisation and ln Z accumul
 W warm-up steps are steps 1..W of the run (bond dimensions reach 8 at step 3), the K
 timed steps are the steady-state steps W+1..W+K.
 
-At h = 0 the library contracts by Z2 charge sectors: three quarters of the 2 D^15 flops have
-an exactly zero factor and are not executed. "value" counts the whole 2 D^15 product of the
+At h = 0 the library contracts by Z2 charge sectors: about three quarters of the 2 D^15 flops
+have an exactly zero factor and are not executed. "value" counts the whole 2 D^15 product of the
 method, as the host arm's does, and is a measure of time per step, not of the tensor pipe;
 "executed_flops_share" says which part of the product runs, and the roofline counts that part.
 
@@ -88,10 +88,10 @@ def parse_args():
 
 
 # DRAM bytes (read + write) per launch of the block-spin GEMM, keyed by (precision, GEMM option,
-# D_cut, temperatures, impure), from an ncu capture of the kernel as built. The sector GEMM of the
-# h = 0 runs has no capture yet; the dense one moved 139.49 GB a launch at D_cut = 8. Workloads
-# without a capture report null.
-GEMM_TRAFFIC = {}
+# D_cut, temperatures, impure), from an ncu capture of the kernel as built (one pass): the sector GEMM of
+# step 6 of the h = 0 run (59.33 GB read, 2.47 written, share 0.29 of the dense product, which moved
+# 139.49 GB). Workloads without a capture report null.
+GEMM_TRAFFIC = {("fp16x3", 0, 8, 1, False): 61.80e9}
 
 
 # --------------------------------------------------------------------------- helpers

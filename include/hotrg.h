@@ -179,7 +179,8 @@ hotrg_status hotrg_step_info(hotrg_ctx* ctx, int b, int step, hotrg_step_record*
 /* Share of the multiply-adds of step `step`'s block-spin products (2 M N K flops each, of batch
  * element b, over every tensor) that the step executes: 1 for a dense contraction; where the
  * contraction ran by Z2 charge sectors, the blocks that are not zero by the charge, from the
- * sizes of the sectors (near 1/4). Tile padding is not counted. Synchronises. */
+ * sizes of the sectors (1/4 where the charges split evenly). Tile padding is not counted.
+ * Synchronises. */
 hotrg_status hotrg_product_share(hotrg_ctx* ctx, int b, int step, double* share);
 
 /* Number of steps done since the last init/set_tensor; current bond dimensions. */

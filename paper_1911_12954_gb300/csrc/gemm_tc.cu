@@ -99,7 +99,7 @@ struct Cfg {
   static constexpr uint32_t IDESC = (1u << 4) | ((F16 ? 0u : 2u) << 7) | ((F16 ? 0u : 2u) << 10) |
                                     ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(MMA_M >> 4) << 24);
 };
-using CfgTF32 = Cfg<64, false, 32>;     // default tf32 pipeline: 4 stages of 16-wide k-blocks
+using CfgTF32 = Cfg<64, false, 32>;     // tf32 on a device without CTA pairs: 4 stages of 16-wide k-blocks
 using CfgTF32W = Cfg<128, false, 32>;   // tf32, 2 stages of 32-wide k-blocks
 using CfgF16 = Cfg<64, true, 128>;      // fp16: 4 stages of 32-wide k-blocks, 128-k chunks
 using CfgF16S = Cfg<64, true, 64>;      // fp16 with 64-k chunks

@@ -8,7 +8,8 @@
 // isometry column it came from. A GEMM operand row (X, Y, c, c', mu) of charge r is nonzero only
 // at summed indices (a2, b2, a1', b1', k) of charge r + p (p the tensor's own parity: 0 for T and
 // M, 1 for S), and C = A B^T has only the blocks with q(row) + q(column) = the output's parity:
-// a quarter of the multiply-adds of the dense product, half of the operand and C bytes.
+// a quarter of the multiply-adds of the dense product where the charges split evenly (0.29 at D_cut = 8
+// near T_c, where 7 of 8 kept columns are even: hotrg_product_share), about half of the operand and C bytes.
 //
 // The sizes of the sectors are known on the device only (they follow from the order of the
 // eigenvalues), so nothing here depends on them on the host: sector_tables_kernel ranks the
@@ -19,8 +20,9 @@
 // An isometry column that mixes charges (which exact arithmetic excludes) drops the element to
 // "every charge 0, every parity 0" (SectorState::dropped, SectorPlan::odd): one sector, the dense product.
 //
-// Sums run over the nonzero terms in the order of the dense passes, so operands, C entries
-// given the same k order, and closed tensors are bit-identical to the dense passes'.
+// Operand entries and the closing sums run over their nonzero terms in the dense passes' order. The
+// product's summed index comes in the order (b2, b1', a2, a1', k), the dense one's in (a2, b2, a1', b1', k),
+// so C agrees with the dense product's up to the order of its sums.
 #include <mutex>
 #include <type_traits>
 
@@ -176,7 +178,8 @@ cudaError_t launch_sector_tables(const SectorArgs& a, int ne, cudaStream_t st) {
 // takes one (X, c, c', mu); a warp takes 64 rests of one segment and charge, two per lane: their O1 entries are
 // nonzero for the j of one charge only, each is loaded once and serves every r and Y, the coefficients are the
 // same for the whole warp (broadcast reads from shared memory), and the stores are pairs in runs of 64.
-// The writes bound it: at D_cut = 8 one pass writes 2.1 GB and reads 0.5 GB (0.4 ms at the copy rate).
+// Instruction issue bounds it (71 % of the issue slots at D_cut = 6, DRAM 26 %), then the writes: at D_cut = 8 a pass
+// writes 2.1 GB and reads 0.5 GB (0.4 ms at the copy rate; both sides in one launch 1.67 ms).
 template <int MODE, typename R>
 __device__ __forceinline__ void sector_store2(R* out, R* out_lo, int64_t o, R v0, R v1) {
   if constexpr (MODE == kTTMSplitF16) {

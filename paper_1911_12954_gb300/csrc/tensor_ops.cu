@@ -351,8 +351,8 @@ __global__ void __launch_bounds__(256) ttm_pair_f16_kernel(const R* __restrict__
 // group (X, c, c', mu; every Y) and n2 values of a2, keeps the hi and lo outputs of that contiguous range of the
 // summed index in shared memory, shifted so that shared and global 16-byte boundaries agree, and writes whole
 // 16-byte pieces. Same products in the same order as the short form, so the same bits. The two-byte stores of that form
-// into runs that start at any two-byte boundary held it at 1.2 TB/s; here the shared-memory accesses (two stores and
-// two loads an output) bound it at 1.5 TB/s. D = 5, T and S of 4 temperatures, both sides, 8 steps: 3.37 -> 2.64 ms.
+// into runs that start at any two-byte boundary held it at 1.2 TB/s; here instruction issue bounds it (79 % of the issue
+// slots; shared memory 49 % of its pipe, DRAM 28 %). D = 5, T and S of 4 temperatures, both sides, 8 steps: 3.37 -> 2.64 ms.
 template <int JM>
 __global__ void __launch_bounds__(256) dense_split_kernel(const __grid_constant__ DenseSplitJobs jobs,
                                                           const float* __restrict__ U) {

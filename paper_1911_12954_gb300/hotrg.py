@@ -257,7 +257,7 @@ class HOTRG:
                     gemm_option=r.gemm_option, tuned=bool(r.tuned), group=r.group)
 
     def product_share(self, step: int, b: int = 0) -> float:
-        """Share of step's block-spin product that was executed: 1 dense, near 1/4 by charge sectors."""
+        """Share of step's block-spin product that was executed: 1 dense, 1/4 or a little more by charge sectors."""
         out = ctypes.c_double()
         _check(self.lib.hotrg_product_share(self.ctx, b, step, ctypes.byref(out)), "product_share")
         return out.value
