@@ -62,6 +62,7 @@ struct StepPlan {
   int R[4];               // rows of the half-Gram per direction = D_nu D_mu
   int Rmax, nmax, nchunks;
   bool lean;              // isometry stage in the least space (see use_less)
+  int jne;                // batch elements whose eigenproblems run together
   int batch;              // batch elements whose isometry stages run together
   int ne;                 // batch elements contracted together (one group of launches)
   bool sect;              // contraction by Z2 charge sectors (sectors.cu)
@@ -430,6 +431,10 @@ StepPlan make_plan(const int D[4], int mu, int dcut, int prec, int batch = 1, in
   const int64_t per = (int64_t)batch * kMaxGramJobs * p.Rmax * p.Rmax * 8;
   while (nc > 1 && nc * per > (256LL << 20)) nc /= 2;
   p.nchunks = (int)nc;
+  // eigenproblems together: all, up to six per SM or 1 GB of work space (one launch after the other lasts as many times
+  // longer: 16 temperatures of 81 x 81 matrices by twos 18.5 ms, in one launch 2.3)
+  const int64_t one = 6 * jacobi_work_doubles(p.nmax) * 8;
+  p.jne = (int)std::min<int64_t>(batch, std::max<int64_t>(152, (1LL << 30) / one));
   p.main_flops = best;
   // every other product of the step, counted as 2 flops per multiply-add
   const double Ed = (double)p.E, rA = (double)p.rowsA_full, rB = (double)p.rowsB, Kd = (double)p.K;
@@ -535,19 +540,10 @@ Scratch scratch_layout(const StepPlan& p, int xs, int xs2, int prec, int impure,
   s.tab = p.sect ? take(ne * sector_tab(p).stride) : 0;
   s.amax = take(2 * ne * nt * sizeof(unsigned));   // A side, then B side: per element (and tensor)
   s.stats = take(4 * 3 * sizeof(unsigned long long));   // hotrg_split_stats counters
-  // as many elements' eigenproblems at a time as the others leave room for (1 MB where they are smaller: 50 elements
-  // at D = 2, two CTAs for every SM)
   const size_t gbytes = nb * kMaxGramJobs * p.nchunks * p.Rmax * p.Rmax * 8;
-  size_t jbytes;
-  if (p.lean) {
-    s.jsweeps = 1;
-    jbytes = (size_t)jacobi_work_doubles(p.nmax, 1) * 8;
-  } else {
-    s.jsweeps = kJacobiLogSweeps;
-    const size_t one = 6 * (size_t)jacobi_work_doubles(p.nmax) * 8, room = std::max<size_t>(std::max(off - shared, gbytes), 1 << 20);
-    s.jne = (int)std::min(nb, std::max<size_t>(room / one, 1));
-    jbytes = s.jne * one;
-  }
+  s.jne = p.lean ? 0 : p.jne;
+  s.jsweeps = p.lean ? 1 : kJacobiLogSweeps;
+  const size_t jbytes = (size_t)(p.lean ? 1 : 6 * p.jne) * jacobi_work_doubles(p.nmax, s.jsweeps) * 8;
   s.total = std::max(off, shared + align_up(std::max(gbytes, jbytes), 256));
   return s;
 }
@@ -1571,7 +1567,15 @@ bool plan_slices(const hotrg_ctx* ctx, StepPlan& p) {
     for (const bool lean : {false, true}) {
       StepPlan s = p;
       if (sect) use_sectors(s, ctx->prec);
-      if (lean) use_less(s);
+      if (lean) {
+        use_less(s);
+      } else {
+        // as many elements' eigenproblems at a time as the workspace holds
+        const Scratch sc = scratch_layout(s, 1, 1, ctx->prec, ctx->impure_active, ctx->rsize);
+        const size_t one = 6 * (size_t)jacobi_work_doubles(s.nmax) * 8, end = ctx->L.persistent_end + sc.jwork;
+        const size_t room = ctx->ws_bytes > end ? (ctx->ws_bytes - end) / 256 * 256 : 0;
+        s.jne = (int)std::min<size_t>(s.jne, std::max<size_t>(room / one, 1));
+      }
       if (choose_slices(ctx, s)) {
         p = s;
         return true;
@@ -1978,9 +1982,9 @@ hotrg_status hotrg_step(hotrg_ctx* ctx, int dir, int dcut) {
     // which buffer holds the tensors, whether it is the first step (M_1 = C(S,S)) and the
     // impure tensors in use. ln c / 2^k and the record slot come from the device counter.
     char key[256];
-    snprintf(key, sizeof(key), "%d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d", dir, dcut, ctx->dims[0],
+    snprintf(key, sizeof(key), "%d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d %d", dir, dcut, ctx->dims[0],
              ctx->dims[1], ctx->dims[2], ctx->dims[3], ctx->cur, ctx->k == 0, ctx->impure_active, p.xs, p.xs2,
-             ctx->batch, p.c, p.gemm_opt, p.ne, ctx->sectors ? 1 : 0, p.sect ? 1 : 0, p.lean ? 1 : 0);
+             ctx->batch, p.c, p.gemm_opt, p.ne, ctx->sectors ? 1 : 0, p.sect ? 1 : 0, p.lean ? 1 : 0, p.jne);
     auto it = ctx->graphs.find(key);
     if (it == ctx->graphs.end()) {
       const uint64_t l0 = ctx->launches;
