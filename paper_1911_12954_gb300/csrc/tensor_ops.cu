@@ -900,9 +900,9 @@ template cudaError_t launch_init<float>(const double*, const double*, float*, fl
 
 // ---------------------------------------------------------------------------- norm
 // Pass 1: each block writes the FP64 sum of squares of its grid-stride share. The FP64 pipe bounds it (an FMA per entry
-// and the sums across a block), so FP32 entries are widened by integer operations on their bits (D = 8: 52 us, 68 with a
-// conversion), and a thread takes at least kNormPer entries: with a block per 256 entries the sums across the blocks of
-// 8 temperatures at D = 4 took 21.8 us, with one per 2048 5.7.
+// and the sums across a block), so FP32 entries are widened by integer operations on their bits and a thread takes
+// kNormPer entries at least, all in flight. D = 8: 33 us (the pipe's rate; 68 with a conversion an entry), 8 temperatures
+// at D = 4 5.1 us (21.8 with a block per 256 entries); FP64 tensors of D = 9 80 us.
 constexpr int kNormBlocks = kNormPartials;
 constexpr int kNormPer = 8;
 
@@ -925,24 +925,28 @@ __global__ void __launch_bounds__(256) sumsq_kernel(const R* __restrict__ x, int
                                                     double* partial) {
   x += blockIdx.y * xstride;                   // batch element blockIdx.y
   partial += blockIdx.y * gridDim.x;
-  double sum[4] = {0, 0, 0, 0};                // four entries in flight
+  // kNormPer entries in flight, one chain of sums: a warp issues an FP64 instruction every 64 cycles, dependent or not
+  double acc = 0;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (; i + 3 * step < n; i += 4 * step) {
-    R v[4];
+  R v[kNormPer];
+  for (; i + (kNormPer - 1) * step < n; i += kNormPer * step) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = x[i + u * step];
+    for (int u = 0; u < kNormPer; ++u) v[u] = x[i + u * step];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kNormPer; ++u) {
       const double d = exact_double(v[u]);
-      sum[u] = fma(d, d, sum[u]);
+      acc = fma(d, d, acc);
     }
   }
-  for (; i < n; i += step) {
-    const double d = exact_double(x[i]);
-    sum[0] = fma(d, d, sum[0]);
+#pragma unroll
+  for (int u = 0; u < kNormPer - 1; ++u) v[u] = i + u * step < n ? x[i + u * step] : (R)0;
+#pragma unroll
+  for (int u = 0; u < kNormPer - 1; ++u) {
+    if (i + u * step >= n) break;              // a branch: an FP64 instruction costs its slot without lanes too
+    const double d = exact_double(v[u]);
+    acc = fma(d, d, acc);
   }
-  double acc = (sum[0] + sum[1]) + (sum[2] + sum[3]);
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
   __shared__ double w[8];
   const int lane = threadIdx.x & 31;
