@@ -102,8 +102,8 @@ cudaError_t launch_gemm_simt(const R* A, int64_t lda, const R* B, int64_t ldb, R
   // Tiles of 128 x 64 do 32 products per 12 operand reads, 64 x 32 ones 8 per 6, but four times as many of them share
   // the SMs more evenly. FP64: the FP64 pipe bounds either, so small tiles win below two large ones per SM (M = N, K =
   // 1024: 1.35 at M = 896, 1.6 at 1100, 1.0 at 1024 and 1536; D = 4 by sectors: 1088 -> 779 us). FP32: operand reads bound
-  // the small ones, which win only while two of them per SM hold the whole product (1.9 at M = 512, 1.26 at 768; 0.97 at
-  // 800, 0.74 at 1024, 0.64 at 1536).
+  // the small ones, which win while at most three of them per SM hold the whole product (operands from HBM, M = N, K =
+  // 1024: 1.7 at M = 512, 1.38 at 768, 1.10 at 960 - from L2 0.97 there - then 0.84 at 1024, 0.66 at 1536).
   auto go = [&](auto tm, auto tn) -> cudaError_t {
     constexpr int TM = decltype(tm)::value, TN = decltype(tn)::value;
     const int64_t more = one.sec.tab.base ? 1 : 0;   // two sectors: at most one more tile row
@@ -118,7 +118,7 @@ cudaError_t launch_gemm_simt(const R* A, int64_t lda, const R* B, int64_t ldb, R
   using I8 = std::integral_constant<int, 8>;
   const int64_t blocks = one.sec.tab.base ? 2 : 1;   // by sectors: half of the tiles of the dense product
   const int64_t large = ((M + 127) / 128) * ((N + 63) / 64) / blocks, small = ((M + 63) / 64) * ((N + 31) / 32) / blocks;
-  return (sizeof(R) == 8 ? large < 2 * 152 : small <= 2 * 152) ? go(I4{}, I2{}) : go(I8{}, I4{});
+  return (sizeof(R) == 8 ? large < 2 * 152 : small <= 3 * 152) ? go(I4{}, I2{}) : go(I8{}, I4{});
 }
 template cudaError_t launch_gemm_simt<double>(const double*, int64_t, const double*, int64_t, double*, int64_t,
                                               int64_t, int64_t, int64_t, double, double, cudaStream_t,

@@ -9,10 +9,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("dims,mu,dcut", [
-    ((4, 4, 4, 3), 3, 4),      # M = N = 768, K = 768: 288 small tiles, two per SM at most
-    ((5, 5, 5, 2), 3, 4),      # M = N = 800, K = 1250: 325
-    ((4, 4, 4, 4), 0, 4),      # M = N = 1024, K = 1024: 512, or 128 large ones
-    ((5, 5, 5, 3), 3, 4),      # M = N = 1200, K = 1875: ragged against both
+    ((4, 4, 4, 3), 3, 4),      # M = N = 768, K = 768: 288 small tiles
+    ((5, 5, 5, 2), 3, 4),      # M = N = 800, K = 1250: 325, ragged
+    ((4, 4, 4, 4), 0, 4),      # M = N = 1024, K = 1024: 512, so 128 large ones
+    ((5, 5, 5, 3), 3, 4),      # M = N = 1200, K = 1875: large ones, ragged
 ])
 @pytest.mark.parametrize("batch", [1, 3])
 def test_fp32_step_vs_fp64(dims, mu, dcut, batch):
