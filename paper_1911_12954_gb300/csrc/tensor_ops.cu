@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(256) ttm_short_kernel(const R* __restrict__ in
 
 // Several contractions of one kind in one launch (blockIdx.z): the first passes of both operand sides and of every
 // tensor are independent, and a small one leaves most of the chip idle (8 temperatures at D_cut = 4: two launches
-// of 13 us).
+// of 13 us, together 20.4; D_cut = 8: 229 + 207 us, together 433).
 template <typename R>
 struct FiberJobs {
   const R* in[kMaxPassJobs];
@@ -254,10 +254,24 @@ struct FiberJobs {
   R* out[kMaxPassJobs];
   FiberArgs a[kMaxPassJobs];
 };
-template <typename R, int MODE>
+// APART: a call for each job, whose arguments stay constant operands; otherwise one call, whose arguments are indexed by
+// blockIdx.z and loaded in every fibre. The calls' code is several times larger, which a small launch pays for.
+template <typename R, int MODE, bool APART>
 __global__ void __launch_bounds__(256) ttm_short_jobs_kernel(const __grid_constant__ FiberJobs<R> j) {
-  const int z = blockIdx.z;
-  ttm_short<R, MODE>(j.in[z], j.U[z], j.out[z], nullptr, j.a[z]);
+  if constexpr (APART) {
+    static_assert(kMaxPassJobs == 6, "a case for each job");
+    switch (blockIdx.z) {
+      case 0: ttm_short<R, MODE>(j.in[0], j.U[0], j.out[0], nullptr, j.a[0]); break;
+      case 1: ttm_short<R, MODE>(j.in[1], j.U[1], j.out[1], nullptr, j.a[1]); break;
+      case 2: ttm_short<R, MODE>(j.in[2], j.U[2], j.out[2], nullptr, j.a[2]); break;
+      case 3: ttm_short<R, MODE>(j.in[3], j.U[3], j.out[3], nullptr, j.a[3]); break;
+      case 4: ttm_short<R, MODE>(j.in[4], j.U[4], j.out[4], nullptr, j.a[4]); break;
+      default: ttm_short<R, MODE>(j.in[5], j.U[5], j.out[5], nullptr, j.a[5]); break;
+    }
+  } else {
+    const int z = blockIdx.z;
+    ttm_short<R, MODE>(j.in[z], j.U[z], j.out[z], nullptr, j.a[z]);
+  }
 }
 
 // The fp16 split of a short contraction, two fibres per thread: when the innermost fibre leg
@@ -811,16 +825,16 @@ cudaError_t launch_ttm_jobs(const TTMJob<R>* jobs, int n, int* launches, cudaStr
     smem = std::max(smem, short_smem(f.a[i].J1 * f.a[i].J2, f.a[i].R1 * f.a[i].R2, sizeof(R)));
     blocks = std::max(blocks, (f.a[i].nfib + 255) / 256);
   }
-  // A job that fills the chip by itself (8 blocks on each of 152 SMs per element) gains nothing from company and
-  // pays for arguments indexed by blockIdx.z: D_cut = 8, both first passes together 802 us, one after the other
-  // 229 + 208 us. The line is drawn per element, so the launches of a step do not grow with the batch.
-  if (blocks > 152 * 8) fused = false;
   if (fused) {
     const int nb = jobs[0].a.nb;
     const int64_t cap = std::max<int64_t>(8, 152 * 16 / ((int64_t)nb * n));
     const dim3 g((unsigned)std::min(blocks, cap), nb, n);
-    if (jobs[0].mode == kTTMStoreMax) ttm_short_jobs_kernel<R, kTTMStoreMax><<<g, 256, smem, st>>>(f);
-    else ttm_short_jobs_kernel<R, kTTMStore><<<g, 256, smem, st>>>(f);
+    // Jobs apart from four blocks per SM on (8 temperatures at D = 4, 1024 blocks: 27 -> 20.4 us; T, S and M of 4 at D = 5: 173
+    // -> 106; D = 8 802 -> 433); below, FP64 at D = 2 and 3 took 22 and 21 us that way, 10.5 and 13.5 indexed.
+    const bool apart = (int64_t)g.x * nb * n >= 152 * 4, bound = jobs[0].mode == kTTMStoreMax;
+    auto kernel = apart ? (bound ? ttm_short_jobs_kernel<R, kTTMStoreMax, true> : ttm_short_jobs_kernel<R, kTTMStore, true>)
+                        : (bound ? ttm_short_jobs_kernel<R, kTTMStoreMax, false> : ttm_short_jobs_kernel<R, kTTMStore, false>);
+    kernel<<<g, 256, smem, st>>>(f);
     *launches = 1;
     return cudaGetLastError();
   }
